@@ -82,34 +82,6 @@ __global__ void k_fourier_d(int npt, int nR, const cx<double> *__restrict__ PT, 
   }
 }
 
-// Batched Hermitian eigensolve, one matrix per thread (FP64, converged to
-// full precision).  w ascending; V columns are eigenvectors.
-template <int N>
-__global__ void k_eigh_d(int nmat, int n, const cx<double> *__restrict__ Ain, double *w, cx<double> *V,
-                         unsigned *dstatus) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nmat) return;
-  constexpr int UR = N <= 4 ? N : 1;
-  cx<double> A[N][N], U[N][N];
-  const cx<double> *a = Ain + (size_t)t * n * n;
-#pragma unroll UR
-  for (int i = 0; i < N; i++)
-#pragma unroll UR
-    for (int j = 0; j < N; j++) A[i][j] = (i < n && j < n) ? a[i * n + j] : mkc(0.0, 0.0);
-  bool nc = false;
-  jacobi_herm<double, N>(A, U, n, jacobi_tol<double>::tol2, jacobi_tol<double>::maxsweep, nc);
-  double ww[N];
-  sort_eig<double, N>(A, U, ww, n);
-  if (nc) atomicOr(dstatus, EPW_DEV_NOT_CONVERGED);
-#pragma unroll UR
-  for (int i = 0; i < N; i++) {
-    if (i < n) w[(size_t)t * n + i] = ww[i];
-#pragma unroll UR
-    for (int j = 0; j < N; j++)
-      if (i < n && j < n) V[(size_t)t * n * n + i * n + j] = U[i][j];
-  }
-}
-
 // omega = sign(w2) sqrt|w2|;  E[ka][nu] = e_{ka,nu} / sqrt(2 M_kappa omega_nu),
 // zero when omega_nu < omega_min.  Outputs are transposed ([..][nq]).
 __global__ void k_phonon_post(int nq, int nm, const double *__restrict__ w2, const cx<double> *__restrict__ ev,
@@ -1076,21 +1048,6 @@ void launch_fourier_d(int npt, int nR, const cx<double> *PT, const cx<double> *X
   size_t n = (size_t)npt * msize;
   if (!n) return;
   k_fourier_d<<<nblocks(n, 256), 256, 0, st>>>(npt, nR, PT, X, msize, out);
-  epw_count_launch();
-}
-
-void launch_eigh_d(int nmat, int n, cx<double> *A, double *w, cx<double> *V, unsigned *dstatus, cudaStream_t st) {
-  if (!nmat) return;
-  // one warp per block: the FP64 pipe is per SM, so small batches spread over more SMs
-  int b = (nmat + 31) / 32;
-  if (n <= 3)
-    k_eigh_d<3><<<b, 32, 0, st>>>(nmat, n, A, w, V, dstatus);
-  else if (n <= 4)
-    k_eigh_d<4><<<b, 32, 0, st>>>(nmat, n, A, w, V, dstatus);
-  else if (n <= 9)
-    k_eigh_d<9><<<(nmat + 63) / 64, 64, 0, st>>>(nmat, n, A, w, V, dstatus);
-  else
-    k_eigh_d<18><<<(nmat + 63) / 64, 64, 0, st>>>(nmat, n, A, w, V, dstatus);
   epw_count_launch();
 }
 
