@@ -360,7 +360,7 @@ static size_t rsize(int prec) { return prec == EPW_FP64 ? sizeof(cx<double>) : s
 
 // Lay out (or, with a null base, measure) the preparation buffers.
 static void plan_prep(Arena &A, const epw_model *m, int nk, int nq, int prec, bool stage_k, bool stage_q,
-                      bool stage_wq, bool need_B, Prep &p) {
+                      bool stage_wq, bool need_B, Prep &p, const Fx64 *fx = nullptr) {
   const size_t sR = rsize(prec);
   const size_t nw2 = (size_t)m->nw * m->nw, nm2 = (size_t)m->nm * m->nm;
   p.kd = stage_k ? A.take<double>(3 * (size_t)nk) : nullptr;
@@ -371,9 +371,14 @@ static void plan_prep(Arena &A, const epw_model *m, int nk, int nq, int prec, bo
   p.Hk = A.take<cx<double>>((size_t)nk * nw2);
   p.epsk = A.take<double>((size_t)nk * m->nw);
   p.Uk = A.take<cx<double>>((size_t)nk * nw2);
-  p.PqTe = A.take<char>(sR * m->nRe * (size_t)nq);
-  p.PqTp = m->same_ep ? p.PqTe : A.take<char>(sR * m->nRp * (size_t)nq);
-  p.PqTph = (m->same_eph && prec == EPW_FP64) ? (cx<double> *)p.PqTe : A.take<cx<double>>((size_t)m->nRph * nq);
+  if (fx && fx->pair) {
+    p.PqTe = p.PqTp = nullptr;  // the phases are digit planes
+    p.PqTph = nullptr;
+  } else {
+    p.PqTe = A.take<char>(sR * m->nRe * (size_t)nq);
+    p.PqTp = m->same_ep ? p.PqTe : A.take<char>(sR * m->nRp * (size_t)nq);
+    p.PqTph = (m->same_eph && prec == EPW_FP64) ? (cx<double> *)p.PqTe : A.take<cx<double>>((size_t)m->nRph * nq);
+  }
   p.D = A.take<cx<double>>((size_t)nq * nm2);
   p.w2 = A.take<double>((size_t)nq * m->nm);
   p.ev = A.take<cx<double>>((size_t)nq * nm2);
@@ -384,7 +389,7 @@ static void plan_prep(Arena &A, const epw_model *m, int nk, int nq, int prec, bo
     size_t nbg = (size_t)nk * m->nRp * m->nm * nw2;
     p.G1 = A.take<char>(sR * nbg);
     p.Bg = A.take<char>(sR * nbg);
-    p.BH = A.take<char>(sR * (size_t)nk * m->nRe * nw2);
+    p.BH = fx && fx->pair ? nullptr : A.take<char>(sR * (size_t)nk * m->nRe * nw2);
     if (prec != EPW_FP64) {
       p.Pk32 = A.take<cx<float>>((size_t)nk * m->nRe);
       p.gw32 = A.take<cx<float>>((size_t)m->nRe * m->nRp * m->nm * nw2);
@@ -396,6 +401,160 @@ static void plan_prep(Arena &A, const epw_model *m, int nk, int nq, int prec, bo
     p.G1 = p.Bg = p.BH = nullptr;
     p.Pk32 = p.gw32 = nullptr;
   }
+}
+
+// --------------------------------------------- fixed-point contractions
+// FP64 instructions (64 cycles a warp on each of 608 sub-partitions) in microseconds at 2 GHz.
+static double fp64_us(double per_thread, double threads) {
+  return per_thread * 0.032 * std::max(1.0, threads / (32.0 * 608.0));
+}
+// D(q) as digit planes costs two passes over them and about 30 us of launches; the CUDA cores
+// take 4 nR nm^2 FP64 instructions per q (316,000 q of 249 R and 6 modes: 18.6 ms).
+static bool fx_dq(const epw_model *m, int nq) {
+  return fp64_us(4.0 * m->nRph * m->nm * m->nm, nq) > 150.0;
+}
+// The pairs: the CUDA cores take 4 nw^2 (nRe + nm nRp) instructions per pair; the planes of both
+// sides, the GEMMs and their launches take about 100 us at least.
+static bool fx_pair(const epw_model *m, int nk, int nq) {
+  return fp64_us(4.0 * m->nw * m->nw * (m->nRe + (double)m->nm * m->nRp), (double)nk * nq) > 150.0;
+}
+
+// g(k,Rp) = sum_Re P_k(Re) g(Re,Rp) in FP64: the CUDA cores take 4 nRe instructions per k and
+// column; the digit planes of g are 90 bytes of traffic per entry, their GEMM 2,490 cycles per
+// 128 k x 32 columns x 16 Re.
+static bool fx_g1(const epw_model *m, int nk) {
+  const double ncol = (double)m->nRp * m->nm * m->nw * m->nw;
+  const double simt = fp64_us(4.0 * m->nRe, ncol * nk);
+  const double tiles = (double)((nk + 127) / 128) * std::ceil(ncol / 32.0) * (fx_kpad(m->nRe) / 32);
+  return 25.0 + m->nRe * ncol * 90.0 / 4e6 + tiles * 2490.0 / (152.0 * 1900.0) < simt;
+}
+// Planes of g per block of columns.
+static const size_t FX_GW_BYTES = (size_t)2 << 30;
+
+// Contraction chunk of the FP64 form.
+static const size_t FX_CT_BYTES = (size_t)2 << 30;
+
+// more: further bytes per k of a chunk (the adjoint's and the interpolation's buffers).
+static void plan_fx(Arena &A, const epw_model *m, int nk, int nq, bool dq, bool pair, bool g1, Fx64 &f,
+                    size_t more = 0) {
+  f = Fx64{};
+  f.dq = dq || pair;
+  f.pair = pair;
+  f.g1 = g1;
+  if (g1) {
+    const int kp = fx_kpad(m->nRe);
+    const size_t ncol = (size_t)m->nRp * m->nm * m->nw * m->nw;
+    f.gcols = (int)std::min<size_t>(ncol, std::max<size_t>(32, FX_GW_BYTES / ((size_t)28 * kp) / 32 * 32));
+    f.Ak = fx_plan(A, nk, kp, true);
+    f.Gw = fx_plan(A, 2 * (size_t)f.gcols, kp, true);
+  }
+  if (!f.dq) return;
+  const size_t nm2 = (size_t)m->nm * m->nm, nw2 = (size_t)m->nw * m->nw;
+  f.Aph = fx_plan(A, nq, fx_kpad(m->nRph), true);
+  f.Phi = fx_plan(A, nm2, fx_kpad(m->nRph), true);
+  f.Dh = A.take<double>(nm2 * nq);
+  if (!pair) return;
+  f.Ae = m->same_eph ? f.Aph : fx_plan(A, nq, fx_kpad(m->nRe), true);
+  f.Ap = m->same_ep ? f.Ae : fx_plan(A, nq, fx_kpad(m->nRp), true);
+  f.ldc = (size_t)(nq + 127) / 128 * 128;
+  const size_t cols = nw2 * (1 + 2 * (size_t)m->nm);
+  const size_t kplanes = 2 * FX_S * nw2 * ((size_t)fx_kpad(m->nRe) + 2 * (size_t)m->nm * fx_kpad(m->nRp));
+  f.kc = (int)std::min<size_t>((size_t)nk, std::max<size_t>(1, FX_CT_BYTES / (cols * f.ldc * 8 + kplanes + more)));
+  f.BH = fx_plan(A, f.kc * nw2, fx_kpad(m->nRe), true);
+  f.BG = fx_plan(A, f.kc * nw2 * 2 * m->nm, fx_kpad(m->nRp), true);
+  f.CH = A.take<long long>(f.kc * nw2 * f.ldc);
+  f.CG = A.take<long long>(f.kc * nw2 * 2 * m->nm * f.ldc);
+  f.omK = A.take<double>((size_t)m->nm * nq);
+  f.nbT = A.take<double>((size_t)m->nm * nq);
+  f.wmax = A.take<double>(nq);
+  f.bad = A.take<int>(1);
+}
+
+// q side: the phases' planes and D(q).
+static epw_status run_fx_q(const epw_model *m, int nq, const double *q, Fx64 &f, cx<double> *D, cudaStream_t st) {
+  fx_phases(nq, q, m->nRph, m->Rph, m->rmax, f.Aph, st);
+  fx_hermitian(1, m->nRph, m->nm, nullptr, m->Phiw, f.Phi, nullptr, st);
+  CKS(fx_gemm_f64(f.Aph, f.Phi, fx_bits(m->nRph), f.Dh, (size_t)m->nm * m->nm, m->dstatus, st));
+  fx_unpack_hermitian(nq, m->nm, f.Dh, D, st);
+  if (f.pair) {
+    if (!m->same_eph) fx_phases(nq, q, m->nRe, m->Re, m->rmax, f.Ae, st);
+    if (!m->same_ep) fx_phases(nq, q, m->nRp, m->Rp, m->rmax, f.Ap, st);
+  }
+  return EPW_OK;
+}
+
+// G1[k][Rp a j i] = sum_Re P_k(Re) g(Re, Rp)_aji in FP64.
+static epw_status run_vertex64(const epw_model *m, int nk, const double *k, const Prep &p, Fx64 *f, cudaStream_t st) {
+  const int ncol = m->nRp * m->nm * m->nw * m->nw;
+  if (!f || !f->g1) {
+    launch_vertex_fewk(nk, m->nRe, ncol, p.PkRM, m->gw, (cx<double> *)p.G1, st);
+    return EPW_OK;
+  }
+  FxOp ak = f->Ak;
+  ak.rows = nk;
+  fx_phases(nk, k, m->nRe, m->Re, m->rmax, ak, st);
+  for (int c0 = 0; c0 < ncol; c0 += f->gcols) {
+    const int nc = std::min(f->gcols, ncol - c0);
+    FxOp gw = f->Gw;
+    gw.rows = 2 * nc;
+    fx_columns(1, m->nRe, nc, ncol, m->gw + c0, gw, nullptr, st);
+    CKS(fx_gemm_f64(ak, gw, fx_bits(m->nRe), (double *)p.G1 + 2 * (size_t)c0, 2 * (size_t)ncol, m->dstatus, st));
+  }
+  return EPW_OK;
+}
+
+// H(k+q) and g(k,q) U_k of the k-points [k0, k0 + kc) into f.CH, f.CG.
+// (hmat: H(k+q) as FP64 into f.Hq [nq][kc][nw^2] instead; vertex: whether g(k,q) U_k is wanted)
+static epw_status run_fx_contract(const epw_model *m, int k0, int kc, const Prep &p, Fx64 &f, cudaStream_t st,
+                                  bool hmat = false, bool vertex = true) {
+  const int nw2 = m->nw * m->nw, ncol = m->nm * nw2;
+  FxOp bh = f.BH, bg = f.BG;  // a last, shorter chunk has fewer rows (and tighter planes)
+  bh.rows = kc * nw2;
+  bg.rows = kc * 2 * ncol;
+  fx_hermitian(kc, m->nRe, m->nw, p.PkRM + (size_t)k0 * m->nRe, m->Hw, bh, f.bad, st);
+  if (hmat)
+    CKS(fx_gemm_f64(f.Ae, bh, fx_bits(m->nRe), f.Hq, (size_t)kc * nw2, m->dstatus, st));
+  else
+    CKS(fx_gemm_i64(f.Ae, bh, fx_bits(m->nRe), f.CH, f.ldc, m->dstatus, st));
+  if (!vertex) return EPW_OK;
+  fx_columns(kc, m->nRp, ncol, ncol, (const cx<double> *)p.Bg + (size_t)k0 * m->nRp * ncol, bg, f.bad, st);
+  return fx_gemm_i64(f.Ap, bg, fx_bits(m->nRp), f.CG, f.ldc, m->dstatus, st);
+}
+
+static Pair64Args pair64_args(const epw_model *m, int k0, int kc, int nq, const double *wq, const epw_params *par,
+                              const Prep &p, const Fx64 &f) {
+  Pair64Args a;
+  std::memset(&a, 0, sizeof(a));
+  a.nq = nq;
+  a.nw = m->nw;
+  a.nm = m->nm;
+  a.k0 = k0;
+  a.nk = kc;
+  a.CH = f.CH;
+  a.CG = f.CG;
+  a.eH = f.BH.e;
+  a.eG = f.BG.e;
+  a.FH = fx_bits(m->nRe);
+  a.FG = fx_bits(m->nRp);
+  a.ldc = f.ldc;
+  a.ET = (const double2 *)p.ET;
+  a.omK = f.omK;
+  a.nbT = f.nbT;
+  a.wmax = f.wmax;
+  a.eps_k = p.epsk;
+  a.wq = wq;
+  a.T = par->T_K;
+  a.EF = par->EF_eV;
+  a.sigma = par->sigma_eV;
+  a.inv_kT = par->T_K > 0.0 ? 1.0 / (EPW_KB * par->T_K) : 0.0;
+  a.inv_sigma = 1.0 / par->sigma_eV;
+  a.gnorm = 1.0 / (par->sigma_eV * 1.7724538509055160273);
+  a.inv_nq = 1.0 / nq;
+  a.dstatus = m->dstatus;
+  a.bad = f.bad;
+  a.Cpol = m->polar ? (const double2 *)p.Cpol : nullptr;
+  a.Uk = p.Uk;
+  return a;
 }
 
 // Phases, k-side bands, phonons and the k-side vertex (Bg, BH).
@@ -418,7 +577,7 @@ static epw_status prep_streams(epw_model *m) {
 // phonon work (FP64) still runs on the second stream.
 static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq, const double *q, int prec,
                            double omega_min, bool need_B, Prep &p, double *omega_out, cudaStream_t st,
-                           bool fork = true, TcBuffers *tcb = nullptr) {
+                           bool fork = true, TcBuffers *tcb = nullptr, Fx64 *fx = nullptr) {
   epw_model *m = const_cast<epw_model *>(mc);
   const int nw = m->nw, nm = m->nm;
   const size_t nw2 = (size_t)nw * nw;
@@ -435,6 +594,8 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   const bool qs = tcb && prec != EPW_FP64 && tc_qside(m, nq, q, *tcb, p.D, sq);
   if (qs) {
     tcb->prebuilt_a = true;
+  } else if (fx && fx->pair) {
+    CK(cudaMemsetAsync(fx->bad, 0, sizeof(int), st));
   } else if (prec == EPW_FP64) {
     launch_phases(nq, q, m->nRe, m->Re, m->rmax, nullptr, (cx<double> *)p.PqTe, nullptr, sq);
     if (!m->same_ep) launch_phases(nq, q, m->nRp, m->Rp, m->rmax, nullptr, (cx<double> *)p.PqTp, nullptr, sq);
@@ -446,7 +607,11 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   }
   if (tcb && fork && !qs) CK(cudaEventRecord(m->ev_phase, sq));
   // phonons (FP64 eigensolve)
-  if (!qs) launch_fourier_d(nq, m->nRph, p.PqTph, m->Phiw, nm * nm, p.D, sq);
+  if (!qs && fx && fx->dq) {
+    CKS(run_fx_q(m, nq, q, *fx, p.D, sq));
+  } else if (!qs) {
+    launch_fourier_d(nq, m->nRph, p.PqTph, m->Phiw, nm * nm, p.D, sq);
+  }
   launch_eigh_d(nq, nm, p.D, p.w2, p.ev, m->dstatus, sq);
   launch_phonon_post(nq, nm, p.w2, p.ev, m->mass, omega_min, p.omegaT,
                      prec == EPW_FP64 ? (cx<double> *)p.ET : nullptr, prec == EPW_FP64 ? nullptr : (cx<float> *)p.ET,
@@ -461,7 +626,7 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   // bands (H(k), eigensolve) run on a third stream beside the vertex GEMM, which
   // needs only the phases, and are joined before the U_k rotation
   launch_phases(nk, k, m->nRe, m->Re, m->rmax, p.PkRM, p.PkT, nullptr, st);
-  const bool fork2 = fork && need_B && prec != EPW_FP64;
+  const bool fork2 = fork && need_B;
   cudaStream_t sk = st;
   if (fork2) {
     CK(cudaEventRecord(m->ev_fork2, st));
@@ -474,8 +639,8 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   if (need_B && nk > 0) {
     const int ncol = m->nRp * nm * (int)nw2;
     if (prec == EPW_FP64) {
-      launch_cgemm<double>(nk, ncol, m->nRe, p.PkRM, m->nRe, false, false, m->gw, ncol, (cx<double> *)p.G1, ncol,
-                           false, st);
+      CKS(run_vertex64(m, nk, k, p, fx, st));
+      if (fork2) CK(cudaStreamWaitEvent(st, m->ev_join2, 0));
       launch_build_B<double>(m, nk, p.PkRM, (const cx<double> *)p.G1, p.Uk, (cx<double> *)p.Bg, (cx<double> *)p.BH,
                              st);
     } else {
@@ -566,7 +731,7 @@ EpwTune epwi_default_tune() {
                  : strcmp(w, "split") == 0 ? TCW_FORM_SPLIT
                  : strcmp(w, "single") == 0 ? TCW_FORM_SINGLE
                                             : TCW_FORM_PAIR;
-  return EpwTune{0, STAGED_CT_BYTES, form, kside};
+  return EpwTune{0, STAGED_CT_BYTES, form, kside, false, false, false};
 }
 
 // The buffers of one pass over nk k-points (k and output staging excluded).
@@ -574,11 +739,13 @@ static epw_status plan_linewidth_pass(Arena &A, const epw_model *m, int nk, int 
                                       const EpwTune &tune, LwPlan &L) {
   const bool tc = prec == EPW_BF16X3 || prec == EPW_TF32X3;
   const int op = prec == EPW_BF16X3 ? TC_OP_BF16 : TC_OP_TF32;
-  plan_prep(A, m, nk, nq, tc ? EPW_FP32 : prec, false, sq, swq, true, L.p);
   L.sg = TcStaged{};
   L.tc = TcBuffers{};
   L.w = TcwBuffers{};
-  if (tc && tc_supported(m)) {
+  const bool narrow = tc && tc_supported(m);
+  plan_fx(A, m, nk, nq, !tune.simt64 && !narrow && fx_dq(m, nq), tune.pair64, tune.g1_64, L.fx);
+  plan_prep(A, m, nk, nq, tc ? EPW_FP32 : prec, false, sq, swq, true, L.p, &L.fx);
+  if (narrow) {
     CKS(tc_plan(A, m, nk, nq, op, L.tc));
     L.tc.a_block_bytes = tune.a_block_bytes;
     L.partial = nullptr;
@@ -626,7 +793,11 @@ static int k_per_pass(const epw_model *m, int nk, int nq, int prec, const EpwTun
 }
 
 epw_status epwi_plan_linewidth(Arena &A, const epw_model *m, int nk, int nq, int prec, bool sk, bool sq, bool swq,
-                               bool sout, const EpwTune &tune, LwPlan &L) {
+                               bool sout, const EpwTune &tune0, LwPlan &L) {
+  // the form is chosen from the whole k list, so that results do not depend on the passes
+  EpwTune tune = tune0;
+  tune.pair64 = !tune.simt64 && prec == EPW_FP64 && fx_pair(m, nk, nq);
+  tune.g1_64 = !tune.simt64 && prec == EPW_FP64 && fx_g1(m, nk);
   L.kchunk = k_per_pass(m, nk, nq, prec, tune);
   double *kd = sk ? A.take<double>(3 * (size_t)nk) : nullptr;  // the whole k list, staged from the host
   CKS(plan_linewidth_pass(A, m, L.kchunk, nq, prec, sq, swq, tune, L));
@@ -765,14 +936,14 @@ static epw_status linewidth_pass(epw_model *m, int nk, const double *kd, int nq,
     if (s != EPW_OK) return fail(s, "tensor-core path: %s", g_err[0] ? g_err : "unsupported shape");
   } else if (tcp && L.w.ok) {
     // wide-shape fused form: per chunk of k, the H(k+q) eigensolve kernel and the vertex kernel
-    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st));
+    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &L.fx));
     epw_status s = tcw_linewidth(m, nk, nq, qd, wqd, par, p.epsk, p.omegaT, (const cx<float> *)p.ET,
                                  (const cx<float> *)p.Bg, (const cx<float> *)p.BH, m->same_eph ? p.PqTph : nullptr,
                                  p.Uk, m->polar ? (const float2 *)p.Cpol : nullptr, L.w, out, st);
     if (s != EPW_OK) return fail(s, "wide tensor-core path: %s", g_err[0] ? g_err : "launch failed");
   } else if (tcp) {
     // staged tensor-core form: contraction per chunk of k on the tensor cores, per-pair work from HBM
-    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st));
+    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &L.fx));
     L.sg.Pq64 = m->same_eph ? p.PqTph : nullptr;
     CKS(tc_staged_phases(m, nq, qd, L.sg, st));
     epw_timing_begin(m, st);
@@ -809,8 +980,23 @@ static epw_status linewidth_pass(epw_model *m, int nk, const double *kd, int nq,
     }
     epw_timing_end(m, st);
     launch_finalize(nk, (nq + 127) / 128, m->nw, L.partial, out, st);
+  } else if (L.fx.pair) {
+    // FP64: the contractions of a chunk of k as digit planes on the tensor cores, per-pair work in FP64
+    CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &L.fx));
+    launch_tables64(nq, m->nm, p.omegaT, par->omega_min_eV, par->T_K, L.fx.omK, L.fx.nbT, L.fx.wmax, st);
+    epw_timing_begin(m, st);
+    for (int k0 = 0; k0 < nk; k0 += L.fx.kc) {
+      const int kc = std::min(L.fx.kc, nk - k0);
+      CKS(run_fx_contract(m, k0, kc, p, L.fx, st));
+      Pair64Args a = pair64_args(m, k0, kc, nq, wqd, par, p, L.fx);
+      a.partial = L.partial;
+      epw_status s = launch_lw64(a, st);
+      if (s != EPW_OK) return fail(s, "FP64 per-pair kernel failed for nw=%d, 3nat=%d", m->nw, m->nm);
+    }
+    epw_timing_end(m, st);
+    launch_finalize(nk, (nq + 127) / 128, m->nw, L.partial, out, st);
   } else {
-    CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st));
+    CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &L.fx));
     PairArgs a;
     std::memset(&a, 0, sizeof(a));
     a.nk = nk;
@@ -868,8 +1054,24 @@ extern "C" epw_status epw_interp_g(const epw_model *mc, int nk, const double *k,
   const bool s_om = omega && !is_device_ptr(omega), s_g = g && !is_device_ptr(g);
   TcBuffers tcb;
   TcStaged sg{};
+  Fx64 fx;
+  const bool want_pairs = nk > 0 && nq > 0 && (eps_kq || g);
+  bool need_B = true;
+  cx<double> *Hq = nullptr, *Uq = nullptr;
+  double *wkq = nullptr;
   auto plan = [&](Arena &A, Prep &p, double *&ekd, double *&ekqd, double *&omd, double *&gd) -> epw_status {
-    plan_prep(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, wprec, sk, sq, false, true, p);
+    const size_t per = (size_t)nq * nw * (40 * nw + 8);  // H(k+q) twice, its eigenvectors and eigenvalues
+    plan_fx(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, !tc && fx_dq(m, nq),
+            precision == EPW_FP64 && want_pairs && fx_pair(m, nk, nq), precision == EPW_FP64 && nk > 0 && g && fx_g1(m, nk), fx, per);
+    if (fx.pair) {
+      const size_t np = (size_t)nq * fx.kc;
+      fx.Hq = A.take<double>(np * nw * nw);
+      Hq = A.take<cx<double>>(np * nw * nw);
+      Uq = A.take<cx<double>>(np * nw * nw);
+      wkq = A.take<double>(np * nw);
+    }
+    need_B = nk > 0 && (g || !fx.pair);  // bands alone need no vertex
+    plan_prep(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, wprec, sk, sq, false, need_B || nk == 0, p, &fx);
     ekd = s_ek ? A.take<double>((size_t)nk * nw) : eps_k;
     ekqd = s_ekq ? A.take<double>((size_t)nk * nq * nw) : eps_kq;
     omd = s_om ? A.take<double>((size_t)nq * nm) : omega;
@@ -895,7 +1097,7 @@ extern "C" epw_status epw_interp_g(const epw_model *mc, int nk, const double *k,
     CK(cudaMemcpyAsync(p.qd, q, sizeof(double) * 3 * nq, cudaMemcpyHostToDevice, st));
     qd = p.qd;
   }
-  CKS(run_prep(m, nk, kd, nq, qd, wprec, omega_min, nk > 0, p, omd, st, true, tc ? &tcb : nullptr));
+  CKS(run_prep(m, nk, kd, nq, qd, wprec, omega_min, need_B, p, omd, st, true, tc ? &tcb : nullptr, &fx));
   if (ekd && nk > 0) CK(cudaMemcpyAsync(ekd, p.epsk, sizeof(double) * nk * nw, cudaMemcpyDeviceToDevice, st));
   if (tc && nk > 0 && nq > 0 && (ekqd || gd)) {
     tcb.Cpol = m->polar ? (const float2 *)p.Cpol : nullptr;
@@ -935,6 +1137,22 @@ extern "C" epw_status epw_interp_g(const epw_model *mc, int nk, const double *k,
       a.cpk = sg.cpk;
       s = launch_pair_staged(a, 1, st);
       if (s != EPW_OK) return fail(s, "no staged per-pair kernel for nw=%d, 3nat=%d", m->nw, m->nm);
+    }
+  } else if (fx.pair) {
+    // FP64: H(k+q) as matrices, the batched Jacobi (the eigenvectors' phases are its), then g
+    for (int k0 = 0; k0 < nk; k0 += fx.kc) {
+      const int kc = std::min(fx.kc, nk - k0);
+      CKS(run_fx_contract(m, k0, kc, p, fx, st, true, gd != nullptr));
+      fx_unpack_hermitian(nq * kc, m->nw, fx.Hq, Hq, st);
+      launch_eigh_d(nq * kc, m->nw, Hq, wkq, Uq, m->dstatus, st);
+      epw_params par{0.0, 0.0, 1.0, omega_min, precision, 0};
+      Pair64Args a = pair64_args(m, k0, kc, nq, nullptr, &par, p, fx);
+      a.wkq = wkq;
+      a.Ukq = Uq;
+      a.eps_kq = ekqd;
+      a.gout = (cx<double> *)gd;
+      epw_status s = launch_g64(a, st);
+      if (s != EPW_OK) return fail(s, "FP64 vertex kernel failed");
     }
   } else if (nk > 0 && nq > 0 && (ekqd || gd)) {
     PairArgs a;
@@ -1000,6 +1218,7 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
   const bool swq = wq && nq > 0 && !is_device_ptr(wq), scot = nk > 0 && !is_device_ptr(cot);
   const bool sdg = dg && !is_device_ptr(dg), sdT = dT && !is_device_ptr(dT), sdE = dEF && !is_device_ptr(dEF);
   const size_t sR = rsize(prec);
+  const bool pair64 = prec == EPW_FP64 && nk > 0 && nq > 0 && fx_pair(m, nk, nq);
   // k chunk so that the per-chunk adjoint buffers stay near 1 GiB
   size_t per_k = (size_t)nq * per * sR + 2 * (size_t)m->nRp * per * sR;
   int nkc = (int)std::max<size_t>(1, std::min<size_t>((size_t)std::max(nk, 1), ((size_t)1 << 30) / std::max<size_t>(per_k, 1)));
@@ -1011,11 +1230,38 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
     TcBwdBuffers tw;
     TcStaged sg;
     TcBwdBuffers sw;  // staged shapes: the q contraction of Xbar on the tensor cores
+    // FP64 in fixed point: Xbar's columns and the conjugate phases of Rp over q, the rotated sums and
+    // the conjugate phases of Re over k, the gradient [nRp 3nat nw^2][nRe]
+    Fx64 fx;
+    FxOp Xq, Pq, Gk, Pk;
+    cx<double> *xb64, *G1b, *gT;
+    double *Bq;
   } b;
   b.sg = TcStaged{};
   auto plan = [&](Arena &A) -> epw_status {
-    plan_prep(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, prec, sk, sq, swq, true, b.p);
+    const int kpq = fx_kpad(nq);
+    plan_fx(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, !tcb && fx_dq(m, nq), pair64,
+            prec == EPW_FP64 && nk > 0 && fx_g1(m, nk), b.fx,
+            per * ((size_t)nq * 16 + 2 * FX_S * (size_t)kpq + 16 * (size_t)fx_splits(kpq) * m->nRp + 16 * (size_t)m->nRp));
+    plan_prep(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, prec, sk, sq, swq, true, b.p, &b.fx);
     b.cotd = scot ? A.take<double>((size_t)nk * m->nw) : (double *)cot;
+    if (pair64) {
+      const size_t kc = b.fx.kc, kpk = fx_kpad((int)kc);
+      b.xb64 = A.take<cx<double>>(kc * per * nq);
+      b.Xq = fx_plan(A, kc * per, kpq, true);
+      b.Pq = fx_plan(A, 2 * (size_t)m->nRp, kpq, false);
+      b.Bq = A.take<double>((size_t)fx_splits(kpq) * kc * per * 2 * m->nRp);
+      b.G1b = A.take<cx<double>>((size_t)m->nRp * per * kc);
+      b.Gk = fx_plan(A, m->nRp * per, (int)kpk, true);
+      b.Pk = fx_plan(A, 2 * (size_t)m->nRe, (int)kpk, false);
+      b.gT = A.take<cx<double>>(ng);
+      b.pT = A.take<double>(kc * nqb);
+      b.pE = A.take<double>(kc * nqb);
+      b.gwbar = nullptr;
+      b.sc = A.take<double>(2);
+      b.dgd = sdg ? A.take<double>(2 * ng) : dg;
+      return EPW_OK;
+    }
     if (tcb) {
       b.xbar = b.Bbar = b.G1bar = b.pT = b.pE = nullptr;
       CKS(tc_bwd_plan(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, b.tc, b.tw));
@@ -1058,8 +1304,41 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
   }
   if (scot) CK(cudaMemcpyAsync(b.cotd, cot, sizeof(double) * nk * m->nw, cudaMemcpyHostToDevice, st));
   CK(cudaMemsetAsync(b.sc, 0, 2 * sizeof(double), st));
-  CK(cudaMemsetAsync(b.gwbar, 0, sR * ng, st));
-  if (nk > 0 && nq > 0 && tcb) {
+  if (!pair64) CK(cudaMemsetAsync(b.gwbar, 0, sR * ng, st));
+  if (pair64) {
+    CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx));
+    launch_tables64(nq, m->nm, p.omegaT, par->omega_min_eV, par->T_K, b.fx.omK, b.fx.nbT, b.fx.wmax, st);
+    if (b.dgd) fx_phases_conj(nq, qd, m->nRp, m->Rp, b.Pq, st);
+    const int splits = fx_splits(b.Xq.kpad);
+    for (int k0 = 0; k0 < nk; k0 += b.fx.kc) {
+      const int kc = std::min(b.fx.kc, nk - k0);
+      CKS(run_fx_contract(m, k0, kc, p, b.fx, st));
+      CK(cudaMemsetAsync(b.xb64, 0, sizeof(cx<double>) * kc * per * nq, st));
+      Pair64Args a = pair64_args(m, k0, kc, nq, wqd, par, p, b.fx);
+      a.cot = b.cotd;
+      a.xbar = (double2 *)b.xb64;
+      a.partialT = b.pT;
+      a.partialE = b.pE;
+      epw_status s = launch_adj64(a, st);
+      if (s != EPW_OK) return fail(s, "no FP64 adjoint kernel for nw=%d, 3nat=%d", m->nw, m->nm);
+      launch_sum_scalar(kc * nqb, b.pT, 1.0, b.sc, st);
+      launch_sum_scalar(kc * nqb, b.pE, 1.0, b.sc + 1, st);
+      if (!b.dgd) continue;
+      // sum over q of conj(P_q(Rp)) Xbar, U_k^dagger, then the sum over k of conj(P_k(Re))
+      FxOp xq = b.Xq, gk = b.Gk, pk = b.Pk;
+      xq.rows = kc * (int)per;
+      const size_t stride = (size_t)xq.rows * 2 * m->nRp;
+      fx_rows(xq.rows, nq, nq, b.xb64, xq, st);
+      CKS(fx_gemm_f64(xq, b.Pq, fx_bits(std::min(nq, FX_KMAX / 2)), b.Bq, 2 * (size_t)m->nRp, m->dstatus, st, false,
+                      stride));
+      launch_adj_rotate64(kc, k0, m->nRp, m->nm, m->nw, splits, stride, b.Bq, p.Uk, b.G1b, st);
+      gk.kpad = pk.kpad = fx_kpad(kc);
+      fx_rows(m->nRp * per, kc, kc, b.G1b, gk, st);
+      fx_phases_conj(kc, kd + 3 * (size_t)k0, m->nRe, m->Re, pk, st);
+      CKS(fx_gemm_f64(gk, pk, fx_bits(std::min(kc, FX_KMAX / 2)), (double *)b.gT, 2 * (size_t)m->nRe, m->dstatus, st,
+                      k0 > 0));
+    }
+  } else if (nk > 0 && nq > 0 && tcb) {
     CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st));
     b.tc.Cpol = m->polar ? (const float2 *)p.Cpol : nullptr;
     b.tc.Uk64 = p.Uk;
@@ -1069,7 +1348,7 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
                                          b.cotd, b.tc, b.tw, (cx<float> *)b.gwbar, b.sc, st);
     if (s != EPW_OK) return fail(s, "tensor-core adjoint failed");
   } else if (nk > 0 && nq > 0) {
-    CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st));
+    CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx));
     b.sg.Pq64 = m->same_eph ? p.PqTph : nullptr;
     if (staged) {
       CKS(tc_staged_phases(m, nq, qd, b.sg, st));
@@ -1145,7 +1424,9 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
     }
   }
   if (b.dgd) {
-    if (prec == EPW_FP64)
+    if (pair64)
+      launch_dg64(m, b.gT, b.dgd, st);
+    else if (prec == EPW_FP64)
       launch_dg_scale<double>(m, (const cx<double> *)b.gwbar, b.dgd, false, st);
     else
       launch_dg_scale<float>(m, (const cx<float> *)b.gwbar, b.dgd, false, st);
@@ -1186,15 +1467,23 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
   const int kper = std::max(1, (std::max(nk, 1) + want - 1) / want);
   struct B {
     Prep p;
+    Fx64 fx;
     TcStaged sg;
     double *partial, *pid, *lamd, *zd, *dosd, *terms, *wkd;
     int nchunk;
   } b;
   auto plan = [&](Arena &A) -> epw_status {
-    plan_prep(A, m, std::max(nk, 1), std::max(nq, 1), wprec, sk, sq, false, true, b.p);
+    plan_fx(A, m, std::max(nk, 1), std::max(nq, 1), fx_dq(m, nq),
+            par->precision == EPW_FP64 && nk > 0 && nq > 0 && fx_pair(m, nk, nq),
+            par->precision == EPW_FP64 && nk > 0 && fx_g1(m, nk), b.fx);
+    plan_prep(A, m, std::max(nk, 1), std::max(nq, 1), wprec, sk, sq, false, true, b.p, &b.fx);
     b.wkd = swk ? A.take<double>((size_t)nk) : nullptr;  // k weights staged from the host
     b.sg = TcStaged{};
     int nchunk = (std::max(nk, 1) + kper - 1) / kper;
+    if (b.fx.pair) {
+      nchunk = 0;
+      for (int k0 = 0; k0 < nk; k0 += b.fx.kc) nchunk += (std::min(b.fx.kc, nk - k0) + kper - 1) / kper;
+    }
     if (tcp) {
       CKS(tc_staged_plan(A, m, std::max(nk, 1), std::max(nq, 1), par->precision == EPW_BF16X3 ? TC_OP_BF16 : TC_OP_TF32,
                          STAGED_CT_BYTES, b.sg, true));
@@ -1240,7 +1529,7 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
     if (b.zd) CK(cudaMemsetAsync(b.zd, 0, sizeof(double) * (size_t)nq, st));
   }
   if (nk > 0 && nq > 0) {
-    CKS(run_prep(m, nk, kd, nq, qd, wprec, par->omega_min_eV, true, p, nullptr, st));
+    CKS(run_prep(m, nk, kd, nq, qd, wprec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx));
   } else if (nk > 0) {
     // bands at k only (N(E_F))
     launch_phases(nk, kd, m->nRe, m->Re, m->rmax, p.PkRM, p.PkT, nullptr, st);
@@ -1251,7 +1540,23 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
     launch_dos_terms(nk, m->nw, p.epsk, wkd, par->EF_eV, par->sigma_eV, b.terms, st);
     launch_sum_scalar(nk, b.terms, 1.0, b.dosd, st);
   }
-  if (nk > 0 && nq > 0) {
+  if (nk > 0 && nq > 0 && b.fx.pair) {
+    launch_tables64(nq, nm, p.omegaT, par->omega_min_eV, par->T_K, b.fx.omK, b.fx.nbT, b.fx.wmax, st);
+    int chunk0 = 0;
+    for (int k0 = 0; k0 < nk; k0 += b.fx.kc) {
+      const int kc = std::min(b.fx.kc, nk - k0), nch = (kc + kper - 1) / kper;
+      CKS(run_fx_contract(m, k0, kc, p, b.fx, st));
+      Pair64Args a = pair64_args(m, k0, kc, nq, nullptr, par, p, b.fx);
+      a.wk = wkd;
+      a.nk_total = nk;
+      a.nkc = kper;
+      a.partial = b.partial + (size_t)chunk0 * nq * (2 * nm + 1);
+      epw_status s = launch_ph64(a, nch, st);
+      if (s != EPW_OK) return fail(s, "no phonon-side kernel for nw=%d, 3nat=%d", m->nw, nm);
+      chunk0 += nch;
+    }
+    launch_ph_finalize(nq, nm, b.nchunk, b.partial, p.omegaT, par->omega_min_eV, b.dosd, b.pid, b.lamd, b.zd, st);
+  } else if (nk > 0 && nq > 0) {
     PairArgs a;
     std::memset(&a, 0, sizeof(a));
     a.nq = nq;
@@ -1544,14 +1849,16 @@ extern "C" epw_status epw_linewidth_noalloc(const epw_model *mc, int nk, const d
   // measure, then lay the buffers out inside the fixed scratch array
   LwPlan L;
   Arena A{nullptr, 0, 0};
-  CKS(plan_linewidth(A, m, nk, nq, prec, false, false, false, false, L));
+  EpwTune tune = epwi_default_tune();
+  tune.simt64 = true;  // the smallest buffers
+  CKS(epwi_plan_linewidth(A, m, nk, nq, prec, false, false, false, false, tune, L));
   if (A.off > EPW_NOALLOC_SCRATCH_BYTES)
     return fail(EPW_ERR_INVALID_ARG, "problem needs %zu bytes of scratch; epw_linewidth_noalloc holds %zu", A.off,
                 (size_t)EPW_NOALLOC_SCRATCH_BYTES);
   char *scratch = nullptr;
   CKS(noalloc_scratch(m->device, &scratch));
   A = Arena{scratch, (size_t)EPW_NOALLOC_SCRATCH_BYTES, 0};
-  CKS(plan_linewidth(A, m, nk, nq, prec, false, false, false, false, L));
+  CKS(epwi_plan_linewidth(A, m, nk, nq, prec, false, false, false, false, tune, L));
   Prep &p = L.p;
   CKS(run_prep(m, nk, k, nq, q, prec, par->omega_min_eV, true, p, nullptr, st, /*fork=*/false));
   PairArgs a;

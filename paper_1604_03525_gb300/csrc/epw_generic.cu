@@ -4,6 +4,7 @@
 // Method: EPW (Ponce et al. 2016), Eq. (linewidthel) for the reduction and the
 // Wannier interpolation of Sec. "Electron-phonon coupling in polar materials"
 // (step iii) with the U rotations of the overlap equation there.
+#include <algorithm>
 #include <type_traits>
 #include <cuda_runtime.h>
 
@@ -67,6 +68,24 @@ __global__ void k_phases_fact(int npt, const double *__restrict__ x, int nR, con
     if (T64) T64[idx] = p;
     if (T32) T32[idx] = mkc((float)p.x, (float)p.y);
   }
+}
+
+// The same sum with 8 lanes per element, for few points: a thread alone would run nR dependent
+// FP64 FMAs of 64 cycles each (24 k of the diamond model: 146 us).
+__global__ void k_fourier_few(int npt, int nR, const cx<double> *__restrict__ PT, const cx<double> *__restrict__ X,
+                              int msize, cx<double> *out) {
+  const size_t idx = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) / 8;
+  const int l = threadIdx.x & 7;
+  const bool in = idx < (size_t)npt * msize;
+  const int i = in ? (int)(idx % npt) : 0, e = in ? (int)(idx / npt) : 0;
+  cx<double> acc = mkc(0.0, 0.0);
+  for (int r = l; r < nR; r += 8) cfma(acc, PT[(size_t)r * npt + i], X[(size_t)r * msize + e]);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+  }
+  if (in && l == 0) out[(size_t)i * msize + e] = acc;
 }
 
 // out[i][e] = sum_r PT[r][i] X[r][e]   (PT transposed phases [nR][npt])
@@ -168,6 +187,38 @@ __global__ void __launch_bounds__(256) k_cgemm(int M, int N, int K, const cx<R> 
         *p = acc ? (*p + c[i][j]) : c[i][j];
       }
     }
+}
+
+// G1[k][c] = sum_r P[k][r] g[r][c] in FP64 for few k: one thread per column and KT k-points, so
+// each 16 bytes of g meet 4 KT FMAs and no thread works on padding (the 64 x 64 tiles of k_cgemm
+// cost 10.2 ms for 3 k as for 24 on the diamond model, 249 x 95,616; this 0.5 and 3.7 ms).
+template <int KT>
+__global__ void __launch_bounds__(128) k_vertex_fewk(int nk, int nR, int ncol, const cx<double> *__restrict__ P,
+                                                     const cx<double> *__restrict__ g, cx<double> *G1) {
+  __shared__ cx<double> Ps[64][KT];
+  const int c = blockIdx.x * 128 + threadIdx.x, k0 = blockIdx.y * KT;
+  cx<double> acc[KT];
+#pragma unroll
+  for (int t = 0; t < KT; t++) acc[t] = mkc(0.0, 0.0);
+  for (int r0 = 0; r0 < nR; r0 += 64) {
+    const int nr = min(64, nR - r0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nr * KT; i += 128) {
+      const int t = i / nr, r = i - t * nr;
+      Ps[r][t] = k0 + t < nk ? P[(size_t)(k0 + t) * nR + r0 + r] : mkc(0.0, 0.0);
+    }
+    __syncthreads();
+    if (c < ncol)
+      for (int r = 0; r < nr; r++) {
+        const cx<double> x = g[(size_t)(r0 + r) * ncol + c];
+#pragma unroll
+        for (int t = 0; t < KT; t++) cfma(acc[t], Ps[r][t], x);
+      }
+  }
+  if (c < ncol)
+#pragma unroll
+    for (int t = 0; t < KT; t++)
+      if (k0 + t < nk) G1[(size_t)(k0 + t) * ncol + c] = acc[t];
 }
 
 // Bg[k][Rp][a][j][n] = sum_i G1[k][Rp][a][j][i] U_k[i][n];  BH[k][Re][i][j] = P_k(Re) Hw(Re)_ij
@@ -1036,7 +1087,10 @@ void launch_phases(int npt, const double *x, int nR, const int *R, int rmax, cx<
                    cx<float> *T32, cudaStream_t st) {
   size_t n = (size_t)npt * nR;
   if (!n) return;
-  if (rmax <= PH_RMAX && nR >= 2 * (2 * PH_RMAX + 1))
+  // FP64 instructions per thread (sincospi about 45) times waves of the 608 x 32 lanes: one thread
+  // per point pays off once the points fill the GPU (1000 k x 135 R: 200 us against 10)
+  const double w1 = std::max(1.0, npt / 19456.0), wn = std::max(1.0, (double)n / 19456.0);
+  if (rmax <= PH_RMAX && (3.0 * (2 * rmax + 1) * 45.0 + 8.0 * nR) * w1 < 52.0 * wn)
     k_phases_fact<<<(npt + 127) / 128, 128, 0, st>>>(npt, x, nR, R, rmax < 0 ? 0 : rmax, rm, T64, T32);
   else
     k_phases<<<nblocks(n, 256), 256, 0, st>>>(npt, x, nR, R, rm, T64, T32);
@@ -1047,7 +1101,10 @@ void launch_fourier_d(int npt, int nR, const cx<double> *PT, const cx<double> *X
                       cudaStream_t st) {
   size_t n = (size_t)npt * msize;
   if (!n) return;
-  k_fourier_d<<<nblocks(n, 256), 256, 0, st>>>(npt, nR, PT, X, msize, out);
+  if (n * 8 <= 4 * 608 * 32)
+    k_fourier_few<<<(unsigned)((n * 8 + 127) / 128), 128, 0, st>>>(npt, nR, PT, X, msize, out);
+  else
+    k_fourier_d<<<nblocks(n, 256), 256, 0, st>>>(npt, nR, PT, X, msize, out);
   epw_count_launch();
 }
 
@@ -1071,6 +1128,19 @@ template void launch_cgemm<double>(int, int, int, const cx<double> *, int, bool,
                                    cx<double> *, int, bool, cudaStream_t);
 template void launch_cgemm<float>(int, int, int, const cx<float> *, int, bool, bool, const cx<float> *, int,
                                   cx<float> *, int, bool, cudaStream_t);
+
+void launch_vertex_fewk(int nk, int nR, int ncol, const cx<double> *P, const cx<double> *g, cx<double> *G1,
+                        cudaStream_t st) {
+  if (nk <= 0 || ncol <= 0) return;
+  const int nb = (ncol + 127) / 128;
+  if (nk >= 4 && (long)nb * ((nk + 3) / 4) >= 608)
+    k_vertex_fewk<4><<<dim3(nb, (nk + 3) / 4), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  else if (nk >= 3 && nb >= 304)
+    k_vertex_fewk<3><<<dim3(nb, (nk + 2) / 3), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  else
+    k_vertex_fewk<1><<<dim3(nb, nk), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  epw_count_launch();
+}
 
 template <typename R>
 void launch_build_B(const epw_model *m, int nk, const cx<double> *Pk, const cx<R> *G1, const cx<double> *Uk,

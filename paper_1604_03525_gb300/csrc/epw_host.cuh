@@ -3,6 +3,7 @@
 // linewidth job and its execution on a stream with device buffers only.
 #pragma once
 #include "epw_internal.cuh"
+#include "epw_pair64.cuh"
 #include "epw_tc.cuh"
 
 // Records the message for epw_last_error (thread-local) and returns s.
@@ -17,6 +18,9 @@ struct EpwTune {
   size_t staged_ct_bytes;  // staged form: contraction buffer per chunk of k
   int wide_form;           // wide-shape form: TCW_FORM_PAIR (fused, CTA pairs), _SPLIT (two kernels), _SINGLE
   size_t k_side_bytes;     // buffers that grow with nk stay within this: larger k lists run in k chunks
+  bool simt64;             // the CUDA cores for FP64 work whatever the size (no fixed-point contractions)
+  bool pair64;             // FP64 form: the pairs' contractions in fixed point (set by the planner from the whole k list)
+  bool g1_64;              // FP64 form: the k-side vertex in fixed point (the same)
 };
 EpwTune epwi_default_tune();
 
@@ -39,9 +43,31 @@ struct Prep {
   void *Cpol;              // [nm][nq] long-range factors C_nu(q), working precision (polar models)
 };
 
+// Fixed-point (tensor-core) contractions of the FP64 work: D(q) in every form, H(k+q) and
+// g(k,q) U_k in the FP64 form.
+struct Fx64 {
+  bool dq;               // D(q) that way
+  bool pair;             // the pairs' contractions that way
+  FxOp Aph, Phi;         // q phases of the Rph set, force constants
+  double *Dh;            // [nq][nm^2] (fx_hermitian's rows)
+  FxOp Ae, Ap;           // q phases of the Re and Rp sets (Aph's planes where the sets agree)
+  FxOp BH, BG;           // k side of one chunk of kc k
+  long long *CH, *CG;    // contractions of one chunk [rows][ldc]
+  double *omK, *nbT;     // frequencies (-1: left out) and Bose factors [nm][nq]
+  double *wmax;          // [nq]
+  int *bad;              // an operand held an infinity or a NaN
+  int kc;
+  size_t ldc;
+  double *Hq;            // interpolation: H(k+q) of one chunk [nq][kc][nw^2] (fx_hermitian's rows)
+  bool g1;               // the k-side vertex g(k,Rp) that way: k phases, a block of g's columns
+  FxOp Ak, Gw;
+  int gcols;
+};
+
 // Buffers of one linewidth job.
 struct LwPlan {
   Prep p;
+  Fx64 fx;
   double *partial;
   double *out_d;
   TcBuffers tc;

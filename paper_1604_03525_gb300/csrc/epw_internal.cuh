@@ -374,6 +374,8 @@ void launch_phonon_post(int nq, int nm, const double *w2, const cx<double> *ev, 
 template <typename R>
 void launch_cgemm(int M, int N, int K, const cx<R> *A, int lda, bool transA, bool conjA, const cx<R> *B, int ldb,
                   cx<R> *C, int ldc, bool accumulate, cudaStream_t st);
+void launch_vertex_fewk(int nk, int nR, int ncol, const cx<double> *P, const cx<double> *g, cx<double> *G1,
+                        cudaStream_t st);
 template <typename R>
 void launch_build_B(const epw_model *m, int nk, const cx<double> *Pk, const cx<R> *G1, const cx<double> *Uk,
                     cx<R> *Bg, cx<R> *BH, cudaStream_t st);
