@@ -6,8 +6,12 @@
 //      the reflectors kept in shared memory; a diagonal phase D makes T = D^dagger T_c D
 //      real (as in the per-thread solver of the wide fused kernel);
 //   2. implicit symmetric QR steps with Wilkinson shifts on T (Golub & Van Loan, Sec.
-//      8.3): every lane runs the same scalar recurrence, lane r applies each Givens
-//      rotation to row r of V (T = V Lambda V^T);
+//      8.3): lane r holds d_r and e_r, every lane runs the same scalar recurrence (its
+//      operands by shuffles), lane r applies each Givens rotation to row r of V
+//      (T = V Lambda V^T, in shared memory, one column carried in a register).  A rolled
+//      loop over the active window: with d, e and the rows of V in registers the chase
+//      was unrolled over all positions, half of the kernel's 52k instructions a pair
+//      (nw = 18), and bound by instruction fetch and registers;
 //   3. the eigenvectors some band n at k can reach, u_m = Q D V e_m, lane m forming u_m;
 //   4. only the (m, n) terms of Eq. (linewidthel) whose Gaussians are not below the
 //      cutoff (|e_nk - e_mk+q| <= max kept w_q,nu + X sigma, X = sqrt(130 ln 2): every
@@ -44,7 +48,7 @@ __device__ __forceinline__ float sp_wmax(float v) {
 // Shared memory of one warp (W: largest nw of the instantiation).
 template <int W>
 struct SpWarp {
-  cx<float> A[W * W];     // H(k+q) during the reduction; then V^T (floats); then X_a
+  cx<float> A[W * W];     // H(k+q) during the reduction; then X_a
   cx<float> Ref[W * W];   // reflector k at Ref[k W + i], i = k+1..n-1; then the term sums
   cx<float> U[W * W];     // eigenvector m at U[i W + m]
   cx<float> E[SP_MMAX * SP_MMAX];  // mode factors of this q, E[a][nu]
@@ -53,6 +57,7 @@ struct SpWarp {
   float tau[W];
   float om[SP_MMAX], nb[SP_MMAX];  // kept frequencies and Bose factors of this q
   float em[W], ek[W];              // eigenvalues at k+q (unsorted), band energies at k
+  float V[W * 33];        // V[row][c] at V[c 33 + row]
   unsigned char tm[W * W], tn[W * W];  // the term list (m, n)
 };
 
@@ -151,115 +156,99 @@ __global__ void __launch_bounds__(SP_WARPS * 32) k_pair_sparse(PairArgs a) {
     }
     if (lane == 0 && n >= 2) S.w[n - 2] = S.A[(n - 1) * W + n - 2];
     __syncwarp();
-    // T = D^dagger T_c D: diagonal d, subdiagonal e = |t|, phases phi (every lane the same)
-    float d[W], e[W];
+    // T = D^dagger T_c D: lane r holds d_r and e_r = |t_r|; phases phi
+    float dr = 0.0f, er = 0.0f;
     {
+      cx<float> u = mkc(1.0f, 0.0f);
+      if (lane < n) dr = S.A[lane * W + lane].x;
+      if (lane < n - 1) {
+        const cx<float> t = S.w[lane];
+        const float m2 = cabs2(t);
+        const float mag = sqrtf(m2);
+        u = m2 > 0.0f ? mkc(t.x / mag, t.y / mag) : mkc(1.0f, 0.0f);
+        er = mag;
+      }
       cx<float> ph = mkc(1.0f, 0.0f);
       if (lane == 0) S.phi[0] = ph;
-#pragma unroll
-      for (int r = 0; r < W; r++) {
-        d[r] = r < n ? S.A[r * W + r].x : 0.0f;
-        e[r] = 0.0f;
-        if (r < n - 1) {
-          const cx<float> t = S.w[r];
-          const float m2 = cabs2(t);
-          const float mag = sqrtf(m2);
-          const cx<float> u = m2 > 0.0f ? mkc(t.x / mag, t.y / mag) : mkc(1.0f, 0.0f);
-          ph = mkc(ph.x * u.x - ph.y * u.y, ph.x * u.y + ph.y * u.x);
-          e[r] = mag;
-          if (lane == 0) S.phi[r + 1] = ph;
-        }
+      for (int r = 0; r < n - 1; r++) {
+        const float ux = __shfl_sync(0xffffffffu, u.x, r), uy = __shfl_sync(0xffffffffu, u.y, r);
+        ph = mkc(ph.x * ux - ph.y * uy, ph.x * uy + ph.y * ux);
+        if (lane == 0) S.phi[r + 1] = ph;
       }
     }
-    // 2. implicit QR steps with Wilkinson shifts on (d, e); lane r keeps row r of V.  A
+    // 2. implicit QR steps with Wilkinson shifts on (d, e); lane r applies them to row r of V.  A
     // subdiagonal entry below 2^-22 max(|d|, |e|) is set to zero; the active block is the
     // bottom unreduced one [l, h].
-    float vr[W];
-#pragma unroll
-    for (int c = 0; c < W; c++) vr[c] = c == lane ? 1.0f : 0.0f;
+    for (int c = 0; c < n; c++) S.V[c * 33 + lane] = c == lane ? 1.0f : 0.0f;
     bool conv = true;
     {
-      float scale = 0.0f;
-#pragma unroll
-      for (int r = 0; r < W; r++) scale = fmaxf(scale, fmaxf(fabsf(d[r]), fabsf(e[r])));
+      const float scale = sp_wmax(fmaxf(fabsf(dr), fabsf(er)));
       const float tol = 2.384185791015625e-07f * scale;
       const int maxit = 8 * n;
 #pragma unroll 1
       for (int it = 0;; it++) {
-        int h = 0;
-#pragma unroll
-        for (int r = 0; r < W - 1; r++) {
-          if (fabsf(e[r]) <= tol) e[r] = 0.0f;
-          if (e[r] != 0.0f) h = r + 1;
-        }
+        if (fabsf(er) <= tol) er = 0.0f;
+        const unsigned live = __ballot_sync(0xffffffffu, er != 0.0f);
+        const int h = 32 - __clz(live);  // 0: none
         if (h == 0) break;
         if (it == maxit) {
           conv = false;
           break;
         }
-        int l = 0;
-#pragma unroll
-        for (int r = 0; r < W - 1; r++)
-          if (r < h && e[r] == 0.0f) l = r + 1;
+        const int l = 32 - __clz(~live & ((1u << h) - 1u));
         // Wilkinson shift from the trailing 2 x 2 block [[p, b], [b, s]] of [l, h]
-        float pa = 0.0f, sc = 0.0f, b = 0.0f, x = 0.0f, z = 0.0f;
-#pragma unroll
-        for (int r = 0; r < W - 1; r++) {
-          if (r == h - 1) {
-            pa = d[r];
-            sc = d[r + 1];
-            b = e[r];
-          }
-          if (r == l) {
-            x = d[r];
-            z = e[r];
-          }
-        }
+        const float pa = __shfl_sync(0xffffffffu, dr, h - 1), sc = __shfl_sync(0xffffffffu, dr, h);
+        const float b = __shfl_sync(0xffffffffu, er, h - 1);
+        float x = __shfl_sync(0xffffffffu, dr, l), z = __shfl_sync(0xffffffffu, er, l);
+        float ak = x, ok = z;  // d_r, e_r of the position
         const float del = 0.5f * (pa - sc);
         const float rr = sqrtf(fmaf(del, del, b * b));
         const float den = del >= 0.0f ? del + rr : del - rr;
         const float mu = den != 0.0f ? sc - b * (b / den) : sc;
         x -= mu;
         // bulge chase over the Givens positions l..h-1 (T <- G^T T G, G = [[c, s], [-s, c]])
-#pragma unroll
-        for (int r = 0; r < W - 1; r++) {
-          if (r >= l && r < h) {
-            const float r2 = fmaf(x, x, z * z);
-            const bool rot = r2 > 0.0f;
-            const float ri = rot ? sp_rsqrt(r2) : 0.0f;
-            const float cg = rot ? x * ri : 1.0f, sg = rot ? -z * ri : 0.0f;
-            if (r > 0 && rot && r > l) e[r - 1] = r2 * ri;
-            const float ak = d[r], bk = d[r + 1], ok = e[r];
-            const float cc = cg * cg, ss = sg * sg, cs = cg * sg;
-            d[r] = fmaf(cc, ak, fmaf(-2.0f * cs, ok, ss * bk));
-            d[r + 1] = fmaf(ss, ak, fmaf(2.0f * cs, ok, cc * bk));
-            e[r] = fmaf(cs, ak - bk, (cc - ss) * ok);
-            if (rot && r + 1 < h) {
-              const float en = e[r + 1];
-              z = -sg * en;
-              e[r + 1] = cg * en;
-              x = e[r];
-            }
-            const float v0 = vr[r], v1 = vr[r + 1];
-            vr[r] = fmaf(-sg, v1, cg * v0);
-            vr[r + 1] = fmaf(sg, v0, cg * v1);
+        float vc = S.V[l * 33 + lane];
+#pragma unroll 1
+        for (int r = l; r < h; r++) {
+          const float bk = __shfl_sync(0xffffffffu, dr, r + 1), en = __shfl_sync(0xffffffffu, er, r + 1);
+          const float v1 = S.V[(r + 1) * 33 + lane];
+          const float r2 = fmaf(x, x, z * z);
+          const bool rot = r2 > 0.0f;
+          const float ri = rot ? sp_rsqrt(r2) : 0.0f;
+          const float cg = rot ? x * ri : 1.0f, sg = rot ? -z * ri : 0.0f;
+          if (lane == r - 1 && rot && r > l) er = r2 * ri;
+          const float cc = cg * cg, ss = sg * sg, cs = cg * sg;
+          const float dn = fmaf(cc, ak, fmaf(-2.0f * cs, ok, ss * bk));
+          const float dn1 = fmaf(ss, ak, fmaf(2.0f * cs, ok, cc * bk));
+          const float e0 = fmaf(cs, ak - bk, (cc - ss) * ok);
+          if (lane == r) {
+            dr = dn;
+            er = e0;
           }
+          ak = dn1;
+          ok = en;
+          if (rot && r + 1 < h) {
+            z = -sg * en;
+            ok = cg * en;
+            x = e0;
+          }
+          S.V[r * 33 + lane] = fmaf(-sg, v1, cg * vc);
+          vc = fmaf(sg, vc, cg * v1);
         }
+        if (lane == h) dr = ak;
+        S.V[h * 33 + lane] = vc;
       }
     }
     if (!conv && lane == 0) atomicOr(a.dstatus, EPW_DEV_NOT_CONVERGED);
-    if (lane == 0) {
-#pragma unroll
-      for (int r = 0; r < W; r++)
-        if (r < n) S.em[r] = d[r];
-    }
+    if (lane < n) S.em[lane] = dr;
+    __syncwarp();
     // reachable (m, n): lane n's bands m, as a bit mask; the term list in lane order
     unsigned mask = 0;
     if (lane < n && thr >= 0.0f) {
       const float ekn = S.ek[lane];
 #pragma unroll
       for (int m = 0; m < W; m++)
-        if (m < n && fabsf(ekn - d[m]) <= thr) mask |= 1u << m;
+        if (m < n && fabsf(ekn - S.em[m]) <= thr) mask |= 1u << m;
     }
     const unsigned need = __reduce_or_sync(0xffffffffu, mask);
     int off = __popc(mask);
@@ -270,14 +259,7 @@ __global__ void __launch_bounds__(SP_WARPS * 32) k_pair_sparse(PairArgs a) {
     }
     const int nterm = __shfl_sync(0xffffffffu, off, 31);
     off -= __popc(mask);
-    // V^T into the A region (H is no longer needed), for the eigenvector columns
     __syncwarp();
-    float *Vt = reinterpret_cast<float *>(S.A);
-    if (lane < n) {
-#pragma unroll
-      for (int c = 0; c < W; c++)
-        if (c < n) Vt[lane * W + c] = vr[c];
-    }
     {
       unsigned mm = mask;
       int j = off;
@@ -296,7 +278,7 @@ __global__ void __launch_bounds__(SP_WARPS * 32) k_pair_sparse(PairArgs a) {
       cx<float> u[W];
 #pragma unroll
       for (int r = 0; r < W; r++) {
-        const float y = r < n ? Vt[r * W + lane] : 0.0f;
+        const float y = r < n ? S.V[lane * 33 + r] : 0.0f;
         const cx<float> ph = r < n ? S.phi[r] : mkc(0.0f, 0.0f);
         u[r] = mkc(ph.x * y, ph.y * y);
       }
