@@ -13,6 +13,7 @@
 //   - many matrices: one thread per matrix, in registers for n <= 6 (k_eigh_reg).
 // launch_eigh_d takes the form whose count times waves of warps is smallest (eigh_cost).
 #include <algorithm>
+#include <cmath>
 
 #include "epw_internal.cuh"
 
@@ -295,7 +296,9 @@ void eigh_coop(int nmat, int n, const cx<double> *A, double *w, cx<double> *V, u
 // 4 567; 13,824 of 9 x 9, 1 2950, 4 3710; 316,000 of 6 x 6, 1 8917, 4 17,679.  The other kernels
 // of the preparation share the FP64 pipe, so more lanes have to win by a quarter.
 double eigh_cost(long nmat, int n, int L) {
-  const double waves = std::max(1.0, (double)((nmat * L + 31) / 32) / 608.0);
+  // (the L-lane form in blocks of four warps, one per sub-partition)
+  const double waves = L == 1 ? std::max(1.0, std::ceil((nmat + 31) / 32 / 608.0))
+                              : std::max(1.0, std::ceil((nmat * L + 127) / 128 / 152.0));
   const double rows = L == 1 ? 2.0 * n - 2.0 : (double)((2 * n + L - 1) / L);
   return waves * (40.0 + 12.0 * rows) * (L == 1 ? 1.0 : 1.25);
 }
@@ -324,6 +327,12 @@ void launch_eigh_d(int nmat, int n, cx<double> *A, double *w, cx<double> *V, uns
   else if (L == 4)
     eigh_coop<4>(nmat, n, A, w, V, dstatus, st);
   else {
+    if (n > 6) {
+      // indexed arrays live in L1, but not in all of it: with no shared memory left on an SM no
+      // block that needs some can join it while this kernel runs
+      const void *f = n == 7 ? (const void *)k_eigh_loc<7> : n == 8 ? (const void *)k_eigh_loc<8> : (const void *)k_eigh_loc<9>;
+      cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
+    }
     switch (n) {
       case 1: k_eigh_reg<1><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
       case 2: k_eigh_reg<2><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;

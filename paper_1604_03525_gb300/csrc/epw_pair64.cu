@@ -390,23 +390,27 @@ __device__ __forceinline__ void pair64_g(const Pair64Args &a, int kl, int q, int
 // terms, the busiest lane of a warp twice that).  term(lane of the pair, n) runs for every
 // term, with the pair's eigenvector, eigenvalue and occupation in sw; step(r0, own0, own1) after
 // the terms r0 .. r0 + 31, with the range of this lane's own terms.
+// (reach: whether a term (band n = j with FP32 energy ek, e_mk+q = em in FP32) is wanted)
+struct P64Window {
+  float thr;
+  __device__ __forceinline__ bool operator()(float ek, float em) const { return p64_reach(ek, em, thr); }
+};
 struct P64NoStep {
   __device__ __forceinline__ void operator()(int, int, int) const {}
 };
-template <int W, bool EX, class F, class G = P64NoStep>
-__device__ __forceinline__ void p64_terms(const Pair64Args &a, const Eig64<W, EX> &S, const float *ekf, double thr,
-                                          P64Warp<W> &sw, F &&term, G step = G{}) {
+template <int W, bool EX, class R, class F, class G = P64NoStep>
+__device__ __forceinline__ void p64_terms(const Pair64Args &a, const Eig64<W, EX> &S, const float *ekf, bool any,
+                                          R reach, P64Warp<W> &sw, F &&term, G step = G{}) {
   const int lane = threadIdx.x & 31;
   const int n = EX ? W : a.nw;
-  const float thrf = __double2float_ru(thr);
   unsigned need = 0;
-  if (thr >= 0.0) {
+  if (any) {
 #pragma unroll(W <= P64_REGW ? W : 1)
     for (int m = 0; m < W; m++) {
       if (m >= n) continue;
       const float em = (float)S.eigenvalue(m);
       for (int j = 0; j < n; j++)
-        if (p64_reach(ekf[j], em, thrf)) need |= 1u << m;
+        if (reach(ekf[j], em)) need |= 1u << m;
     }
   }
   while (__any_sync(0xffffffffu, need != 0)) {
@@ -417,7 +421,7 @@ __device__ __forceinline__ void p64_terms(const Pair64Args &a, const Eig64<W, EX
       const double em = S.eigenvalue(m);
       const float emf = (float)em;
       for (int j = 0; j < n; j++)
-        if (p64_reach(ekf[j], emf, thrf)) todo |= 1u << j;
+        if (reach(ekf[j], emf)) todo |= 1u << j;
       double2 u[W];
       S.vector(n, m, u);
 #pragma unroll(W <= 9 ? W : 1)
@@ -474,7 +478,7 @@ __global__ void __launch_bounds__(128, 2) k_lw64(Pair64Args a) {
   for (int j = 0; j < W; j++) acc[j] = 0.0;
   P64Warp<W> &sw = sws[warp];
   const int qw = qi - lane;
-  p64_terms<W, EX>(a, S, ekf, thr, sw, [&](int sl, int nb) {
+  p64_terms<W, EX>(a, S, ekf, thr >= 0.0, P64Window{__double2float_ru(thr)}, sw, [&](int sl, int nb) {
     const int qs = qw + sl;
     double2 g[MM];
     pair64_g<W, EX, MM>(a, kl, qs, nb, sw.u, sl, g);
@@ -545,7 +549,7 @@ __global__ void __launch_bounds__(128, 2) k_adj64(Pair64Args a) {
   const int qw = qi - lane;
   double sT = 0.0, sE = 0.0;
   double2 *xb = a.xbar + (size_t)kl * nm * n * n * a.nq;
-  p64_terms<W, EX>(a, S, ekf, thr, sw, [&](int sl, int nb) {
+  p64_terms<W, EX>(a, S, ekf, thr >= 0.0, P64Window{__double2float_ru(thr)}, sw, [&](int sl, int nb) {
     const int qs = qw + sl;
     double2 g[MM];
     pair64_g<W, EX, MM>(a, kl, qs, nb, sw.u, sl, g);
@@ -627,8 +631,6 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
   P64Warp<W> &sw = sws[warp];
   const double wm = a.wmax[q];
   double thr = valid && __double2hiint(wm) >= 0 ? wm + P64_CUT * a.sigma : -1.0;
-  // a pair of bands that both lie within the Gaussian of E_F counts for lambda
-  if (thr >= 0.0) thr = fmax(thr, 2.0 * P64_CUT * a.sigma);
   if (thr >= 0.0 && *a.bad) thr = __longlong_as_double(0x7ff0000000000000LL);
   double sp[MM], sl_[MM], sz = 0.0;
 #pragma unroll
@@ -661,8 +663,14 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
       }
       sz = fma(wk * zn, a.gnorm * zm, sz);
     }
+    // Pi'': |e_nk - e_mk+q - w| within the Gaussian; lambda: both bands within that of E_F
+    const float thrf = __double2float_ru(thr), cutf = __double2float_ru(P64_CUT * a.sigma), ef = (float)a.EF;
     p64_terms<W, EX>(
-        a, S, ekf, thr, sw,
+        a, S, ekf, thr >= 0.0,
+        [&](float en, float em) {
+          return p64_reach(en, em, thrf) || (p64_reach(en, ef, cutf) && p64_reach(em, ef, cutf));
+        },
+        sw,
         [&](int sl, int nb) {
           const int qs = qw + sl;
           const double em = sw.em[sl], en = ek[nb], x = en - em, dn = dn_s[nb];
@@ -732,17 +740,18 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
 }
 
 // e_k+q and g_mn,nu = sum_a E[a][nu] (U_k+q^dagger X_a)_mn (plus the long-range part): lanes over q
-// (the contractions' contiguous index), the block's 8 rows over (m, n).
+// (the contractions' contiguous index), one (m, n) per row of the block.
 __global__ void __launch_bounds__(256) k_g64(Pair64Args a) {
   const int q = blockIdx.x * 32 + threadIdx.x, kl = blockIdx.y, k = a.k0 + kl;
   if (q >= a.nq) return;
   const int n = a.nw, nm = a.nm, n2 = n * n;
   const size_t pr = (size_t)q * a.nk + kl;
-  if (a.eps_kq && threadIdx.y == 0)
+  if (a.eps_kq && threadIdx.y == 0 && blockIdx.z == 0)
     for (int m = 0; m < n; m++) a.eps_kq[((size_t)k * a.nq + q) * n + m] = a.wkq[pr * n + m];
   if (!a.gout) return;
   const cx<double> *U = a.Ukq + pr * n2, *Uk = a.Uk + (size_t)k * n2;
-  for (int mn = threadIdx.y; mn < n2; mn += 8) {
+  const int mn = blockIdx.z * 8 + threadIdx.y;
+  if (mn < n2) {
     const int m = mn / n, nb = mn - m * n;
     double2 g[P64_MM];
 #pragma unroll
@@ -914,7 +923,7 @@ epw_status launch_ph64(const Pair64Args &a, int nchunk, cudaStream_t st) {
 
 epw_status launch_g64(const Pair64Args &a, cudaStream_t st) {
   if (a.nk <= 0 || a.nq <= 0) return EPW_OK;
-  k_g64<<<dim3((a.nq + 31) / 32, a.nk), dim3(32, 8), 0, st>>>(a);
+  k_g64<<<dim3((a.nq + 31) / 32, a.nk, a.gout ? (a.nw * a.nw + 7) / 8 : 1), dim3(32, 8), 0, st>>>(a);
   epw_count_launch();
   return cudaGetLastError() == cudaSuccess ? EPW_OK : EPW_ERR_CUDA;
 }
