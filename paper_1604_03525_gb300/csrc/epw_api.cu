@@ -84,11 +84,12 @@ static void free_model_arrays(epw_model *m) {
   if (m->ev_fork) cudaEventDestroy(m->ev_fork);
   if (m->ev_join) cudaEventDestroy(m->ev_join);
   if (m->ev_phase) cudaEventDestroy(m->ev_phase);
+  if (m->ev_gate) cudaEventDestroy(m->ev_gate);
   if (m->aux2) cudaStreamDestroy(m->aux2);
   if (m->ev_fork2) cudaEventDestroy(m->ev_fork2);
   if (m->ev_join2) cudaEventDestroy(m->ev_join2);
   m->aux = m->aux2 = nullptr;
-  m->ev_fork = m->ev_join = m->ev_phase = m->ev_fork2 = m->ev_join2 = nullptr;
+  m->ev_fork = m->ev_join = m->ev_phase = m->ev_gate = m->ev_fork2 = m->ev_join2 = nullptr;
   if (m->ev) {
     for (int i = 0; i < 2 * EPW_MAX_TIMED; i++)
       if (m->ev[i]) cudaEventDestroy(m->ev[i]);
@@ -470,9 +471,26 @@ static void plan_fx(Arena &A, const epw_model *m, int nk, int nq, bool dq, bool 
   f.bad = A.take<int>(1);
 }
 
+struct PhaseA;
+static PhaseA staged_a(const epw_model *m, TcStaged &s);
+// The A operand of a tensor-core form that takes the phases of one R set, Re = Rp: built with the
+// planes of D(q) when there are any and Re = Rph.
+struct PhaseA {
+  int op, kpad;
+  void *hi, *lo;
+  bool *done;
+};
+static PhaseA staged_a(const epw_model *m, TcStaged &s) {
+  // (with two R sets the operand is built from q: no destination here)
+  return m->same_ep ? PhaseA{s.op, s.kpad, s.Ahi, s.Alo, &s.a_done} : PhaseA{s.op, s.kpad, nullptr, nullptr, &s.a_done};
+}
 // q side: the phases' planes and D(q).
-static epw_status run_fx_q(const epw_model *m, int nq, const double *q, Fx64 &f, cx<double> *D, cudaStream_t st) {
-  fx_phases(nq, q, m->nRph, m->Rph, m->rmax, f.Aph, st);
+static epw_status run_fx_q(const epw_model *m, int nq, const double *q, Fx64 &f, cx<double> *D, cudaStream_t st,
+                           const PhaseA *pa) {
+  if (pa)
+    tc_phases_a(pa->op, nq, q, m->nRe, m->Re, m->rmax, f.Aph, pa->kpad, pa->hi, pa->lo, st);
+  else
+    fx_phases(nq, q, m->nRph, m->Rph, m->rmax, f.Aph, st);
   fx_hermitian(1, m->nRph, m->nm, nullptr, m->Phiw, f.Phi, nullptr, st);
   CKS(fx_gemm_f64(f.Aph, f.Phi, fx_bits(m->nRph), f.Dh, (size_t)m->nm * m->nm, m->dstatus, st));
   fx_unpack_hermitian(nq, m->nm, f.Dh, D, st);
@@ -566,6 +584,7 @@ static epw_status prep_streams(epw_model *m) {
   CK(cudaEventCreateWithFlags(&m->ev_fork, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&m->ev_join, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&m->ev_phase, cudaEventDisableTiming));
+  CK(cudaEventCreateWithFlags(&m->ev_gate, cudaEventDisableTiming));
   CK(cudaStreamCreateWithFlags(&m->aux2, cudaStreamNonBlocking));
   CK(cudaEventCreateWithFlags(&m->ev_fork2, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&m->ev_join2, cudaEventDisableTiming));
@@ -577,7 +596,8 @@ static epw_status prep_streams(epw_model *m) {
 // phonon work (FP64) still runs on the second stream.
 static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq, const double *q, int prec,
                            double omega_min, bool need_B, Prep &p, double *omega_out, cudaStream_t st,
-                           bool fork = true, TcBuffers *tcb = nullptr, Fx64 *fx = nullptr) {
+                           bool fork = true, TcBuffers *tcb = nullptr, Fx64 *fx = nullptr,
+                           const PhaseA *pa = nullptr) {
   epw_model *m = const_cast<epw_model *>(mc);
   const int nw = m->nw, nm = m->nm;
   const size_t nw2 = (size_t)nw * nw;
@@ -600,6 +620,12 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
     launch_phases(nq, q, m->nRe, m->Re, m->rmax, nullptr, (cx<double> *)p.PqTe, nullptr, sq);
     if (!m->same_ep) launch_phases(nq, q, m->nRp, m->Rp, m->rmax, nullptr, (cx<double> *)p.PqTp, nullptr, sq);
     if (!m->same_eph) launch_phases(nq, q, m->nRph, m->Rph, m->rmax, nullptr, p.PqTph, nullptr, sq);
+  } else if (pa) {
+    // staged and wide forms read no phase arrays: the A operand (from FP64 phases when Re = Rph)
+    const bool dq = fx && fx->dq;
+    *pa->done = dq && m->same_eph && pa->hi;
+    if (!*pa->done && (!dq || (m->same_eph && pa->hi)))
+      launch_phases(nq, q, m->nRph, m->Rph, m->rmax, nullptr, p.PqTph, nullptr, sq);
   } else {
     launch_phases(nq, q, m->nRe, m->Re, m->rmax, nullptr, m->same_eph ? p.PqTph : nullptr, (cx<float> *)p.PqTe, sq);
     if (!m->same_ep) launch_phases(nq, q, m->nRp, m->Rp, m->rmax, nullptr, nullptr, (cx<float> *)p.PqTp, sq);
@@ -608,10 +634,16 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   if (tcb && fork && !qs) CK(cudaEventRecord(m->ev_phase, sq));
   // phonons (FP64 eigensolve)
   if (!qs && fx && fx->dq) {
-    CKS(run_fx_q(m, nq, q, *fx, p.D, sq));
+    CKS(run_fx_q(m, nq, q, *fx, p.D, sq, pa && *pa->done ? pa : nullptr));
   } else if (!qs) {
     launch_fourier_d(nq, m->nRph, p.PqTph, m->Phiw, nm * nm, p.D, sq);
   }
+  // The eigensolves are one long wave of FP64-bound warps: they start on an empty GPU and spread
+  // over every SM, and the k-side vertex (a GEMM that fills the GPU) starts after them.  The other
+  // way round their blocks share the few SMs that happen to have room (13,824 of 9 x 9: 6.6 ms
+  // against 2.4; 1728: 3.3 against 0.8).
+  const bool gate = fork && fx && fx->dq;
+  if (gate) CK(cudaEventRecord(m->ev_gate, sq));
   launch_eigh_d(nq, nm, p.D, p.w2, p.ev, m->dstatus, sq);
   launch_phonon_post(nq, nm, p.w2, p.ev, m->mass, omega_min, p.omegaT,
                      prec == EPW_FP64 ? (cx<double> *)p.ET : nullptr, prec == EPW_FP64 ? nullptr : (cx<float> *)p.ET,
@@ -638,6 +670,7 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   if (fork2) CK(cudaEventRecord(m->ev_join2, sk));
   if (need_B && nk > 0) {
     const int ncol = m->nRp * nm * (int)nw2;
+    if (gate) CK(cudaStreamWaitEvent(st, m->ev_gate, 0));
     if (prec == EPW_FP64) {
       CKS(run_vertex64(m, nk, k, p, fx, st));
       if (fork2) CK(cudaStreamWaitEvent(st, m->ev_join2, 0));
@@ -936,14 +969,16 @@ static epw_status linewidth_pass(epw_model *m, int nk, const double *kd, int nq,
     if (s != EPW_OK) return fail(s, "tensor-core path: %s", g_err[0] ? g_err : "unsupported shape");
   } else if (tcp && L.w.ok) {
     // wide-shape fused form: per chunk of k, the H(k+q) eigensolve kernel and the vertex kernel
-    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &L.fx));
+    const PhaseA pa{L.w.op, L.w.kpad, L.w.Ahi, L.w.Alo, &L.w.a_done};
+    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &L.fx, &pa));
     epw_status s = tcw_linewidth(m, nk, nq, qd, wqd, par, p.epsk, p.omegaT, (const cx<float> *)p.ET,
                                  (const cx<float> *)p.Bg, (const cx<float> *)p.BH, m->same_eph ? p.PqTph : nullptr,
                                  p.Uk, m->polar ? (const float2 *)p.Cpol : nullptr, L.w, out, st);
     if (s != EPW_OK) return fail(s, "wide tensor-core path: %s", g_err[0] ? g_err : "launch failed");
   } else if (tcp) {
     // staged tensor-core form: contraction per chunk of k on the tensor cores, per-pair work from HBM
-    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &L.fx));
+    const PhaseA pa = staged_a(m, L.sg);
+    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &L.fx, &pa));
     L.sg.Pq64 = m->same_eph ? p.PqTph : nullptr;
     CKS(tc_staged_phases(m, nq, qd, L.sg, st));
     epw_timing_begin(m, st);
@@ -1348,7 +1383,9 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
                                          b.cotd, b.tc, b.tw, (cx<float> *)b.gwbar, b.sc, st);
     if (s != EPW_OK) return fail(s, "tensor-core adjoint failed");
   } else if (nk > 0 && nq > 0) {
-    CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx));
+    const PhaseA pa = staged_a(m, b.sg);
+    CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx,
+                 staged ? &pa : nullptr));
     b.sg.Pq64 = m->same_eph ? p.PqTph : nullptr;
     if (staged) {
       CKS(tc_staged_phases(m, nq, qd, b.sg, st));
@@ -1394,7 +1431,8 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
         a.ldc = b.sg.pair_ld();
         a.cpk = b.sg.cpk;
       }
-      epw_status s = staged ? launch_pair_staged(a, 2, st)
+      if (staged) CK(cudaMemsetAsync(b.xbar, 0, sR * (size_t)nq * kc * per, st));
+      epw_status s = staged ? launch_adj_staged(a, st)
                             : prec == EPW_FP64 ? launch_pair<double>(a, 2, st) : launch_pair<float>(a, 2, st);
       if (s != EPW_OK) return fail(s, "no per-pair kernel for nw=%d, 3nat=%d", m->nw, m->nm);
       launch_sum_scalar(kc * nqb, b.pT, 1.0, b.sc, st);
@@ -1529,7 +1567,9 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
     if (b.zd) CK(cudaMemsetAsync(b.zd, 0, sizeof(double) * (size_t)nq, st));
   }
   if (nk > 0 && nq > 0) {
-    CKS(run_prep(m, nk, kd, nq, qd, wprec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx));
+    const PhaseA pa = staged_a(m, b.sg);
+    CKS(run_prep(m, nk, kd, nq, qd, wprec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx,
+                 tcp ? &pa : nullptr));
   } else if (nk > 0) {
     // bands at k only (N(E_F))
     launch_phases(nk, kd, m->nRe, m->Re, m->rmax, p.PkRM, p.PkT, nullptr, st);
@@ -1645,12 +1685,14 @@ extern "C" epw_status epw_selfenergy(const epw_model *mc, int nk, const double *
   int kc = (int)std::max<size_t>(1, std::min<size_t>((size_t)nk, ((size_t)1 << 30) / per_k));
   struct B {
     Prep p;
+    Fx64 fx;
     TcStaged sg;
-    double *omd, *sigd, *specd;
+    double *omd, *sigd, *specd, *re0;
     double2 *part;
   } b;
   auto plan = [&](Arena &A) -> epw_status {
-    plan_prep(A, m, nk, std::max(nq, 1), wprec, sk, sq, swq, true, b.p);
+    plan_fx(A, m, nk, std::max(nq, 1), fx_dq(m, nq), false, wprec == EPW_FP64 && nq > 0 && fx_g1(m, nk), b.fx);
+    plan_prep(A, m, nk, std::max(nq, 1), wprec, sk, sq, swq, true, b.p, &b.fx);
     b.sg = TcStaged{};
     if (tcp) {
       CKS(tc_staged_plan(A, m, nk, std::max(nq, 1), par->precision == EPW_BF16X3 ? TC_OP_BF16 : TC_OP_TF32,
@@ -1662,6 +1704,7 @@ extern "C" epw_status epw_selfenergy(const epw_model *mc, int nk, const double *
     b.sigd = ssig ? (double *)A.take<double2>(nout) : sigma;
     b.specd = ssp ? A.take<double>(nout) : spectral;
     b.part = A.take<double2>((size_t)kc * nqw * nw * (nomega + 1));
+    b.re0 = A.take<double>((size_t)kc * nw);
     return EPW_OK;
   };
   Arena A{nullptr, 0, 0};
@@ -1689,7 +1732,9 @@ extern "C" epw_status epw_selfenergy(const epw_model *mc, int nk, const double *
     CK(cudaMemsetAsync(b.sigd, 0, nout * sizeof(double2), st));
     if (b.specd) CK(cudaMemsetAsync(b.specd, 0, nout * sizeof(double), st));
   } else {
-    CKS(run_prep(m, nk, kd, nq, qd, wprec, par->omega_min_eV, true, p, nullptr, st));
+    const PhaseA pa = staged_a(m, b.sg);
+    CKS(run_prep(m, nk, kd, nq, qd, wprec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx,
+                 tcp ? &pa : nullptr));
     b.sg.Pq64 = m->same_eph ? p.PqTph : nullptr;
     if (tcp) CKS(tc_staged_phases(m, nq, qd, b.sg, st));
     PairArgs a;
@@ -1728,7 +1773,7 @@ extern "C" epw_status epw_selfenergy(const epw_model *mc, int nk, const double *
       epw_status s = wprec == EPW_FP64 ? launch_pair_se<double>(a, nomega, b.omd, delta, b.part, st)
                                        : launch_pair_se<float>(a, nomega, b.omd, delta, b.part, st);
       if (s != EPW_OK) return fail(s, "no self-energy kernel for nw=%d, 3nat=%d", nw, m->nm);
-      launch_se_finalize(n, k0, nw, nqw, nomega, b.part, b.omd, p.epsk, par->EF_eV, (double2 *)b.sigd, b.specd, st);
+      launch_se_finalize(n, k0, nw, nqw, nomega, b.part, b.omd, p.epsk, par->EF_eV, (double2 *)b.sigd, b.specd, b.re0, st);
     }
   }
   CK(cudaGetLastError());

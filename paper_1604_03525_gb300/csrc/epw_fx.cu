@@ -278,76 +278,21 @@ __global__ void __launch_bounds__(FX_THREADS, 1)
 }
 
 // ------------------------------------------------------------ digit planes
-// The digits of X (|X| <= 2^55), most significant first, as bf16 pairs (x in the low half).
-// Balanced base 256: adding 128 to each of the six lower bytes makes them unsigned, the rest is d_1.
-__device__ __forceinline__ void fx_digits2(long long X, long long Y, uint32_t (&p)[FX_S]) {
-  const long long bias = 0x0000808080808080LL;
-  const long long xb = X + bias, yb = Y + bias;
-  const uint32_t x0 = (uint32_t)xb, x1 = (uint32_t)(xb >> 32), y0 = (uint32_t)yb, y1 = (uint32_t)(yb >> 32);
-  auto pack = [](float a, float b) { return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632); };
-  p[0] = pack((float)((int)x1 >> 16), (float)((int)y1 >> 16));
-#pragma unroll
-  for (int i = 1; i < FX_S; i++) {
-    const int b = FX_S - 1 - i;  // byte
-    const uint32_t xs = b >= 4 ? x1 : x0, ys = b >= 4 ? y1 : y0;
-    const uint32_t fx = __byte_perm(xs, 0x4B000000u, 0x7440 | (b & 3)), fy = __byte_perm(ys, 0x4B000000u, 0x7440 | (b & 3));
-    p[i] = pack(__uint_as_float(fx) - 8388736.0f, __uint_as_float(fy) - 8388736.0f);  // byte - 128
-  }
-}
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
 
-constexpr int FX_PRMAX = 8;
-// Blocks of 4 warps take 16 points: the one-axis factors e^{2 pi i (x_j n mod 1)}, n = 1..rmax
-// (n < 0: the conjugate), one per thread, then a warp per point, lanes over R (128-byte stores
-// per plane).  rmax > FX_PRMAX: the phase of each R by itself.
 __global__ void __launch_bounds__(128) k_fx_phases(int npt, const double *__restrict__ x, int nR,
                                                    const int *__restrict__ R, int rmax, int kpad, size_t plane,
                                                    __nv_bfloat16 *d, short *e) {
-  __shared__ double2 F[16][3][2 * FX_PRMAX + 1];
-  const int p0 = blockIdx.x * 16, np = min(16, npt - p0);
-  const bool fact = rmax <= FX_PRMAX;
-  if (fact) {
-    const int per = 3 * (rmax + 1);
-    for (int t = threadIdx.x; t < np * per; t += 128) {
-      const int p = t / per, j = (t - p * per) / (rmax + 1), n = t % (rmax + 1);
-      double a = x[3 * (size_t)(p0 + p) + j] * n;
-      a -= rint(a);
-      double s, c;
-      sincospi(2.0 * a, &s, &c);
-      F[p][j][FX_PRMAX + n] = make_double2(c, s);
-      F[p][j][FX_PRMAX - n] = make_double2(c, -s);
-    }
-  }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int p = warp; p < np; p += 4) {
-    const size_t row = (size_t)(p0 + p);
-    const double q0 = x[3 * row], q1 = x[3 * row + 1], q2 = x[3 * row + 2];
-    const bool fin = isfinite(q0) && isfinite(q1) && isfinite(q2);
-    if (lane == 0 && e) e[row] = fin ? 0 : FX_BAD;
-    for (int r = lane; r < kpad / 2; r += 32) {
-      double c = 0.0, s = 0.0;
-      if (r < nR && fin) {
-        if (fact) {
-          const double2 f0 = F[p][0][R[3 * r] + FX_PRMAX], f1 = F[p][1][R[3 * r + 1] + FX_PRMAX],
-                        f2 = F[p][2][R[3 * r + 2] + FX_PRMAX];
-          const double2 f = make_double2(fma(f0.x, f1.x, -f0.y * f1.y), fma(f0.x, f1.y, f0.y * f1.x));
-          c = fma(f.x, f2.x, -f.y * f2.y);
-          s = fma(f.x, f2.y, f.y * f2.x);
-        } else {
-          double a = q0 * R[3 * r] + q1 * R[3 * r + 1] + q2 * R[3 * r + 2];
-          a -= rint(a);
-          sincospi(2.0 * a, &s, &c);
-        }
-      }
-      // |c|, |s| exceed 1 by rounding at most, which the leading digit has room for
-      uint32_t pl[FX_S];
-      fx_digits2(__double2ll_rn(c * 36028797018963968.0), __double2ll_rn(s * 36028797018963968.0), pl);  // 2^55
-      uint32_t *o = reinterpret_cast<uint32_t *>(d + row * kpad) + r;
+  __shared__ FxFactors F;
+  fx_point_phases(
+      npt, x, nR, R, rmax, kpad / 2, F, [&](size_t row, bool fin) { e[row] = fin ? 0 : FX_BAD; },
+      [&](size_t row, int r, double c, double s) {
+        uint32_t pl[FX_S];
+        fx_phase_digits(c, s, pl);
+        uint32_t *o = reinterpret_cast<uint32_t *>(d + row * kpad) + r;
 #pragma unroll
-      for (int i = 0; i < FX_S; i++) o[i * (plane / 2)] = pl[i];
-    }
-  }
+        for (int i = 0; i < FX_S; i++) o[i * (plane / 2)] = pl[i];
+      });
 }
 
 // Exponent of a row from the largest |x|'s high word: |x| < 2^e; FX_BAD when not finite.

@@ -297,6 +297,45 @@ __device__ __forceinline__ float fermi_diff_scaled(float a, float b, float ia, f
   return num * ia * ib;
 }
 
+// A_ij += sum_r P[r nq] B[r rs + i nw + j] (r ascending) for MW <= 4, by a block of 128 threads with
+// the same B: tiles of 16 r go through shared memory, the next tile on its way in registers while
+// this one is used.  (Reading B with uniform global loads left the two warps of a scheduler waiting
+// on L1 half of the time.)
+template <typename R, int MW>
+__device__ __forceinline__ void contract_tiles(cx<R> (&A)[MW][MW], const cx<R> *__restrict__ P, size_t nq,
+                                               const cx<R> *__restrict__ B, size_t rs, int nR, int nw, cx<R> *sm) {
+  constexpr int TR = 16, E = MW * MW, PER = (TR * E + 127) / 128;
+  cx<R> nx[PER];
+  auto fetch = [&](int r0) {
+#pragma unroll
+    for (int t = 0; t < PER; t++) {
+      const int e = threadIdx.x + 128 * t, rr = e / E, i = (e % E) / MW, j = e % MW;
+      nx[t] = (rr < TR && r0 + rr < nR && i < nw && j < nw) ? B[(size_t)(r0 + rr) * rs + i * nw + j] : mkc<R>(0, 0);
+    }
+  };
+  fetch(0);
+  int buf = 0;
+  for (int r0 = 0; r0 < nR; r0 += TR, buf ^= 1) {
+    // (this buffer's readers of two tiles ago passed the barrier of the tile between)
+#pragma unroll
+    for (int t = 0; t < PER; t++)
+      if (threadIdx.x + 128 * t < TR * E) sm[buf * TR * E + threadIdx.x + 128 * t] = nx[t];
+    __syncthreads();
+    if (r0 + TR < nR) fetch(r0 + TR);
+    const int nr = min(TR, nR - r0);
+#pragma unroll 4
+    for (int rr = 0; rr < nr; rr++) {
+      const cx<R> p = P[(size_t)(r0 + rr) * nq];
+      const cx<R> *b = sm + (buf * TR + rr) * E;
+#pragma unroll
+      for (int i = 0; i < MW; i++)
+#pragma unroll
+        for (int j = 0; j < MW; j++) cfma(A[i][j], p, b[i * MW + j]);
+    }
+  }
+  __syncthreads();
+}
+
 // The vertex of one pair (k, q) (kl = k - a.k0; qq a valid q):
 //   H(k+q)   = sum_Re P_q(Re) BH_k(Re)  (or the staged contraction)  -> Jacobi -> e_m (ascending), U
 //   X_a      = sum_Rp P_q(Rp) Bg_k(Rp, a)   (= g_a(k,q) U_k)
@@ -314,11 +353,14 @@ __device__ __forceinline__ bool pair_vertex(const PairArgs &a, int kl, int k, in
   const cx<R> *Bg = (const cx<R> *)a.Bg + (size_t)k * a.nRp * nm * nw2;
   const cx<R> *ET = (const cx<R> *)a.ET;
   cx<R> A[MW][MW];
+  __shared__ cx<R> btile[(!FROMC && MW <= 4) ? 2 * 16 * MW * MW : 1];
 #pragma unroll UW
   for (int i = 0; i < MW; i++)
 #pragma unroll UW
     for (int j = 0; j < MW; j++) A[i][j] = mkc<R>(0, 0);
-  if constexpr (FROMC) {
+  if constexpr (!FROMC && MW <= 4) {
+    contract_tiles<R, MW>(A, PqTe + qq, nq, BH, nw2, a.nRe, nw, btile);
+  } else if constexpr (FROMC) {
     // Hermitian part of the staged H(k+q)
     const float *C = a.Cq + (size_t)kl * a.cpk * a.ldc + qq;
 #pragma unroll UW
@@ -376,7 +418,9 @@ __device__ __forceinline__ bool pair_vertex(const PairArgs &a, int kl, int k, in
     for (int i = 0; i < MW; i++)
 #pragma unroll UW
       for (int j = 0; j < MW; j++) X[i][j] = mkc<R>(0, 0);
-    if constexpr (FROMC) {
+    if constexpr (!FROMC && MW <= 4) {
+      contract_tiles<R, MW>(X, PqTp + qq, nq, Bg + (size_t)al * nw2, (size_t)nm * nw2, a.nRp, nw, btile);
+    } else if constexpr (FROMC) {
       const float *C = a.Cq + ((size_t)kl * a.cpk + 2 * (size_t)nw2 * (1 + al)) * a.ldc + qq;
 #pragma unroll UW
       for (int i = 0; i < MW; i++)
@@ -687,35 +731,48 @@ __global__ void __launch_bounds__(128) k_pair_ph(PairArgs a) {
   o[2 * nm] = sz;
 }
 
-// Sum of the per-chunk partials in chunk order; Pi'' = 2 pi sum_p, lambda = sum_l / (N(E_F) w)
-// for kept modes (0 otherwise), zeta = sum_z.  dos: N(E_F) on the device.
-__global__ void k_ph_finalize(int nq, int nm, int nchunk, const double *__restrict__ partial,
-                              const double *__restrict__ omegaT, double omega_min, const double *__restrict__ dos,
-                              double *pi_im, double *lam, double *zeta) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nq) return;
-  const int st = 2 * nm + 1;
-  for (int j = 0; j < st; j++) {
-    double s = 0.0, c = 0.0;  // Neumaier over chunks
-    for (int ch = 0; ch < nchunk; ch++) {
-      const double x = partial[((size_t)ch * nq + q) * st + j];
-      const double t = s + x;
-      c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
-      s = t;
-    }
-    s += c;
-    if (j < nm) {
-      const double w = omegaT[(size_t)j * nq + q];
-      const bool keep = w >= omega_min && w > 0.0;
-      if (pi_im) pi_im[(size_t)q * nm + j] = keep ? 2.0 * EPW_PI * s : 0.0;
-    } else if (j < 2 * nm) {
-      const int v = j - nm;
-      const double w = omegaT[(size_t)v * nq + q];
-      const bool keep = w >= omega_min && w > 0.0 && dos[0] > 0.0;
-      if (lam) lam[(size_t)q * nm + v] = keep ? s / (dos[0] * w) : 0.0;
-    } else if (zeta) {
-      zeta[q] = s;
-    }
+__device__ __forceinline__ void neumaier_add(double &s, double &c, double x) {
+  const double u = s + x;
+  c += fabs(s) >= fabs(x) ? (s - u) + x : (x - u) + s;
+  s = u;
+}
+// The 32 lanes' (sum, compensation) pairs into lane 0's, by a fixed tree.
+__device__ __forceinline__ void neumaier_tree(double &s, double &c) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double s2 = __shfl_down_sync(0xffffffffu, s, o), c2 = __shfl_down_sync(0xffffffffu, c, o);
+    neumaier_add(s, c, s2);
+    c += c2;
+  }
+}
+
+// Sum of the per-chunk partials (compensated, fixed order); Pi'' = 2 pi sum_p, lambda = sum_l /
+// (N(E_F) w) for kept modes (0 otherwise), zeta = sum_z.  dos: N(E_F) on the device.  One warp per
+// (q, output): a thread per q left 216 q x 7 sums of 297 chunks to two blocks (613 us).
+__global__ void __launch_bounds__(128) k_ph_finalize(int nq, int nm, int nchunk, const double *__restrict__ partial,
+                                                     const double *__restrict__ omegaT, double omega_min,
+                                                     const double *__restrict__ dos, double *pi_im, double *lam,
+                                                     double *zeta) {
+  const int st = 2 * nm + 1, lane = threadIdx.x & 31;
+  const size_t w_ = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5;
+  if (w_ >= (size_t)nq * st) return;
+  const int q = (int)(w_ / st), j = (int)(w_ % st);
+  double s = 0.0, c = 0.0;
+  for (int ch = lane; ch < nchunk; ch += 32) neumaier_add(s, c, partial[((size_t)ch * nq + q) * st + j]);
+  neumaier_tree(s, c);
+  if (lane != 0) return;
+  s += c;
+  if (j < nm) {
+    const double w = omegaT[(size_t)j * nq + q];
+    const bool keep = w >= omega_min && w > 0.0;
+    if (pi_im) pi_im[(size_t)q * nm + j] = keep ? 2.0 * EPW_PI * s : 0.0;
+  } else if (j < 2 * nm) {
+    const int v = j - nm;
+    const double w = omegaT[(size_t)v * nq + q];
+    const bool keep = w >= omega_min && w > 0.0 && dos[0] > 0.0;
+    if (lam) lam[(size_t)q * nm + v] = keep ? s / (dos[0] * w) : 0.0;
+  } else if (zeta) {
+    zeta[q] = s;
   }
 }
 
@@ -730,13 +787,31 @@ __global__ void k_dos_terms(int nk, int nw, const double *__restrict__ epsk, con
   terms[k] = (wk ? wk[k] : 1.0 / nk) * s;
 }
 
+// Sums of NV (a power of two <= 16) values per lane over the warp: on return v[0] of lane l is the
+// sum of value l / (32 / NV).
+template <typename R, int NV>
+__device__ __forceinline__ void warp_sums(R (&v)[NV], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int h = NV / 2; h > 0; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int t = 0; t < h; t++) {
+      const R give = up ? v[t] : v[t + h], keep = up ? v[t + h] : v[t];
+      v[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+}
+
 // Complex self-energy of Eq. (elselfenergy) on a frequency grid (omega from E_F, i delta
 // broadening): one thread per (k, q) pair, a block holds 128 consecutive q of one k.  For
 // each band n and grid point i (the grid, then omega = 0 for the shift of Eq. (realpartselfenergy)),
 // the thread sums over (m, nu), each warp sums its 32 q (shuffles), and lane 0 writes
 //   out[(kl * nqw + q / 32) * nw + n][i]   (complex, re/im),  nqw = ceil(nq / 32).
 template <typename R, int MW, int MM, bool FROMC>
-__global__ void __launch_bounds__(128) k_pair_se(PairArgs a, int nom, const double *__restrict__ omega,
+__global__ void __launch_bounds__(128, sizeof(R) == 4 && MW <= 4 ? 3 : 1) k_pair_se(PairArgs a, int nom, const double *__restrict__ omega,
                                                  double delta, double2 *out) {
   constexpr int UW = MW <= 4 ? MW : 1;
   constexpr int UM = MM <= 4 ? MM : 1;
@@ -799,62 +874,84 @@ __global__ void __launch_bounds__(128) k_pair_se(PairArgs a, int nom, const doub
         }
       }
     }
-#pragma unroll UW
-    for (int n = 0; n < MW; n++) {
-      if (n >= nw) continue;
-      // warp sum in the working precision (FP32 forms: 32 terms, a few ulp; the FP64
-      // pipe is a small fraction of FP32 here), then FP64 for the cross-warp sum
-      R dr = sr[n], di = -dl * si[n];
+    // warp sums in the working precision (FP32 forms: 32 terms, a few ulp; the FP64 pipe is a small
+    // fraction of FP32 here), then FP64 for the cross-warp sum.  The 2 MW sums share one butterfly:
+    // at each step a lane keeps half of its values and gives away the other half, so 32 lanes x 2 MW
+    // values take 2 MW + log2(32 / (2 MW)) - 1 shuffles instead of 5 x 2 MW; every sum adds the same
+    // pairs of lanes (l, l + 16), then (l, l + 8), ... as a plain tree.
+    R v[2 * MW];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        dr += __shfl_down_sync(0xffffffffu, dr, o);
-        di += __shfl_down_sync(0xffffffffu, di, o);
-      }
-      if (lane == 0 && q - lane < nq)
-        out[(((size_t)kl * nqw + (q >> 5)) * nw + n) * (nom + 1) + i] = make_double2((double)dr, (double)di);
+    for (int n = 0; n < MW; n++) {
+      v[2 * n] = sr[n];
+      v[2 * n + 1] = -dl * si[n];
     }
+    warp_sums<R, 2 * MW>(v, lane);
+    // the sum of value j is in the lanes whose top bits are j
+    constexpr int LPV = 32 / (2 * MW);
+    const int j = lane / LPV;
+    const R mine = v[0], other = __shfl_down_sync(0xffffffffu, mine, LPV);
+    if (lane % (2 * LPV) == 0 && (j >> 1) < nw && q - lane < nq)
+      out[(((size_t)kl * nqw + (q >> 5)) * nw + (j >> 1)) * (nom + 1) + i] = make_double2((double)mine, (double)other);
   }
 }
 
-// Sum over the per-warp partials (fixed order, compensated) into Sigma_nk(omega_i) and, with
-// spec, the spectral function of Eq. (spectral_funct) (Sigma'' = -Im Sigma, real part shifted
-// by its value at omega = 0): one block per (k, n), one thread per grid point (the q-warp rows
-// of a (k, n) are read along omega, contiguously), then the spectral function from the sums.
-__global__ void k_se_finalize(int nkc, int k0, int nw, int nqw, int nom, const double2 *__restrict__ part,
-                              const double *__restrict__ omega, const double *__restrict__ epsk, double EF,
-                              double2 *sig, double *spec) {
-  __shared__ double re0s;
+// Sum over the per-warp partials (fixed order, compensated) into Sigma_nk(omega_i) (the extra point
+// omega = 0 into re0): a block takes 64 grid points of one (k, n), its four warp pairs a quarter of
+// the q-warps each.  Eight partials are added plainly, the groups compensated: the additions are FP64
+// instructions of 64 cycles, and one thread per point over all of them took 234 us for 21 k x 4 bands
+// x 202 points x 250 partials.
+__global__ void __launch_bounds__(256) k_se_finalize(int k0, int nw, int nqw, int nom,
+                                                     const double2 *__restrict__ part, double2 *sig, double *re0) {
+  __shared__ double sh[4][4][64];
   const int kl = blockIdx.x / nw, n = blockIdx.x % nw, k = k0 + kl;
+  const int x = threadIdx.x & 63, y = threadIdx.x >> 6, i = blockIdx.y * 64 + x;
   const size_t stride = (size_t)nw * (nom + 1);
   const double2 *base = part + ((size_t)kl * nqw * nw + n) * (nom + 1);
-  for (int i = threadIdx.x; i <= nom; i += blockDim.x) {
-    double sr = 0.0, cr = 0.0, si = 0.0, ci = 0.0;
-    for (int j = 0; j < nqw; j++) {
-      const double2 x = base[(size_t)j * stride + i];
-      double u = sr + x.x;
-      cr += fabs(sr) >= fabs(x.x) ? (sr - u) + x.x : (x.x - u) + sr;
-      sr = u;
-      u = si + x.y;
-      ci += fabs(si) >= fabs(x.y) ? (si - u) + x.y : (x.y - u) + si;
-      si = u;
+  const int per = (nqw + 3) / 4, j1 = min(nqw, (y + 1) * per);
+  double sr = 0.0, cr = 0.0, si = 0.0, ci = 0.0;
+  if (i <= nom)
+    for (int j = y * per; j < j1; j += 8) {
+      double2 g = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int t = 0; t < 8; t++)
+        if (j + t < j1) {
+          const double2 v = base[(size_t)(j + t) * stride + i];
+          g.x += v.x;
+          g.y += v.y;
+        }
+      neumaier_add(sr, cr, g.x);
+      neumaier_add(si, ci, g.y);
     }
-    const double2 t = make_double2(sr + cr, si + ci);
-    if (i < nom)
-      sig[((size_t)k * nw + n) * nom + i] = t;
-    else
-      re0s = t.x;
-  }
+  sh[y][0][x] = sr;
+  sh[y][1][x] = cr;
+  sh[y][2][x] = si;
+  sh[y][3][x] = ci;
   __syncthreads();
-  if (!spec) return;
-  const double re0 = re0s;
-  const double e = epsk[(size_t)k * nw + n] - EF;
-  for (int i = threadIdx.x; i < nom; i += blockDim.x) {
-    const size_t o = ((size_t)k * nw + n) * nom + i;
-    const double2 t = sig[o];
-    const double s2 = -t.y;
-    const double den = omega[i] - e - (t.x - re0);
-    spec[o] = fabs(s2) / (EPW_PI * (den * den + s2 * s2));
+  if (y != 0 || i > nom) return;
+  for (int t = 1; t < 4; t++) {
+    neumaier_add(sr, cr, sh[t][0][x]);
+    cr += sh[t][1][x];
+    neumaier_add(si, ci, sh[t][2][x]);
+    ci += sh[t][3][x];
   }
+  if (i < nom)
+    sig[((size_t)k * nw + n) * nom + i] = make_double2(sr + cr, si + ci);
+  else
+    re0[blockIdx.x] = sr + cr;
+}
+
+// The spectral function from the sums (re0: Re Sigma at omega = 0 of each (k, n) of the chunk).
+__global__ void k_spectral(size_t total, int k0, int nw, int nom, const double2 *__restrict__ sig,
+                           const double *__restrict__ re0, const double *__restrict__ omega,
+                           const double *__restrict__ epsk, double EF, double *spec) {
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (t >= total) return;
+  const int i = (int)(t % nom);
+  const size_t kn = t / nom, o = ((size_t)k0 * nw + kn) * nom + i;
+  const double2 v = sig[o];
+  const double s2 = -v.y, e = epsk[(size_t)k0 * nw + kn] - EF;
+  const double den = omega[i] - e - (v.x - re0[kn]);
+  spec[o] = fabs(s2) / (EPW_PI * (den * den + s2 * s2));
 }
 
 // C_nu(q) = pref sum_{kappa,a} E[kappa a][nu] F_{kappa a}(q), F = sum_{G, q+G != 0} damp(q+G)
@@ -945,12 +1042,6 @@ __global__ void k_set_vertex(int nRe, int nRp, size_t per, const void *__restric
   }
 }
 
-__device__ __forceinline__ void neumaier_add(double &s, double &c, double x) {
-  const double u = s + x;
-  c += fabs(s) >= fabs(x) ? (s - u) + x : (x - u) + s;
-  s = u;
-}
-
 // out[k][n] = pi * sum_qb partial[k][qb][n], compensated (Neumaier).  One warp
 // per (k, n): lane l sums qb = l, l+32, ... in order, then the 32 partial sums
 // are combined by a fixed shuffle tree, so the result does not depend on timing.
@@ -1013,29 +1104,36 @@ __global__ void __launch_bounds__(128) k_finalize_k(int nk, int nqb, int nw, con
   }
 }
 
-// out[0] (+)= scale * sum_i partial[i], one block, fixed order, compensated.
-__global__ void k_sum_scalar(int n, const double *__restrict__ partial, double scale, double *out) {
-  __shared__ double ss[256], cc[256];
+// out[0] += scale * sum_i partial[i], one block, fixed order, compensated: each thread a stride of
+// the terms, then the pairs (sum, compensation) by a shuffle tree and one warp over the warps' (a
+// single thread over 256 pairs took 65 us of dependent FP64 additions).
+__global__ void __launch_bounds__(256) k_sum_scalar(int n, const double *__restrict__ partial, double scale,
+                                                    double *out) {
+  __shared__ double ss[8], cc[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double s = 0.0, c = 0.0;
-  for (int i = threadIdx.x; i < n; i += 256) {
-    double x = partial[i];
-    double u = s + x;
-    c += fabs(s) >= fabs(x) ? (s - u) + x : (x - u) + s;
-    s = u;
+  for (int i = threadIdx.x; i < n; i += 256) neumaier_add(s, c, partial[i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double s2 = __shfl_down_sync(0xffffffffu, s, o), c2 = __shfl_down_sync(0xffffffffu, c, o);
+    neumaier_add(s, c, s2);
+    c += c2;
   }
-  ss[threadIdx.x] = s;
-  cc[threadIdx.x] = c;
+  if (lane == 0) {
+    ss[warp] = s;
+    cc[warp] = c;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double S = 0.0, C = 0.0;
-    for (int i = 0; i < 256; i++) {
-      double x = ss[i];
-      double u = S + x;
-      C += fabs(S) >= fabs(x) ? (S - u) + x : (x - u) + S;
-      S = u;
-      C += cc[i];
+  if (warp == 0) {
+    s = lane < 8 ? ss[lane] : 0.0;
+    c = lane < 8 ? cc[lane] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      const double s2 = __shfl_down_sync(0xffffffffu, s, o), c2 = __shfl_down_sync(0xffffffffu, c, o);
+      neumaier_add(s, c, s2);
+      c += c2;
     }
-    out[0] += scale * (S + C);
+    if (lane == 0) out[0] += scale * (s + c);
   }
 }
 
@@ -1197,9 +1295,9 @@ template epw_status launch_pair<double>(const PairArgs &, int, cudaStream_t);
 template epw_status launch_pair<float>(const PairArgs &, int, cudaStream_t);
 
 epw_status launch_pair_staged(const PairArgs &a, int mode, cudaStream_t st) {
-  int nkl = (mode == 2) ? a.nkc : a.nk;
+  const int nkl = a.nk;
   if (nkl <= 0 || a.nq <= 0) return EPW_OK;
-  if (!a.Cq) return EPW_ERR_UNSUPPORTED;
+  if (!a.Cq || mode == 2) return EPW_ERR_UNSUPPORTED;  // (the adjoint: launch_adj_staged)
   if (a.nw > 8 || a.nm > 9) {
     // linewidth: only the terms within the Gaussian cutoff (EPW_STAGED_PAIR=dense: every term,
     // cyclic Jacobi per warp)
@@ -1210,10 +1308,8 @@ epw_status launch_pair_staged(const PairArgs &a, int mode, cudaStream_t st) {
   dim3 grid((a.nq + 127) / 128, nkl);
   if (mode == 0)
     k_pair<float, 8, 9, 0, true><<<grid, 128, 0, st>>>(a);
-  else if (mode == 1)
-    k_pair<float, 8, 9, 1, true><<<grid, 128, 0, st>>>(a);
   else
-    k_pair<float, 8, 9, 2, true><<<grid, 128, 0, st>>>(a);
+    k_pair<float, 8, 9, 1, true><<<grid, 128, 0, st>>>(a);
   epw_count_launch();
   return EPW_OK;
 }
@@ -1248,7 +1344,7 @@ template epw_status launch_pair_ph<float>(const PairArgs &, int, cudaStream_t);
 void launch_ph_finalize(int nq, int nm, int nchunk, const double *partial, const double *omegaT, double omega_min,
                         const double *dos, double *pi_im, double *lam, double *zeta, cudaStream_t st) {
   if (nq <= 0) return;
-  k_ph_finalize<<<(nq + 127) / 128, 128, 0, st>>>(nq, nm, nchunk, partial, omegaT, omega_min, dos, pi_im, lam, zeta);
+  k_ph_finalize<<<(unsigned)(((size_t)nq * (2 * nm + 1) + 3) / 4), 128, 0, st>>>(nq, nm, nchunk, partial, omegaT, omega_min, dos, pi_im, lam, zeta);
   epw_count_launch();
 }
 
@@ -1289,11 +1385,14 @@ template epw_status launch_pair_se<double>(const PairArgs &, int, const double *
 template epw_status launch_pair_se<float>(const PairArgs &, int, const double *, double, double2 *, cudaStream_t);
 
 void launch_se_finalize(int nkc, int k0, int nw, int nqw, int nom, const double2 *part, const double *omega,
-                        const double *epsk, double EF, double2 *sig, double *spec, cudaStream_t st) {
+                        const double *epsk, double EF, double2 *sig, double *spec, double *re0, cudaStream_t st) {
   const int n = nkc * nw;
   if (n <= 0) return;
-  const int bs = nom + 1 <= 64 ? 64 : nom + 1 <= 128 ? 128 : 256;
-  k_se_finalize<<<n, bs, 0, st>>>(nkc, k0, nw, nqw, nom, part, omega, epsk, EF, sig, spec);
+  k_se_finalize<<<dim3(n, (nom + 1 + 63) / 64), 256, 0, st>>>(k0, nw, nqw, nom, part, sig, re0);
+  epw_count_launch();
+  if (!spec) return;
+  const size_t total = (size_t)n * nom;
+  k_spectral<<<(unsigned)((total + 127) / 128), 128, 0, st>>>(total, k0, nw, nom, sig, re0, omega, epsk, EF, spec);
   epw_count_launch();
 }
 

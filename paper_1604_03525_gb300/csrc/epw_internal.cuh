@@ -136,10 +136,12 @@ __device__ __forceinline__ float fermi_diff_f(float ea, float eb, double EF, dou
 // Stops when the off-diagonal weight falls below tol2 * total weight; sets
 // *nonconv when maxsweep sweeps were not enough.  On return the diagonal of A
 // holds the eigenvalues (unsorted) and V the eigenvectors (columns).
-template <typename R, int N>
+// UR: unrolling (N: arrays in registers, n a constant).  Loops over pairs run over the full square
+// with a condition: an inner trip count that depends on the outer index is not unrolled by a factor,
+// and the arrays would end up in local memory.
+template <typename R, int N, int UR = (N <= 4 ? N : 1)>
 __device__ __forceinline__ void jacobi_herm(cx<R> (&A)[N][N], cx<R> (&V)[N][N], int n, R tol2, int maxsweep,
                                             bool &nonconv) {
-  constexpr int UR = N <= 4 ? N : 1;
 #pragma unroll UR
   for (int i = 0; i < N; i++)
 #pragma unroll UR
@@ -149,11 +151,12 @@ __device__ __forceinline__ void jacobi_herm(cx<R> (&A)[N][N], cx<R> (&V)[N][N], 
   for (int i = 0; i < N; i++) {
     A[i][i].y = R(0);
 #pragma unroll UR
-    for (int j = i + 1; j < N; j++) {
-      cx<R> a = R(0.5) * (A[i][j] + conjc(A[j][i]));
-      A[i][j] = a;
-      A[j][i] = conjc(a);
-    }
+    for (int j = 0; j < N; j++)
+      if (j > i) {
+        cx<R> a = R(0.5) * (A[i][j] + conjc(A[j][i]));
+        A[i][j] = a;
+        A[j][i] = conjc(a);
+      }
   }
   bool done = false;
   for (int sweep = 0; sweep < maxsweep && !done; sweep++) {
@@ -162,8 +165,8 @@ __device__ __forceinline__ void jacobi_herm(cx<R> (&A)[N][N], cx<R> (&V)[N][N], 
     for (int i = 0; i < N; i++) {
       if (i < n) diag += A[i][i].x * A[i][i].x;
 #pragma unroll UR
-      for (int j = i + 1; j < N; j++)
-        if (j < n) off += cabs2(A[i][j]);
+      for (int j = 0; j < N; j++)
+        if (j > i && j < n) off += cabs2(A[i][j]);
     }
     if (off <= tol2 * (diag + R(2) * off)) {
       done = true;
@@ -172,42 +175,44 @@ __device__ __forceinline__ void jacobi_herm(cx<R> (&A)[N][N], cx<R> (&V)[N][N], 
 #pragma unroll UR
     for (int p = 0; p < N - 1; p++) {
 #pragma unroll UR
-      for (int q = p + 1; q < N; q++) {
-        if (q >= n) continue;
+      for (int q = 1; q < N; q++) {
         cx<R> apq = A[p][q];
         R m2 = cabs2(apq);
-        if (m2 == R(0)) continue;
-        R mag = sqrt(m2);
-        R rinv = R(1) / mag;
-        cx<R> e = mkc(apq.x * rinv, apq.y * rinv);
-        R theta = (A[q][q].x - A[p][p].x) * (R(0.5) * rinv);
-        R t = R(1) / (fabs(theta) + sqrt(fma(theta, theta, R(1))));
-        t = theta < R(0) ? -t : t;
-        R c = R(1) / sqrt(fma(t, t, R(1)));
-        R s = t * c;
-        A[p][p].x -= t * mag;
-        A[q][q].x += t * mag;
-        A[p][q] = mkc(R(0), R(0));
-        A[q][p] = mkc(R(0), R(0));
-        cx<R> se = s * e;          // s e
-        cx<R> sec = s * conjc(e);  // s conj(e)
+        if (q > p && q < n && m2 != R(0)) {
+          R mag = sqrt(m2);
+          R rinv = R(1) / mag;
+          cx<R> e = mkc(apq.x * rinv, apq.y * rinv);
+          R theta = (A[q][q].x - A[p][p].x) * (R(0.5) * rinv);
+          R t = R(1) / (fabs(theta) + sqrt(fma(theta, theta, R(1))));
+          t = theta < R(0) ? -t : t;
+          R c = R(1) / sqrt(fma(t, t, R(1)));
+          R s = t * c;
+          A[p][p].x -= t * mag;
+          A[q][q].x += t * mag;
+          A[p][q] = mkc(R(0), R(0));
+          A[q][p] = mkc(R(0), R(0));
+          cx<R> se = s * e;          // s e
+          cx<R> sec = s * conjc(e);  // s conj(e)
 #pragma unroll UR
-        for (int r = 0; r < N; r++) {
-          if (r == p || r == q || r >= n) continue;
-          cx<R> arp = A[r][p], arq = A[r][q];
-          cx<R> nrp = c * arp - sec * arq;
-          cx<R> nrq = se * arp + c * arq;
-          A[r][p] = nrp;
-          A[p][r] = conjc(nrp);
-          A[r][q] = nrq;
-          A[q][r] = conjc(nrq);
-        }
+          for (int r = 0; r < N; r++) {
+            if (r != p && r != q && r < n) {
+              cx<R> arp = A[r][p], arq = A[r][q];
+              cx<R> nrp = c * arp - sec * arq;
+              cx<R> nrq = se * arp + c * arq;
+              A[r][p] = nrp;
+              A[p][r] = conjc(nrp);
+              A[r][q] = nrq;
+              A[q][r] = conjc(nrq);
+            }
+          }
 #pragma unroll UR
-        for (int r = 0; r < N; r++) {
-          if (r >= n) continue;
-          cx<R> vrp = V[r][p], vrq = V[r][q];
-          V[r][p] = c * vrp - sec * vrq;
-          V[r][q] = se * vrp + c * vrq;
+          for (int r = 0; r < N; r++) {
+            if (r < n) {
+              cx<R> vrp = V[r][p], vrq = V[r][q];
+              V[r][p] = c * vrp - sec * vrq;
+              V[r][q] = se * vrp + c * vrq;
+            }
+          }
         }
       }
     }
@@ -219,25 +224,24 @@ __device__ __forceinline__ void jacobi_herm(cx<R> (&A)[N][N], cx<R> (&V)[N][N], 
     for (int i = 0; i < N; i++) {
       if (i < n) diag += A[i][i].x * A[i][i].x;
 #pragma unroll UR
-      for (int j = i + 1; j < N; j++)
-        if (j < n) off += cabs2(A[i][j]);
+      for (int j = 0; j < N; j++)
+        if (j > i && j < n) off += cabs2(A[i][j]);
     }
     if (!(off <= tol2 * (diag + R(2) * off))) nonconv = true;
   }
 }
 
 // Sort eigenvalues (diagonal of A) ascending into w[], permuting columns of V.
-template <typename R, int N>
+template <typename R, int N, int UR = (N <= 4 ? N : 1)>
 __device__ __forceinline__ void sort_eig(cx<R> (&A)[N][N], cx<R> (&V)[N][N], R (&w)[N], int n) {
-  constexpr int UR = N <= 4 ? N : 1;
 #pragma unroll UR
   for (int i = 0; i < N; i++) w[i] = A[i][i].x;
   // insertion network over the first n entries (compile-time loops)
 #pragma unroll UR
   for (int i = 1; i < N; i++) {
 #pragma unroll UR
-    for (int j = i; j > 0; j--) {
-      if (j < n && w[j] < w[j - 1]) {
+    for (int j = N - 1; j > 0; j--) {
+      if (j <= i && j < n && w[j] < w[j - 1]) {
         R t = w[j];
         w[j] = w[j - 1];
         w[j - 1] = t;
@@ -325,7 +329,7 @@ struct epw_model {
   unsigned char *ev_tag;  // [EPW_MAX_TIMED] tag of each timed launch
   // second stream for the q side of the preparation, and its fork / join events
   cudaStream_t aux;
-  cudaEvent_t ev_fork, ev_join, ev_phase;
+  cudaEvent_t ev_fork, ev_join, ev_phase, ev_gate;
   // third stream: the k-side bands (H(k) and its eigensolve) beside the k-side vertex GEMM
   cudaStream_t aux2;
   cudaEvent_t ev_fork2, ev_join2;
@@ -414,6 +418,9 @@ struct PairArgs {
 // mode: 0 linewidth, 1 interp, 2 backward
 template <typename R>
 epw_status launch_pair(const PairArgs &a, int mode, cudaStream_t st);
+// adjoint per pair on a staged contraction (FP32, nw <= 8, 3nat <= 9): only the terms whose Gaussians
+// do not underflow; a.xbar is [nkc 3nat nw^2][nq] here and zeroed by the caller
+epw_status launch_adj_staged(const PairArgs &a, cudaStream_t st);
 // per-pair kernel on a staged contraction (a.Cq set; FP32)
 epw_status launch_pair_staged(const PairArgs &a, int mode, cudaStream_t st);
 // phonon side (per-(q, nu) sums over k, nw <= 8, 3nat <= 9): grid (q blocks, nchunk), each chunk
@@ -442,7 +449,7 @@ template <typename R>
 epw_status launch_pair_se(const PairArgs &a, int nom, const double *omega, double delta, double2 *out,
                           cudaStream_t st);
 void launch_se_finalize(int nkc, int k0, int nw, int nqw, int nom, const double2 *part, const double *omega,
-                        const double *epsk, double EF, double2 *sig, double *spec, cudaStream_t st);
+                        const double *epsk, double EF, double2 *sig, double *spec, double *re0, cudaStream_t st);
 // warp-per-pair kernel for nw, 3nat up to 18 (modes 0 and 1; a.Cq set: staged
 // contraction in the q-major layout Cq[q*ldc + kl*cpk + 2c + s], FP32 only)
 template <typename R>

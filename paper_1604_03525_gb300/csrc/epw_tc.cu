@@ -36,6 +36,7 @@
 #include <cstring>
 
 #include "epw_eig4.cuh"
+#include "epw_fx.cuh"
 #include "epw_tc.cuh"
 #include "epw_tcgen05.cuh"
 
@@ -1107,6 +1108,40 @@ __global__ void k_a_pad(int nq, int k0, int kpad, T *hi, T *lo) {
     split_store<T>(0.0, hi, lo, (i / w) * kpad + k0 + i % w);
 }
 
+// The A operand and the digit planes of the FP64 contractions (epw_fx.cuh) in one pass over the q
+// phases: no FP64 phase array in between (316,000 q x 249 R: 8.2 ms as phases, planes and operand
+// one after the other).
+template <typename T>
+__global__ void __launch_bounds__(128) k_phases_a(int nq, const double *__restrict__ q, int nR,
+                                                  const int *__restrict__ R, int rmax, int kpad_fx, size_t plane,
+                                                  __nv_bfloat16 *d, short *e, int kpad, T *hi, T *lo) {
+  __shared__ FxFactors F;
+  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  fx_point_phases(
+      nq, q, nR, R, rmax, max(kpad_fx, kpad) / 2, F,
+      [&](size_t row, bool fin) {
+        e[row] = fin ? 0 : FX_BAD;
+        if (!fin) split_store<T>(nan, hi, lo, row * kpad);  // (the point's status is D(q)'s)
+      },
+      [&](size_t row, int r, double c, double s) {
+        if (r < kpad_fx / 2) {
+          uint32_t pl[FX_S];
+          fx_phase_digits(c, s, pl);
+          uint32_t *o = reinterpret_cast<uint32_t *>(d + row * kpad_fx) + r;
+#pragma unroll
+          for (int i = 0; i < FX_S; i++) o[i * (plane / 2)] = pl[i];
+        }
+        if (r < nR) {
+          const size_t o = row * kpad + 2 * (size_t)(nR - 1 - r);
+          split_store<T>(c, hi, lo, o);
+          split_store<T>(s, hi, lo, o + 1);
+        } else if (2 * r < kpad) {
+          split_store<T>(0.0, hi, lo, row * kpad + 2 * r);
+          split_store<T>(0.0, hi, lo, row * kpad + 2 * r + 1);
+        }
+      });
+}
+
 // hi/lo split of an FP32 value, in FP32: v - hi is exact (hi is v rounded to
 // fewer mantissa bits), so this equals split_store of (double)v.
 template <typename T>
@@ -1538,6 +1573,18 @@ void tc_build_a_raw(int op, int nq, int nR, int kpad, const double *q, const int
     build_a<__nv_bfloat16>(nq, nR, kpad, q, R, P64, (__nv_bfloat16 *)hi, (__nv_bfloat16 *)lo, st);
   else
     build_a<float>(nq, nR, kpad, q, R, P64, (float *)hi, (float *)lo, st);
+}
+void tc_phases_a(int op, int nq, const double *q, int nR, const int *R, int rmax, const FxOp &o, int kpad, void *hi,
+                 void *lo, cudaStream_t st) {
+  if (nq <= 0) return;
+  const size_t plane = (size_t)o.rows * o.kpad;
+  const int grid = (nq + FX_PPB - 1) / FX_PPB;
+  if (op == TC_OP_BF16)
+    k_phases_a<__nv_bfloat16><<<grid, 128, 0, st>>>(nq, q, nR, R, rmax, o.kpad, plane, o.d, o.e, kpad,
+                                                    (__nv_bfloat16 *)hi, (__nv_bfloat16 *)lo);
+  else
+    k_phases_a<float><<<grid, 128, 0, st>>>(nq, q, nR, R, rmax, o.kpad, plane, o.d, o.e, kpad, (float *)hi, (float *)lo);
+  epw_count_launch();
 }
 bool tc_make_map(CUtensorMap *map, const void *base, int op, uint64_t inner, uint64_t rows, uint32_t box_rows) {
   return make_map(map, base, op, inner, rows, box_rows);
@@ -2060,33 +2107,21 @@ epw_status tc_bwd_plan(Arena &A, const epw_model *m, int nk, int nq, TcBuffers &
 }
 
 // ------------------------------------------------------ staged adjoint
-// The q contraction of the staged adjoint, Bbar[Rp][kl nc + c] = sum_q conj(P_q(Rp)) Xbar[q][kl][c],
-// as the same split-TF32 GEMM on the tensor cores: Xbar (FP32 complex, q-major, written by the
-// per-pair adjoint kernel) is transposed into K-major rows split into two tf32 terms, K index
-// 2q + (re, im), against the conj-phase operand of the Rp set.
+// The q contraction of the staged adjoint, Bbar[Rp][kl nc + c] = sum_q conj(P_q(Rp)) Xbar[kl nc + c][q],
+// as the same split-TF32 GEMM on the tensor cores: Xbar (FP32 complex rows over q, written by the
+// per-pair adjoint kernel) is split into two tf32 terms, K index 2q + (re, im), against the
+// conj-phase operand of the Rp set.
 
-// xhi/xlo[m][2q + t] (t = re, im) from xbar[q][m], m < nrow: 32 x 32 tiles through shared memory
-__global__ void k_xbar_split(int nq, int nrow, int ld, const float2 *__restrict__ xbar, float *hi, float *lo) {
-  __shared__ float2 tile[32][33];
-  const int tq = (nq + 31) / 32, tm = (nrow + 31) / 32;
-  for (int t = blockIdx.x; t < tq * tm; t += gridDim.x) {
-    const int q0 = (t / tm) * 32, m0 = (t % tm) * 32;
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-      const int q = q0 + i, mm = m0 + threadIdx.x;
-      tile[i][threadIdx.x] = (q < nq && mm < nrow) ? xbar[(size_t)q * nrow + mm] : make_float2(0.0f, 0.0f);
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-      const int mm = m0 + i, q = q0 + threadIdx.x;
-      if (mm < nrow && q < nq) {
-        const float2 v = tile[threadIdx.x][i];
-        const float h0 = tf32_rn(v.x), h1 = tf32_rn(v.y);
-        const size_t o = (size_t)mm * ld + 2 * (size_t)q;
-        *reinterpret_cast<float2 *>(hi + o) = make_float2(h0, h1);
-        *reinterpret_cast<float2 *>(lo + o) = make_float2(tf32_rn(v.x - h0), tf32_rn(v.y - h1));
-      }
-    }
+// xhi/xlo[m][2q + t] (t = re, im) from xbar[m][q]
+__global__ void k_xbar_split(int nq, size_t nrow, int ld, const float2 *__restrict__ xbar, float *hi, float *lo) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= nq) return;
+  for (size_t m = blockIdx.y; m < nrow; m += gridDim.y) {
+    const float2 v = xbar[m * nq + q];
+    const float h0 = tf32_rn(v.x), h1 = tf32_rn(v.y);
+    const size_t o = m * ld + 2 * (size_t)q;
+    *reinterpret_cast<float2 *>(hi + o) = make_float2(h0, h1);
+    *reinterpret_cast<float2 *>(lo + o) = make_float2(tf32_rn(v.x - h0), tf32_rn(v.y - h1));
   }
 }
 
@@ -2124,11 +2159,9 @@ epw_status tc_sbwd_contract(const epw_model *m, int kc, int nq, const cx<float> 
                             cx<float> *Bbar, cudaStream_t st) {
   if (kc > w.kc) return EPW_ERR_UNSUPPORTED;
   const int nc = w.nc, M = kc * nc;
-  {
-    const int tiles = ((nq + 31) / 32) * ((M + 31) / 32);
-    k_xbar_split<<<std::min(tiles, 152 * 16), dim3(32, 8), 0, st>>>(nq, M, w.ld, (const float2 *)xbar, w.xhi, w.xlo);
-    epw_count_launch();
-  }
+  k_xbar_split<<<dim3((nq + 255) / 256, std::min(M, 32768)), 256, 0, st>>>(nq, M, w.ld, (const float2 *)xbar, w.xhi,
+                                                                          w.xlo);
+  epw_count_launch();
   CUtensorMap xh, xl, ph, pl;
   if (!make_map_f32(&xh, w.xhi, 2 * (uint64_t)nq, w.ld, (uint64_t)M, 128) ||
       !make_map_f32(&xl, w.xlo, 2 * (uint64_t)nq, w.ld, (uint64_t)M, 128) ||
@@ -2325,6 +2358,7 @@ epw_status tc_staged_plan(Arena &A, const epw_model *m, int nk, int nq, int op, 
 
 epw_status tc_staged_phases(const epw_model *m, int nq, const double *q, TcStaged &s, cudaStream_t st) {
   if (!s.ok) return EPW_ERR_UNSUPPORTED;
+  if (s.a_done) return EPW_OK;  // built with the digit planes
   if (s.op == TC_OP_BF16)
     build_a<__nv_bfloat16>(nq, m->nRe, s.kpad, q, m->Re, s.Pq64, (__nv_bfloat16 *)s.Ahi, (__nv_bfloat16 *)s.Alo, st,
                            m->nRp, m->Rp, s.kg0);

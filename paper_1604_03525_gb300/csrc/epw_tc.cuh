@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda.h>
 
+#include "epw_fx.cuh"
 #include "epw_internal.cuh"
 
 // Operand split of the tensor-core contraction.
@@ -63,6 +64,9 @@ void tc_build_b_raw(int op, int nk, int nk_pad, int nR, int nw, int nm, int cpk,
                     const cx<float> *Bg, void *hi, void *lo, cudaStream_t st);
 void tc_build_a_raw(int op, int nq, int nR, int kpad, const double *q, const int *R, const cx<double> *P64, void *hi,
                     void *lo, cudaStream_t st);
+// A [nq][kpad] and the phases' digit planes o in one pass.
+void tc_phases_a(int op, int nq, const double *q, int nR, const int *R, int rmax, const FxOp &o, int kpad, void *hi,
+                 void *lo, cudaStream_t st);
 // 2D K-major map [rows][inner], box [box_rows][128 bytes], 128-byte swizzle.
 bool tc_make_map(CUtensorMap *map, const void *base, int op, uint64_t inner, uint64_t rows, uint32_t box_rows);
 // The same with rows of row_bytes (128: 128-byte swizzle; 64: 64-byte swizzle).
@@ -92,6 +96,7 @@ struct TcwBuffers {
   int op, kpad, kpadG, kc, ldq, nqt, cpk, kpt, entp, cn, bng;
   bool ok;
   bool fused;          // one kernel (E and G overlapped, eigen-data through a ring in L2); else two per chunk
+  bool a_done;         // the Re operand is built already (with the digit planes of D(q))
   bool pair;           // the fused kernel on CTA pairs (cta_group::2 MMAs over 256 q rows)
 };
 // forms of the wide path: the fused kernel on CTA pairs (default), the two-kernel form, the
@@ -128,7 +133,7 @@ struct TcBwdBuffers {
 // Lay out the adjoint's buffers (forward operands at TF32 included).
 epw_status tc_bwd_plan(Arena &A, const epw_model *m, int nk, int nq, TcBuffers &b, TcBwdBuffers &w);
 // Staged adjoint's q contraction on the tensor cores (TF32 split), chunks of up to kc k:
-// Bbar[Rp][kl][c] = sum_q conj(P_q(Rp)) xbar[q][kl][c] (xbar FP32 complex [nq][kc][nc]).
+// Bbar[Rp][kl][c] = sum_q conj(P_q(Rp)) xbar[kl][c][q] (xbar FP32 complex [kc][nc][nq]).
 epw_status tc_sbwd_plan(Arena &A, const epw_model *m, int nq, int kc, TcBwdBuffers &w);
 epw_status tc_sbwd_phases(const epw_model *m, int nq, const double *q, TcBwdBuffers &w, cudaStream_t st);
 epw_status tc_sbwd_contract(const epw_model *m, int kc, int nq, const cx<float> *xbar, TcBwdBuffers &w,
@@ -153,6 +158,7 @@ struct TcStaged {
   int op, kpad, cpk, kc, mtiles, ldc;
   int kg0;          // K offset of the vertex's Rp phases when Rp differs from Re (0: one shared set)
   bool ok;
+  bool a_done;      // A is built already (with the digit planes of D(q))
   bool qmajor;      // layout read by the warp-per-pair kernel (nw > 8 or 3nat > 9)
   size_t ldn;
   const cx<double> *Pq64;  // FP64 q phases of the Re set [nR][nq] when already formed (else null)

@@ -1296,7 +1296,7 @@ epw_status tcw_linewidth(const epw_model *m, int nk, int nq, const double *q, co
   if (!b.ok) return EPW_ERR_UNSUPPORTED;
   const int nw = m->nw, nm = m->nm, nR = m->nRe, nRp = m->nRp, op = b.op;
   const int esz = op == TC_OP_BF16 ? 2 : 4;
-  tc_build_a_raw(op, nq, nR, b.kpad, q, m->Re, P64, b.Ahi, b.Alo, st);
+  if (!b.a_done) tc_build_a_raw(op, nq, nR, b.kpad, q, m->Re, P64, b.Ahi, b.Alo, st);
   if (!m->same_ep) tc_build_a_raw(op, nq, nRp, b.kpadG, q, m->Rp, nullptr, b.AGhi, b.AGlo, st);
   tc_tables(nq, nm, nk, nw, omegaT, par->T_K, wq, epsk, b.nbT, b.omF, b.wqF, b.ekF, st);
   const float cut = (float)(CUT_SIGMAS * par->sigma_eV);
