@@ -76,8 +76,8 @@ static epw_status upload(T **dst, const T *src, size_t n) {
 }
 
 static void free_model_arrays(epw_model *m) {
-  void *ptrs[] = {m->Re, m->Rp, m->Rph, m->wRe, m->wRp, m->Hw, m->Phiw, m->Phidf, m->gw, m->mass, m->dstatus, m->ws,
-                  m->pZ};
+  void *ptrs[] = {m->Re, m->Rp, m->Rph, m->wRe, m->wRp, m->Hw, m->Phiw, m->Phidf, m->gw, m->mass, m->exptab, m->dstatus,
+                  m->ws, m->pZ};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   if (m->aux) cudaStreamDestroy(m->aux);
@@ -160,6 +160,9 @@ extern "C" epw_status epw_load_wannier(const epw_wannier_desc *d, epw_model **ou
       }
     }
 
+  std::vector<double> exptab(EPW_EXPTAB);
+  for (int j = 0; j < EPW_EXPTAB; j++) exptab[j] = std::exp2(-(double)j / EPW_EXPTAB);
+
   epw_model *m = (epw_model *)calloc(1, sizeof(epw_model));
   if (!m) return fail(EPW_ERR_OOM, "host allocation failed");
   m->device = dev;
@@ -185,7 +188,8 @@ extern "C" epw_status epw_load_wannier(const epw_wannier_desc *d, epw_model **ou
       (s = upload(&m->Hw, Hw.data(), Hw.size())) != EPW_OK || (s = upload(&m->Phiw, Phiw.data(), Phiw.size())) != EPW_OK ||
       (s = upload(&m->Phidf, Phidf.data(), Phidf.size())) != EPW_OK ||
       (s = upload(&m->gw, gw.data(), gw.size())) != EPW_OK ||
-      (s = upload(&m->mass, d->mass, (size_t)nat)) != EPW_OK) {
+      (s = upload(&m->mass, d->mass, (size_t)nat)) != EPW_OK ||
+      (s = upload(&m->exptab, exptab.data(), exptab.size())) != EPW_OK) {
     free_model_arrays(m);
     free(m);
     return s;
@@ -521,22 +525,30 @@ static epw_status run_vertex64(const epw_model *m, int nk, const double *k, cons
   return EPW_OK;
 }
 
-// H(k+q) and g(k,q) U_k of the k-points [k0, k0 + kc) into f.CH, f.CG.
-// (hmat: H(k+q) as FP64 into f.Hq [nq][kc][nw^2] instead; vertex: whether g(k,q) U_k is wanted)
-static epw_status run_fx_contract(const epw_model *m, int k0, int kc, const Prep &p, Fx64 &f, cudaStream_t st,
-                                  bool hmat = false, bool vertex = true) {
-  const int nw2 = m->nw * m->nw, ncol = m->nm * nw2;
-  FxOp bh = f.BH, bg = f.BG;  // a last, shorter chunk has fewer rows (and tighter planes)
-  bh.rows = kc * nw2;
-  bg.rows = kc * 2 * ncol;
+// H(k+q) of the k-points [k0, k0 + kc): as fixed point into f.CH, or as FP64 into f.Hq [nq][kc][nw^2].
+static FxOp fx_bh(const epw_model *m, int k0, int kc, const Prep &p, Fx64 &f, cudaStream_t st) {
+  FxOp bh = f.BH;  // a last, shorter chunk has fewer rows (and tighter planes)
+  bh.rows = kc * m->nw * m->nw;
   fx_hermitian(kc, m->nRe, m->nw, p.PkRM + (size_t)k0 * m->nRe, m->Hw, bh, f.bad, st);
-  if (hmat)
-    CKS(fx_gemm_f64(f.Ae, bh, fx_bits(m->nRe), f.Hq, (size_t)kc * nw2, m->dstatus, st));
-  else
-    CKS(fx_gemm_i64(f.Ae, bh, fx_bits(m->nRe), f.CH, f.ldc, m->dstatus, st));
-  if (!vertex) return EPW_OK;
+  return bh;
+}
+static epw_status run_fx_hmat(const epw_model *m, int k0, int kc, const Prep &p, Fx64 &f, cudaStream_t st) {
+  const FxOp bh = fx_bh(m, k0, kc, p, f, st);
+  return fx_gemm_f64(f.Ae, bh, fx_bits(m->nRe), f.Hq, (size_t)kc * m->nw * m->nw, m->dstatus, st);
+}
+// g(k,q) U_k into f.CG.
+static epw_status run_fx_vertex(const epw_model *m, int k0, int kc, const Prep &p, Fx64 &f, cudaStream_t st) {
+  const int ncol = m->nm * m->nw * m->nw;
+  FxOp bg = f.BG;
+  bg.rows = kc * 2 * ncol;
   fx_columns(kc, m->nRp, ncol, ncol, (const cx<double> *)p.Bg + (size_t)k0 * m->nRp * ncol, bg, f.bad, st);
   return fx_gemm_i64(f.Ap, bg, fx_bits(m->nRp), f.CG, f.ldc, m->dstatus, st);
+}
+// Both of a chunk.
+static epw_status run_fx_contract(const epw_model *m, int k0, int kc, const Prep &p, Fx64 &f, cudaStream_t st) {
+  const FxOp bh = fx_bh(m, k0, kc, p, f, st);
+  CKS(fx_gemm_i64(f.Ae, bh, fx_bits(m->nRe), f.CH, f.ldc, m->dstatus, st));
+  return run_fx_vertex(m, k0, kc, p, f, st);
 }
 
 static Pair64Args pair64_args(const epw_model *m, int k0, int kc, int nq, const double *wq, const epw_params *par,
@@ -570,6 +582,7 @@ static Pair64Args pair64_args(const epw_model *m, int k0, int kc, int nq, const 
   a.inv_nq = 1.0 / nq;
   a.dstatus = m->dstatus;
   a.bad = f.bad;
+  a.exptab = m->exptab;
   a.Cpol = m->polar ? (const double2 *)p.Cpol : nullptr;
   a.Uk = p.Uk;
   return a;
@@ -695,11 +708,26 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
       tcb->prebuilt_a = true;
     }
   }
+  if (fx && fx->pair && fx->omK)
+    launch_tables64(nq, nm, p.omegaT, omega_min, fx->T, fx->omK, fx->nbT, fx->wmax, sq);
   if (fork) {
     CK(cudaEventRecord(m->ev_join, sq));
-    CK(cudaStreamWaitEvent(st, m->ev_join, 0));
+    if (fx) fx->late = fx->late && gate;
+    if (fx && fx->late)
+      CK(cudaStreamWaitEvent(st, m->ev_gate, 0));  // the q phases' operands; the phonons follow
+    else
+      CK(cudaStreamWaitEvent(st, m->ev_join, 0));
+  } else if (fx) {
+    fx->late = false;
   }
   CK(cudaGetLastError());
+  return EPW_OK;
+}
+// With fx.late: joins the q side's phonons into st (contractions that read only its operands have
+// run beside its eigensolves).
+static epw_status prep_join(const epw_model *m, Fx64 &fx, cudaStream_t st) {
+  if (fx.late) CK(cudaStreamWaitEvent(st, m->ev_join, 0));
+  fx.late = false;
   return EPW_OK;
 }
 
@@ -978,6 +1006,7 @@ static epw_status linewidth_pass(epw_model *m, int nk, const double *kd, int nq,
   } else if (tcp) {
     // staged tensor-core form: contraction per chunk of k on the tensor cores, per-pair work from HBM
     const PhaseA pa = staged_a(m, L.sg);
+    L.fx.late = true;
     CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &L.fx, &pa));
     L.sg.Pq64 = m->same_eph ? p.PqTph : nullptr;
     CKS(tc_staged_phases(m, nq, qd, L.sg, st));
@@ -986,6 +1015,7 @@ static epw_status linewidth_pass(epw_model *m, int nk, const double *kd, int nq,
       const int kc = std::min(L.sg.kc, nk - k0);
       epw_status s = tc_staged_contract(m, k0, kc, nq, (const cx<float> *)p.Bg, (const cx<float> *)p.BH, L.sg, st);
       if (s != EPW_OK) return fail(s, "staged tensor-core contraction failed");
+      CKS(prep_join(m, L.fx, st));
       PairArgs a;
       std::memset(&a, 0, sizeof(a));
       a.nk = kc;
@@ -1017,12 +1047,14 @@ static epw_status linewidth_pass(epw_model *m, int nk, const double *kd, int nq,
     launch_finalize(nk, (nq + 127) / 128, m->nw, L.partial, out, st);
   } else if (L.fx.pair) {
     // FP64: the contractions of a chunk of k as digit planes on the tensor cores, per-pair work in FP64
+    L.fx.T = par->T_K;
+    L.fx.late = true;
     CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &L.fx));
-    launch_tables64(nq, m->nm, p.omegaT, par->omega_min_eV, par->T_K, L.fx.omK, L.fx.nbT, L.fx.wmax, st);
     epw_timing_begin(m, st);
     for (int k0 = 0; k0 < nk; k0 += L.fx.kc) {
       const int kc = std::min(L.fx.kc, nk - k0);
       CKS(run_fx_contract(m, k0, kc, p, L.fx, st));
+      CKS(prep_join(m, L.fx, st));
       Pair64Args a = pair64_args(m, k0, kc, nq, wqd, par, p, L.fx);
       a.partial = L.partial;
       epw_status s = launch_lw64(a, st);
@@ -1100,6 +1132,7 @@ extern "C" epw_status epw_interp_g(const epw_model *mc, int nk, const double *k,
             precision == EPW_FP64 && want_pairs && fx_pair(m, nk, nq), precision == EPW_FP64 && nk > 0 && g && fx_g1(m, nk), fx, per);
     if (fx.pair) {
       const size_t np = (size_t)nq * fx.kc;
+      fx.omK = nullptr;  // (no tables: no occupations here)
       fx.Hq = A.take<double>(np * nw * nw);
       Hq = A.take<cx<double>>(np * nw * nw);
       Uq = A.take<cx<double>>(np * nw * nw);
@@ -1132,6 +1165,7 @@ extern "C" epw_status epw_interp_g(const epw_model *mc, int nk, const double *k,
     CK(cudaMemcpyAsync(p.qd, q, sizeof(double) * 3 * nq, cudaMemcpyHostToDevice, st));
     qd = p.qd;
   }
+  fx.late = fx.pair;
   CKS(run_prep(m, nk, kd, nq, qd, wprec, omega_min, need_B, p, omd, st, true, tc ? &tcb : nullptr, &fx));
   if (ekd && nk > 0) CK(cudaMemcpyAsync(ekd, p.epsk, sizeof(double) * nk * nw, cudaMemcpyDeviceToDevice, st));
   if (tc && nk > 0 && nq > 0 && (ekqd || gd)) {
@@ -1177,9 +1211,11 @@ extern "C" epw_status epw_interp_g(const epw_model *mc, int nk, const double *k,
     // FP64: H(k+q) as matrices, the batched Jacobi (the eigenvectors' phases are its), then g
     for (int k0 = 0; k0 < nk; k0 += fx.kc) {
       const int kc = std::min(fx.kc, nk - k0);
-      CKS(run_fx_contract(m, k0, kc, p, fx, st, true, gd != nullptr));
+      CKS(run_fx_hmat(m, k0, kc, p, fx, st));
       fx_unpack_hermitian(nq * kc, m->nw, fx.Hq, Hq, st);
       launch_eigh_d(nq * kc, m->nw, Hq, wkq, Uq, m->dstatus, st);
+      if (gd) CKS(run_fx_vertex(m, k0, kc, p, fx, st));
+      CKS(prep_join(m, fx, st));
       epw_params par{0.0, 0.0, 1.0, omega_min, precision, 0};
       Pair64Args a = pair64_args(m, k0, kc, nq, nullptr, &par, p, fx);
       a.wkq = wkq;
@@ -1341,13 +1377,15 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
   CK(cudaMemsetAsync(b.sc, 0, 2 * sizeof(double), st));
   if (!pair64) CK(cudaMemsetAsync(b.gwbar, 0, sR * ng, st));
   if (pair64) {
+    b.fx.T = par->T_K;
+    b.fx.late = true;
     CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx));
-    launch_tables64(nq, m->nm, p.omegaT, par->omega_min_eV, par->T_K, b.fx.omK, b.fx.nbT, b.fx.wmax, st);
     if (b.dgd) fx_phases_conj(nq, qd, m->nRp, m->Rp, b.Pq, st);
     const int splits = fx_splits(b.Xq.kpad);
     for (int k0 = 0; k0 < nk; k0 += b.fx.kc) {
       const int kc = std::min(b.fx.kc, nk - k0);
       CKS(run_fx_contract(m, k0, kc, p, b.fx, st));
+      CKS(prep_join(m, b.fx, st));
       CK(cudaMemsetAsync(b.xb64, 0, sizeof(cx<double>) * kc * per * nq, st));
       Pair64Args a = pair64_args(m, k0, kc, nq, wqd, par, p, b.fx);
       a.cot = b.cotd;
@@ -1384,6 +1422,7 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
     if (s != EPW_OK) return fail(s, "tensor-core adjoint failed");
   } else if (nk > 0 && nq > 0) {
     const PhaseA pa = staged_a(m, b.sg);
+    b.fx.late = staged;
     CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx,
                  staged ? &pa : nullptr));
     b.sg.Pq64 = m->same_eph ? p.PqTph : nullptr;
@@ -1396,6 +1435,7 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
       if (staged) {
         epw_status s = tc_staged_contract(m, k0, kc, nq, (const cx<float> *)p.Bg, (const cx<float> *)p.BH, b.sg, st);
         if (s != EPW_OK) return fail(s, "staged tensor-core contraction failed");
+        CKS(prep_join(m, b.fx, st));
       }
       PairArgs a;
       std::memset(&a, 0, sizeof(a));
@@ -1502,7 +1542,9 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
   // chunks of k per q block: enough blocks to fill the GPU a few times over
   const int nqb = (std::max(nq, 1) + 127) / 128;
   const int want = std::max(1, (4 * 152 + nqb - 1) / nqb);
-  const int kper = std::max(1, (std::max(nk, 1) + want - 1) / want);
+  int kper = std::max(1, (std::max(nk, 1) + want - 1) / want);
+  // (FP64 in fixed point: warps of 32 q x kper k, about eight waves of two per sub-partition)
+  const int kper64 = (int)std::max<long>(1, (long)std::max(nk, 1) * ((std::max(nq, 1) + 31) / 32) / 9728);
   struct B {
     Prep p;
     Fx64 fx;
@@ -1519,6 +1561,7 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
     b.sg = TcStaged{};
     int nchunk = (std::max(nk, 1) + kper - 1) / kper;
     if (b.fx.pair) {
+      kper = kper64;
       nchunk = 0;
       for (int k0 = 0; k0 < nk; k0 += b.fx.kc) nchunk += (std::min(b.fx.kc, nk - k0) + kper - 1) / kper;
     }
@@ -1568,6 +1611,8 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
   }
   if (nk > 0 && nq > 0) {
     const PhaseA pa = staged_a(m, b.sg);
+    b.fx.T = par->T_K;
+    b.fx.late = b.fx.pair;
     CKS(run_prep(m, nk, kd, nq, qd, wprec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx,
                  tcp ? &pa : nullptr));
   } else if (nk > 0) {
@@ -1581,11 +1626,11 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
     launch_sum_scalar(nk, b.terms, 1.0, b.dosd, st);
   }
   if (nk > 0 && nq > 0 && b.fx.pair) {
-    launch_tables64(nq, nm, p.omegaT, par->omega_min_eV, par->T_K, b.fx.omK, b.fx.nbT, b.fx.wmax, st);
     int chunk0 = 0;
     for (int k0 = 0; k0 < nk; k0 += b.fx.kc) {
       const int kc = std::min(b.fx.kc, nk - k0), nch = (kc + kper - 1) / kper;
       CKS(run_fx_contract(m, k0, kc, p, b.fx, st));
+      CKS(prep_join(m, b.fx, st));
       Pair64Args a = pair64_args(m, k0, kc, nq, nullptr, par, p, b.fx);
       a.wk = wkd;
       a.nk_total = nk;

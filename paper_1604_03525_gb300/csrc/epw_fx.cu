@@ -408,56 +408,77 @@ __global__ void k_fx_phases_conj(int npt, const double *__restrict__ x, int nR, 
   }
 }
 
-// One warp per row (element h of the n^2 of one k), lanes over R.
+struct FxRows {
+  double x, y, z, w;
+};
+// One warp per element (i, j), i <= j, of one k: its one or two rows (real part h(i,j), imaginary part
+// h(j,i)), lanes over R.  The products P(r) X_r stay in registers between the search for the largest
+// and the digits when nR <= 256 (beyond, the rest is formed twice): they are most of the work.
 __global__ void __launch_bounds__(128) k_fx_hermitian(int nk, int nR, int n, const double2 *__restrict__ p,
                                                       const double2 *__restrict__ X, int kpad, size_t plane,
                                                       __nv_bfloat16 *d, short *e, int *bad) {
-  const int lane = threadIdx.x & 31;
-  const size_t row = (size_t)blockIdx.x * 4 + (threadIdx.x >> 5);
-  if (row >= (size_t)nk * n * n) return;
-  const int k = (int)(row / (n * n)), h = (int)(row % (n * n));
-  const bool im = h / n > h % n;  // (j, i), j > i: the imaginary part of element (i, j)
-  const int i = min(h / n, h % n), j = max(h / n, h % n);
-  auto value = [&](int r, double &c, double &s) {  // coefficients of (cos, sin)
+  constexpr int NV = 8;
+  const int lane = threadIdx.x & 31, ne = n * (n + 1) / 2;
+  const size_t w = (size_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (w >= (size_t)nk * ne) return;
+  const int k = (int)(w / ne);
+  int i = 0, j = (int)(w % ne);
+  while (j >= n - i) j -= n - i++;
+  j += i;
+  // coefficients of (cos, sin): v.x, v.y of the real part's row, v.z, v.w of the imaginary part's
+  auto value = [&](int r) {
     double2 a = X[(size_t)r * n * n + i * n + j], b = X[(size_t)r * n * n + j * n + i];
     if (p) {
       const double2 f = p[(size_t)k * nR + r];
       a = make_double2(f.x * a.x - f.y * a.y, f.x * a.y + f.y * a.x);
       b = make_double2(f.x * b.x - f.y * b.y, f.x * b.y + f.y * b.x);
     }
-    if (i == j) {
-      c = a.x;
-      s = -a.y;
-    } else if (!im) {
-      c = 0.5 * (a.x + b.x);
-      s = -0.5 * (a.y + b.y);
-    } else {
-      c = 0.5 * (a.y - b.y);
-      s = 0.5 * (a.x - b.x);
-    }
+    FxRows v;
+    v.x = i == j ? a.x : 0.5 * (a.x + b.x);
+    v.y = i == j ? -a.y : -0.5 * (a.y + b.y);
+    v.z = 0.5 * (a.y - b.y);
+    v.w = 0.5 * (a.x - b.x);
+    return v;
   };
-  unsigned m = 0;
-  for (int r = lane; r < nR; r += 32) {
-    double c, s;
-    value(r, c, s);
-    m = max(m, absmax_hi(c, s));
-  }
-  m = __reduce_max_sync(0xffffffffu, m);
-  const int ex = fx_exponent(m);
-  if (lane == 0) {
-    e[row] = (short)ex;
-    if (ex == FX_BAD && bad) atomicOr(bad, 1);
-  }
-  const double sc = ex == FX_BAD ? 0.0 : pow2d(55 - ex);
-  uint32_t *o = reinterpret_cast<uint32_t *>(d + row * kpad);
-  for (int r = lane; r < kpad / 2; r += 32) {
-    double c = 0.0, s = 0.0;
-    if (r < nR && ex != FX_BAD) value(r, c, s);
-    uint32_t a[FX_S];
-    fx_digits2(__double2ll_rn(c * sc), __double2ll_rn(s * sc), a);
+  FxRows c[NV];
+  unsigned m0 = 0, m1 = 0;
 #pragma unroll
-    for (int z = 0; z < FX_S; z++) o[z * (plane / 2) + r] = a[z];
+  for (int t = 0; t < NV; t++) {
+    c[t] = FxRows{0.0, 0.0, 0.0, 0.0};
+    const int r = lane + 32 * t;
+    if (r < nR) c[t] = value(r);
+    m0 = max(m0, absmax_hi(c[t].x, c[t].y));
+    m1 = max(m1, absmax_hi(c[t].z, c[t].w));
   }
+  for (int r = lane + 32 * NV; r < nR; r += 32) {
+    const FxRows v = value(r);
+    m0 = max(m0, absmax_hi(v.x, v.y));
+    m1 = max(m1, absmax_hi(v.z, v.w));
+  }
+  const int e0 = fx_exponent(__reduce_max_sync(0xffffffffu, m0)), e1 = fx_exponent(__reduce_max_sync(0xffffffffu, m1));
+  const size_t r0 = (size_t)k * n * n + i * n + j, r1 = (size_t)k * n * n + j * n + i;
+  if (lane == 0) {
+    e[r0] = (short)e0;
+    if (i != j) e[r1] = (short)e1;
+    if ((e0 == FX_BAD || e1 == FX_BAD) && bad) atomicOr(bad, 1);
+  }
+  const double s0 = e0 == FX_BAD ? 0.0 : pow2d(55 - e0), s1 = e1 == FX_BAD ? 0.0 : pow2d(55 - e1);
+  auto put = [&](int r, const FxRows &v) {
+    uint32_t a[FX_S];
+    uint32_t *o = reinterpret_cast<uint32_t *>(d + r0 * kpad) + r;
+    fx_digits2(e0 == FX_BAD ? 0 : __double2ll_rn(v.x * s0), e0 == FX_BAD ? 0 : __double2ll_rn(v.y * s0), a);
+#pragma unroll
+    for (int z = 0; z < FX_S; z++) o[z * (plane / 2)] = a[z];
+    if (i == j) return;
+    o = reinterpret_cast<uint32_t *>(d + r1 * kpad) + r;
+    fx_digits2(e1 == FX_BAD ? 0 : __double2ll_rn(v.z * s1), e1 == FX_BAD ? 0 : __double2ll_rn(v.w * s1), a);
+#pragma unroll
+    for (int z = 0; z < FX_S; z++) o[z * (plane / 2)] = a[z];
+  };
+#pragma unroll
+  for (int t = 0; t < NV; t++)
+    if (lane + 32 * t < kpad / 2) put(lane + 32 * t, c[t]);
+  for (int r = lane + 32 * NV; r < kpad / 2; r += 32) put(r, r < nR ? value(r) : FxRows{0.0, 0.0, 0.0, 0.0});
 }
 
 __global__ void k_fx_scales(size_t n, const short *__restrict__ e, int F, double *scale) {
@@ -567,7 +588,7 @@ void fx_phases_conj(int npt, const double *x, int nR, const int *R, const FxOp &
 
 void fx_hermitian(int nk, int nR, int n, const cx<double> *p, const cx<double> *X, const FxOp &o, int *bad,
                   cudaStream_t st) {
-  const size_t rows = (size_t)nk * n * n;
+  const size_t rows = (size_t)nk * (n * (n + 1) / 2);
   if (!rows) return;
   k_fx_hermitian<<<(unsigned)((rows + 3) / 4), 128, 0, st>>>(nk, nR, n, (const double2 *)p, (const double2 *)X, o.kpad,
                                                             (size_t)o.rows * o.kpad, o.d, o.e, bad);

@@ -56,6 +56,8 @@ struct Fx64 {
   double *omK, *nbT;     // frequencies (-1: left out) and Bose factors [nm][nq]
   double *wmax;          // [nq]
   int *bad;              // an operand held an infinity or a NaN
+  double T;              // temperature of the tables (set by the caller)
+  bool late;             // the caller joins the q side itself (prep_join), after work that needs only its planes
   int kc;
   size_t ldc;
   double *Hq;            // interpolation: H(k+q) of one chunk [nq][kc][nw^2] (fx_hermitian's rows)

@@ -319,6 +319,7 @@ struct epw_model {
   float4 *Phidf;          // Phiw in double-float: (Re hi, Re lo, Im hi, Im lo) per entry
   cx<double> *gw;         // [nRe][nRp][nm][nw][nw], wRe wRp folded
   double *mass;           // [nat]
+  double *exptab;         // [EPW_EXPTAB] 2^(-j/EPW_EXPTAB), for the FP64 per-pair kernels
   unsigned int *dstatus;  // device status word
   void *ws;               // workspace arena
   size_t ws_bytes;
@@ -343,6 +344,7 @@ struct epw_model {
 };
 
 #define EPW_MAX_TIMED 4096
+#define EPW_EXPTAB 512
 
 // Record the start / stop event of a timed launch (no-op unless timing is on).
 void epw_timing_begin(epw_model *m, cudaStream_t st);

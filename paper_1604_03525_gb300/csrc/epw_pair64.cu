@@ -23,6 +23,23 @@ __device__ __forceinline__ double fx_value(long long I, int e, int F) {
   return e == FX_BAD ? __longlong_as_double(0x7ff8000000000000LL) : (I == 0 ? 0.0 : v);
 }
 
+// exp(-z) for z >= 0, table-driven (Tang, ACM Trans. Math. Softw. 15, 144 (1989)): z = n ln2/512 + r,
+// exp(-z) = 2^(-n div 512) T[n mod 512] (1 + p(r)), |r| <= ln2/1024, p the Taylor polynomial of
+// exp(-r) - 1 to r^4 (the next term is 1e-18).  Nine FP64 instructions; CUDA's exp takes 16 or 17.
+// Below 2^-1020 the result is 0.
+__device__ __forceinline__ double exp64n(const double *__restrict__ tab, double z) {
+  const double magic = 6755399441055744.0;  // 1.5 2^52: the sum's low bits are the rounded integer
+  const double t = fma(z, 738.6598609351493, magic);                        // 512 / ln 2
+  const int n = __double2loint(t);
+  const double nf = t - magic;
+  double r = fma(nf, -0.001353803086658445, z);                           // ln 2 / 512: 32 bits and the rest
+  r = fma(nf, -3.7269822837316166e-13, r);
+  const double p = r * fma(r, fma(r, fma(r, 1.0 / 24.0, -1.0 / 6.0), 0.5), -1.0);
+  const double T = tab[n & (EPW_EXPTAB - 1)], v = fma(T, p, T);
+  const double s = __hiloint2double(__double2hiint(v) - ((n >> 9) << 20), __double2loint(v));
+  return z <= 707.0 ? s : (z != z ? z : 0.0);
+}
+
 __device__ __forceinline__ double wsum64(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -307,21 +324,21 @@ __device__ __forceinline__ bool pair64_eig(const Pair64Args &a, int kl, int q, E
 
 constexpr int P64_MM = 18;  // modes
 
-// What a warp shares while it works through the terms of its 32 pairs: each lane's current
-// eigenvector (component i of lane l at u[i][l]), eigenvalue and occupation, and the list of
-// (lane, n) terms.
-template <int W>
+// What a warp shares while it works through the terms of its 32 pairs: eigenvectors (component i of
+// lane l's at u[s][i][l]), eigenvalues and occupations of MS bands per lane (all of them, or the
+// current one), and the list of terms: lane, slot s, band n.
+template <int W, int MS, bool OCC = true>
 struct P64Warp {
-  double2 u[W][32];
-  double em[32], f[32];
-  unsigned short list[32 * W];
+  double2 u[MS][W][32];
+  double em[MS][32], f[OCC ? MS : 1][32];
+  unsigned short list[32 * W * MS];
 };
 
 // f(e) with one exponential and one reciprocal for either sign of e - E_F
 __device__ __forceinline__ double fermi64(const Pair64Args &a, double e) {
   const double d = e - a.EF;
   if (!(a.T > 0.0)) return d < 0.0 ? 1.0 : (d > 0.0 ? 0.0 : 0.5);
-  const double t = exp(-fabs(d) * a.inv_kT), r = 1.0 / (1.0 + t);
+  const double t = exp64n(a.exptab, fabs(d) * a.inv_kT), r = 1.0 / (1.0 + t);
   return __double2hiint(d) < 0 ? r : t * r;
 }
 
@@ -334,7 +351,7 @@ __device__ __forceinline__ bool p64_reach(float ek, float em, float thr) {
 // g_mn,nu of one term (pair (kl, q), band n = nb, eigenvector u[.][sl]):
 // t_a = u^dagger X_a[:, n], g_nu = sum_a E[a][nu] t_a (plus i C_nu u^dagger U_k[:, n])
 template <int W, bool EX, int MM>
-__device__ __forceinline__ void pair64_g(const Pair64Args &a, int kl, int q, int nb, const double2 (&u)[W][32], int sl,
+__device__ __forceinline__ void pair64_g(const Pair64Args &a, int kl, int q, int nb, const double2 (*u)[32], int sl,
                                          double2 (&g)[MM]) {
   const int n = EX ? W : a.nw, nm = EX ? MM : a.nm;
   constexpr int UM = MM <= 9 ? MM : 1;
@@ -384,12 +401,12 @@ __device__ __forceinline__ void pair64_g(const Pair64Args &a, int kl, int q, int
   }
 }
 
-// Walks the reachable terms of a warp's pairs: each lane takes its next band m that some n
-// reaches and forms its eigenvector; the lanes' (lane, n) terms of that step then go through the
-// warp 32 at a time, whichever pair they belong to (on the fcc model a pair has about 5 of 16
-// terms, the busiest lane of a warp twice that).  term(lane of the pair, n) runs for every
-// term, with the pair's eigenvector, eigenvalue and occupation in sw; step(r0, own0, own1) after
-// the terms r0 .. r0 + 31, with the range of this lane's own terms.
+// Walks the reachable terms of a warp's pairs, 32 at a time whichever pair they belong to (on the fcc
+// model a pair has about 5 of 16 terms, the busiest lane of a warp twice that).  MS = 1: each lane
+// takes its next band m that some n reaches and forms its eigenvector, then the lanes' terms of that
+// step go through the warp; MS = W (narrow matrices, whose eigenvectors all fit shared memory): one
+// list of all terms, so that only its last 32 can be short.  term(lane of the pair, slot, n) runs for
+// every term; step(r0, own0, own1) after the terms r0 .. r0 + 31, with this lane's own range.
 // (reach: whether a term (band n = j with FP32 energy ek, e_mk+q = em in FP32) is wanted)
 struct P64Window {
   float thr;
@@ -398,9 +415,10 @@ struct P64Window {
 struct P64NoStep {
   __device__ __forceinline__ void operator()(int, int, int) const {}
 };
-template <int W, bool EX, class R, class F, class G = P64NoStep>
+template <int W, bool EX, bool OCC, int MS, class R, class F, class G = P64NoStep>
 __device__ __forceinline__ void p64_terms(const Pair64Args &a, const Eig64<W, EX> &S, const float *ekf, bool any,
-                                          R reach, P64Warp<W> &sw, F &&term, G step = G{}) {
+                                          R reach, P64Warp<W, MS, OCC> &sw, F &&term,
+                                          G step = G{}) {
   const int lane = threadIdx.x & 31;
   const int n = EX ? W : a.nw;
   unsigned need = 0;
@@ -413,24 +431,23 @@ __device__ __forceinline__ void p64_terms(const Pair64Args &a, const Eig64<W, EX
         if (reach(ekf[j], em)) need |= 1u << m;
     }
   }
-  while (__any_sync(0xffffffffu, need != 0)) {
+  // band m of this lane into slot s; its terms as a mask
+  auto band = [&](int m, int s) {
+    const double em = S.eigenvalue(m);
+    const float emf = (float)em;
     unsigned todo = 0;
-    if (need) {
-      const int m = __ffs(need) - 1;
-      need &= need - 1;
-      const double em = S.eigenvalue(m);
-      const float emf = (float)em;
-      for (int j = 0; j < n; j++)
-        if (reach(ekf[j], emf)) todo |= 1u << j;
-      double2 u[W];
-      S.vector(n, m, u);
+    for (int j = 0; j < n; j++)
+      if (reach(ekf[j], emf)) todo |= 1u << j;
+    double2 u[W];
+    S.vector(n, m, u);
 #pragma unroll(W <= 9 ? W : 1)
-      for (int i = 0; i < W; i++)
-        if (i < n) sw.u[i][lane] = u[i];
-      sw.em[lane] = em;
-      sw.f[lane] = fermi64(a, em);
-    }
-    const int cnt = __popc(todo);
+    for (int i = 0; i < W; i++)
+      if (i < n) sw.u[s][i][lane] = u[i];
+    sw.em[s][lane] = em;
+    if constexpr (OCC) sw.f[s][lane] = fermi64(a, em);
+    return todo;
+  };
+  auto run = [&](int cnt, auto &&fill) {
     int off = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -439,18 +456,61 @@ __device__ __forceinline__ void p64_terms(const Pair64Args &a, const Eig64<W, EX
     }
     const int total = __shfl_sync(0xffffffffu, off, 31);
     off -= cnt;
-    const int own0 = off;  // this lane's terms: own0 .. own0 + cnt
-    while (todo) {
-      sw.list[off++] = (unsigned short)((lane << 8) | (__ffs(todo) - 1));
-      todo &= todo - 1;
-    }
+    fill(off);  // this lane's terms: off .. off + cnt
     __syncwarp();
     for (int r0 = 0; r0 < total; r0 += 32) {
       const int j = r0 + lane;
-      if (j < total) term(sw.list[j] >> 8, sw.list[j] & 255);
-      step(r0, own0, own0 + cnt);
+      if (j < total) {
+        const unsigned e = sw.list[j];
+        term((int)(e >> 10), (int)((e >> 5) & 31), (int)(e & 31));
+      }
+      step(r0, off, off + cnt);
     }
     __syncwarp();
+  };
+  if constexpr (MS > 1) {
+    static_assert(MS == W, "a slot per band");
+    unsigned todo[W];
+    int cnt = 0, left = need;
+    // (the lanes' bands in step, so that the eigenvectors are formed together)
+#pragma unroll
+    for (int t = 0; t < W; t++) todo[t] = 0;
+#pragma unroll 1
+    for (int t = 0; __any_sync(0xffffffffu, left != 0); t++) {
+      if (left) {
+        const int m = __ffs(left) - 1;
+        left &= left - 1;
+        const unsigned d = band(m, t);
+#pragma unroll
+        for (int c = 0; c < W; c++) todo[c] |= c == t ? d : 0u;
+        cnt += __popc(d);
+      }
+    }
+    run(cnt, [&](int off) {
+#pragma unroll
+      for (int t = 0; t < W; t++) {
+        unsigned d = todo[t];
+        while (d) {
+          sw.list[off++] = (unsigned short)((lane << 10) | (t << 5) | (__ffs(d) - 1));
+          d &= d - 1;
+        }
+      }
+    });
+  } else {
+    while (__any_sync(0xffffffffu, need != 0)) {
+      unsigned todo = 0;
+      if (need) {
+        const int m = __ffs(need) - 1;
+        need &= need - 1;
+        todo = band(m, 0);
+      }
+      run(__popc(todo), [&](int off) {
+        while (todo) {
+          sw.list[off++] = (unsigned short)((lane << 10) | (__ffs(todo) - 1));
+          todo &= todo - 1;
+        }
+      });
+    }
   }
 }
 
@@ -458,7 +518,8 @@ template <int W, bool EX, int MM>
 __global__ void __launch_bounds__(128, 2) k_lw64(Pair64Args a) {
   __shared__ double sh[4][W];
   __shared__ float ekf[W];
-  __shared__ P64Warp<W> sws[4];
+  constexpr int MS = W <= 4 ? W : 1;
+  __shared__ P64Warp<W, MS> sws[4];
   const int qi = blockIdx.x * 128 + threadIdx.x, kl = blockIdx.y, k = a.k0 + kl;
   const bool valid = qi < a.nq;
   const int q = valid ? qi : 0;  // lanes past the last q keep step with their warp
@@ -476,13 +537,13 @@ __global__ void __launch_bounds__(128, 2) k_lw64(Pair64Args a) {
   double acc[W];
 #pragma unroll(W <= P64_REGW ? W : 1)
   for (int j = 0; j < W; j++) acc[j] = 0.0;
-  P64Warp<W> &sw = sws[warp];
+  P64Warp<W, MS> &sw = sws[warp];
   const int qw = qi - lane;
-  p64_terms<W, EX>(a, S, ekf, thr >= 0.0, P64Window{__double2float_ru(thr)}, sw, [&](int sl, int nb) {
+  p64_terms<W, EX, true, MS>(a, S, ekf, thr >= 0.0, P64Window{__double2float_ru(thr)}, sw, [&](int sl, int ms, int nb) {
     const int qs = qw + sl;
     double2 g[MM];
-    pair64_g<W, EX, MM>(a, kl, qs, nb, sw.u, sl, g);
-    const double x = ek[nb] - sw.em[sl], f = sw.f[sl];
+    pair64_g<W, EX, MM>(a, kl, qs, nb, sw.u[ms], sl, g);
+    const double x = ek[nb] - sw.em[ms][sl], f = sw.f[ms][sl];
     double s = 0.0;
 #pragma unroll(MM <= 9 ? MM : 1)
     for (int v = 0; v < MM; v++) {
@@ -491,7 +552,8 @@ __global__ void __launch_bounds__(128, 2) k_lw64(Pair64Args a) {
       if (__double2hiint(w) < 0) continue;
       const double nbv = a.nbT[(size_t)v * a.nq + qs];
       const double yp = (x + w) * a.inv_sigma, ym = (x - w) * a.inv_sigma;
-      const double t = (nbv + f) * exp(-yp * yp) + (nbv + 1.0 - f) * exp(-ym * ym);
+      const double t =
+          fma(nbv + f, exp64n(a.exptab, yp * yp), (nbv + 1.0 - f) * exp64n(a.exptab, ym * ym));
       s = fma(fma(g[v].x, g[v].x, g[v].y * g[v].y), t, s);
     }
     s *= a.wq ? a.wq[qs] : a.inv_nq;
@@ -519,7 +581,7 @@ __global__ void __launch_bounds__(128, 2) k_lw64(Pair64Args a) {
 // dp and dm the two Gaussians with their norm
 __device__ __forceinline__ double gauss_diff64(const Pair64Args &a, double x, double w, double dp, double dm) {
   const double p = x * a.inv_sigma, b = w * a.inv_sigma, y = 2.0 * p * b;
-  return fabs(y) > 1.0 ? dp - dm : -2.0 * a.gnorm * exp(-fma(p, p, b * b)) * sinh(y);
+  return fabs(y) > 1.0 ? dp - dm : -2.0 * a.gnorm * exp64n(a.exptab, fma(p, p, b * b)) * sinh(y);
 }
 
 // Adjoint of L = sum c_nk Im Sigma_nk per pair.  With W_nu,mn = c_nk pi w_q [(n+f) d+ + (n+1-f) d-]:
@@ -530,7 +592,8 @@ template <int W, bool EX, int MM>
 __global__ void __launch_bounds__(128, 2) k_adj64(Pair64Args a) {
   __shared__ double sh[2][4];
   __shared__ float ekf[W];
-  __shared__ P64Warp<W> sws[4];
+  constexpr int MS = 1;  // (a barrier between the terms of a pair's bands m: they add to the same Xbar)
+  __shared__ P64Warp<W, MS> sws[4];
   const int qi = blockIdx.x * 128 + threadIdx.x, kl = blockIdx.y, k = a.k0 + kl;
   const bool valid = qi < a.nq;
   const int q = valid ? qi : 0;
@@ -545,15 +608,15 @@ __global__ void __launch_bounds__(128, 2) k_adj64(Pair64Args a) {
   const double wm = a.wmax[q];
   double thr = valid && __double2hiint(wm) >= 0 ? wm + P64_CUT * a.sigma : -1.0;
   if (thr >= 0.0 && *a.bad) thr = __longlong_as_double(0x7ff0000000000000LL);
-  P64Warp<W> &sw = sws[warp];
+  P64Warp<W, MS> &sw = sws[warp];
   const int qw = qi - lane;
   double sT = 0.0, sE = 0.0;
   double2 *xb = a.xbar + (size_t)kl * nm * n * n * a.nq;
-  p64_terms<W, EX>(a, S, ekf, thr >= 0.0, P64Window{__double2float_ru(thr)}, sw, [&](int sl, int nb) {
+  p64_terms<W, EX, true, MS>(a, S, ekf, thr >= 0.0, P64Window{__double2float_ru(thr)}, sw, [&](int sl, int ms, int nb) {
     const int qs = qw + sl;
     double2 g[MM];
-    pair64_g<W, EX, MM>(a, kl, qs, nb, sw.u, sl, g);
-    const double em = sw.em[sl], f = sw.f[sl], x = ek[nb] - em;
+    pair64_g<W, EX, MM>(a, kl, qs, nb, sw.u[ms], sl, g);
+    const double em = sw.em[ms][sl], f = sw.f[ms][sl], x = ek[nb] - em;
     const double c = cot[nb] * EPW_PI * (a.wq ? a.wq[qs] : a.inv_nq);
     const double ff = fermi_ff_d(em - a.EF, a.T);
     const double dfE = ff * a.inv_kT, dfT = dfE * (em - a.EF) / a.T;
@@ -568,7 +631,7 @@ __global__ void __launch_bounds__(128, 2) k_adj64(Pair64Args a) {
       }
       const double nbv = a.nbT[(size_t)v * a.nq + qs];
       const double yp = (x + w) * a.inv_sigma, ym = (x - w) * a.inv_sigma;
-      const double dp = a.gnorm * exp(-yp * yp), dm = a.gnorm * exp(-ym * ym);
+      const double dp = a.gnorm * exp64n(a.exptab, yp * yp), dm = a.gnorm * exp64n(a.exptab, ym * ym);
       const double g2 = fma(g[v].x, g[v].x, g[v].y * g[v].y);
       const double dn = nbv * (nbv + 1.0) * w * a.inv_kT / a.T;
       const double dd = gauss_diff64(a, x, w, dp, dm);
@@ -594,7 +657,7 @@ __global__ void __launch_bounds__(128, 2) k_adj64(Pair64Args a) {
       for (int i = 0; i < W; i++) {
         if (i >= n) continue;
         double2 *o = xb + (size_t)((al * n + i) * n + nb) * a.nq + qs;
-        const double2 u = sw.u[i][sl];
+        const double2 u = sw.u[ms][i][sl];
         double2 t = *o;
         t.x = fma(u.x, y.x, fma(-u.y, y.y, t.x));
         t.y = fma(u.x, y.y, fma(u.y, y.x, t.y));
@@ -615,38 +678,45 @@ __global__ void __launch_bounds__(128, 2) k_adj64(Pair64Args a) {
   }
 }
 
-// Phonon-side sums (see k_pair_ph): a block's 128 q against a.nkc of the chunk's k-points.  The
-// terms of a q go back to its lane through shared memory, in order.
+// Phonon-side sums (see k_pair_ph): each warp 32 q against a.nkc of the chunk's k-points (few q are
+// the rule here: blocks of 128 q left lanes and sub-partitions idle).  The terms of a q go back to
+// its lane through shared memory, in order.
 template <int W, bool EX, int MM>
 __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
-  __shared__ float ekf[W];
-  __shared__ double dn_s[W], ia_s[W];
-  __shared__ P64Warp<W> sws[4];
+  __shared__ float ekf_s[4][W];
+  __shared__ double dn_w[4][W], ia_w[4][W];
+  constexpr int MS = W <= 4 ? W : 1;
+  __shared__ P64Warp<W, MS, false> sws[4];
   __shared__ double res[4][32][2 * MM];
-  const int qi = blockIdx.x * 128 + threadIdx.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nqw = (a.nq + 31) / 32, w_ = blockIdx.x * 4 + warp, chunk = w_ / nqw, qw = (w_ - chunk * nqw) * 32;
+  const int nchunk = (a.nk + a.nkc - 1) / a.nkc;
+  if (chunk >= nchunk) return;  // the whole warp; only warp-level synchronisation below
+  float *ekf = ekf_s[warp];
+  double *dn_s = dn_w[warp], *ia_s = ia_w[warp];
+  const int qi = qw + lane;
   const bool valid = qi < a.nq;
   const int q = valid ? qi : 0;
   const int n = EX ? W : a.nw, nm = EX ? MM : a.nm;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, qw = qi - lane;
-  P64Warp<W> &sw = sws[warp];
+  P64Warp<W, MS, false> &sw = sws[warp];
   const double wm = a.wmax[q];
   double thr = valid && __double2hiint(wm) >= 0 ? wm + P64_CUT * a.sigma : -1.0;
   if (thr >= 0.0 && *a.bad) thr = __longlong_as_double(0x7ff0000000000000LL);
   double sp[MM], sl_[MM], sz = 0.0;
 #pragma unroll
   for (int v = 0; v < MM; v++) sp[v] = sl_[v] = 0.0;
-  const int kc1 = min(a.nk, (int)(blockIdx.y + 1) * a.nkc);
-  for (int kl = blockIdx.y * a.nkc; kl < kc1; kl++) {
+  const int kc1 = min(a.nk, (chunk + 1) * a.nkc);
+  for (int kl = chunk * a.nkc; kl < kc1; kl++) {
     const int k = a.k0 + kl;
     const double *ek = a.eps_k + (size_t)k * n;
-    __syncthreads();
-    if (threadIdx.x < n) {
-      const double e = ek[threadIdx.x], y = (e - a.EF) * a.inv_sigma;
-      ekf[threadIdx.x] = (float)e;
-      dn_s[threadIdx.x] = a.gnorm * exp(-y * y);
-      ia_s[threadIdx.x] = a.T > 0.0 ? 1.0 / (1.0 + exp(-fabs(e - a.EF) * a.inv_kT)) : 0.0;
+    __syncwarp();
+    if (lane < n) {
+      const double e = ek[lane], y = (e - a.EF) * a.inv_sigma;
+      ekf[lane] = (float)e;
+      dn_s[lane] = a.gnorm * exp64n(a.exptab, y * y);
+      ia_s[lane] = a.T > 0.0 ? 1.0 / (1.0 + exp64n(a.exptab, fabs(e - a.EF) * a.inv_kT)) : 0.0;
     }
-    __syncthreads();
+    __syncwarp();
     Eig64<W, EX> S;
     const bool conv = pair64_eig<W, EX>(a, kl, q, S);
     if (!conv && valid) atomicOr(a.dstatus, EPW_DEV_NOT_CONVERGED);
@@ -659,23 +729,23 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
       for (int m = 0; m < W; m++) {
         if (m >= n) continue;
         const double y = (S.eigenvalue(m) - a.EF) * a.inv_sigma;
-        zm += exp(-y * y);
+        zm += exp64n(a.exptab, y * y);
       }
       sz = fma(wk * zn, a.gnorm * zm, sz);
     }
     // Pi'': |e_nk - e_mk+q - w| within the Gaussian; lambda: both bands within that of E_F
     const float thrf = __double2float_ru(thr), cutf = __double2float_ru(P64_CUT * a.sigma), ef = (float)a.EF;
-    p64_terms<W, EX>(
+    p64_terms<W, EX, false, MS>(
         a, S, ekf, thr >= 0.0,
         [&](float en, float em) {
           return p64_reach(en, em, thrf) || (p64_reach(en, ef, cutf) && p64_reach(em, ef, cutf));
         },
         sw,
-        [&](int sl, int nb) {
+        [&](int sl, int ms, int nb) {
           const int qs = qw + sl;
-          const double em = sw.em[sl], en = ek[nb], x = en - em, dn = dn_s[nb];
+          const double em = sw.em[ms][sl], en = ek[nb], x = en - em, dn = dn_s[nb];
           const double ym = (em - a.EF) * a.inv_sigma;
-          const double z = dn != 0.0 ? dn * a.gnorm * exp(-ym * ym) : 0.0;
+          const double z = dn != 0.0 ? dn * a.gnorm * exp64n(a.exptab, ym * ym) : 0.0;
           double *r = res[warp][lane];
           // the Gaussians of e_nk - e_mk+q - w; with all of them and z zero the term is
           double gs[MM], any = z;
@@ -686,7 +756,7 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
             const double w = a.omK[(size_t)v * a.nq + qs];
             if (__double2hiint(w) < 0) continue;
             const double y = (x - w) * a.inv_sigma;
-            gs[v] = a.gnorm * exp(-y * y);
+            gs[v] = a.gnorm * exp64n(a.exptab, y * y);
             any += gs[v];
           }
           if (any == 0.0 && !*a.bad) {
@@ -699,14 +769,14 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
           if (a.T > 0.0) {
             const double aa = (en - a.EF) * a.inv_kT, bb = (em - a.EF) * a.inv_kT;
             const double d = bb - aa, S2 = fabs(aa) + fabs(bb), ad = fabs(d);
-            const double num = exp(0.5 * (ad - S2)) * expm1(-ad);
-            const double ib = 1.0 / (1.0 + exp(-fabs(bb)));
+            const double num = exp64n(a.exptab, fmax(0.5 * (S2 - ad), 0.0)) * expm1(-ad);
+            const double ib = 1.0 / (1.0 + exp64n(a.exptab, fabs(bb)));
             fd = (d >= 0.0 ? -num : num) * ia_s[nb] * ib;
           } else {
             fd = fermi_d(en, a.EF, a.T) - fermi_d(em, a.EF, a.T);
           }
           double2 g[MM];
-          pair64_g<W, EX, MM>(a, kl, qs, nb, sw.u, sl, g);
+          pair64_g<W, EX, MM>(a, kl, qs, nb, sw.u[ms], sl, g);
 #pragma unroll
           for (int v = 0; v < MM; v++) {
             const bool keep = v < nm && __double2hiint(a.omK[(size_t)(v < nm ? v : 0) * a.nq + qs]) >= 0;
@@ -729,7 +799,7 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
         });
   }
   if (!valid) return;
-  double *o = a.partial + ((size_t)blockIdx.y * a.nq + q) * (2 * nm + 1);
+  double *o = a.partial + ((size_t)chunk * a.nq + q) * (2 * nm + 1);
 #pragma unroll
   for (int v = 0; v < MM; v++)
     if (v < nm) {
@@ -906,7 +976,7 @@ epw_status launch_adj64(const Pair64Args &a, cudaStream_t st) {
 
 epw_status launch_ph64(const Pair64Args &a, int nchunk, cudaStream_t st) {
   if (a.nk <= 0 || a.nq <= 0) return EPW_OK;
-  const dim3 grid((a.nq + 127) / 128, nchunk);
+  const dim3 grid((unsigned)(((size_t)((a.nq + 31) / 32) * nchunk + 3) / 4));
   const int n = a.nw, nm = a.nm;
   if (n > 8 || nm > 9) return EPW_ERR_UNSUPPORTED;
   if (n == 1 && nm == 3)

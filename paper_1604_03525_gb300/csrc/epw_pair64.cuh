@@ -18,6 +18,7 @@ struct Pair64Args {
   double inv_kT, inv_sigma, gnorm, inv_nq;  // 1/kT (T > 0), 1/sigma, 1/(sigma sqrt pi), 1/nq
   double *partial;             // [nk of the call][ceil(nq/128)][nw]
   unsigned *dstatus;
+  const double *exptab;        // 2^(-j/EPW_EXPTAB)
   const int *bad;              // nonzero: some operand held an infinity or a NaN
   const double2 *Cpol;         // long-range factors [nm][nq] or null
   const cx<double> *Uk;        // [nk of the call][nw][nw]
@@ -40,7 +41,7 @@ struct Pair64Args {
 epw_status launch_lw64(const Pair64Args &a, cudaStream_t st);
 // Adjoint of the linewidth per pair: Xbar and the sums for dL/dT, dL/dE_F.
 epw_status launch_adj64(const Pair64Args &a, cudaStream_t st);
-// Sums over the chunk's k per (q, nu): Pi'', lambda and nesting terms (nw <= 8, 3nat <= 9).
+// Sums over the chunk's k per (q, nu): Pi'', lambda and nesting terms (nw <= 8, 3nat <= 9), a.nkc k per warp.
 epw_status launch_ph64(const Pair64Args &a, int nchunk, cudaStream_t st);
 // e_k+q and g_mn,nu from given eigenvectors.
 epw_status launch_g64(const Pair64Args &a, cudaStream_t st);
