@@ -76,7 +76,7 @@ static epw_status upload(T **dst, const T *src, size_t n) {
 }
 
 static void free_model_arrays(epw_model *m) {
-  void *ptrs[] = {m->Re, m->Rp, m->Rph, m->wRe, m->wRp, m->Hw, m->Phiw, m->Phidf, m->gw, m->mass, m->exptab, m->dstatus,
+  void *ptrs[] = {m->Re, m->Rp, m->Rph, m->wRe, m->wRp, m->Hw, m->Phiw, m->Phidf, m->gw, m->gw32, m->mass, m->exptab, m->dstatus,
                   m->ws, m->pZ};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -85,11 +85,12 @@ static void free_model_arrays(epw_model *m) {
   if (m->ev_join) cudaEventDestroy(m->ev_join);
   if (m->ev_phase) cudaEventDestroy(m->ev_phase);
   if (m->ev_gate) cudaEventDestroy(m->ev_gate);
+  if (m->ev_vertex) cudaEventDestroy(m->ev_vertex);
   if (m->aux2) cudaStreamDestroy(m->aux2);
   if (m->ev_fork2) cudaEventDestroy(m->ev_fork2);
   if (m->ev_join2) cudaEventDestroy(m->ev_join2);
   m->aux = m->aux2 = nullptr;
-  m->ev_fork = m->ev_join = m->ev_phase = m->ev_gate = m->ev_fork2 = m->ev_join2 = nullptr;
+  m->ev_fork = m->ev_join = m->ev_phase = m->ev_gate = m->ev_vertex = m->ev_fork2 = m->ev_join2 = nullptr;
   if (m->ev) {
     for (int i = 0; i < 2 * EPW_MAX_TIMED; i++)
       if (m->ev[i]) cudaEventDestroy(m->ev[i]);
@@ -194,12 +195,17 @@ extern "C" epw_status epw_load_wannier(const epw_wannier_desc *d, epw_model **ou
     free(m);
     return s;
   }
-  cudaError_t e = cudaMalloc((void **)&m->dstatus, 16);
+  cudaError_t e = cudaMalloc((void **)&m->gw32, gw.size() * sizeof(cx<float>));
+  if (e == cudaSuccess) {
+    launch_cast_c64_to_c32(gw.size(), m->gw, m->gw32, 0);
+    e = cudaStreamSynchronize(0);
+  }
+  if (e == cudaSuccess) e = cudaMalloc((void **)&m->dstatus, 16);
   if (e == cudaSuccess) e = cudaMemset(m->dstatus, 0, 16);
   if (e != cudaSuccess) {
     free_model_arrays(m);
     free(m);
-    return fail(EPW_ERR_CUDA, "status word: %s", cudaGetErrorString(e));
+    return fail(e == cudaErrorMemoryAllocation ? EPW_ERR_OOM : EPW_ERR_CUDA, "model buffers: %s", cudaGetErrorString(e));
   }
   *out = m;
   return EPW_OK;
@@ -397,14 +403,12 @@ static void plan_prep(Arena &A, const epw_model *m, int nk, int nq, int prec, bo
     p.BH = fx && fx->pair ? nullptr : A.take<char>(sR * (size_t)nk * m->nRe * nw2);
     if (prec != EPW_FP64) {
       p.Pk32 = A.take<cx<float>>((size_t)nk * m->nRe);
-      p.gw32 = A.take<cx<float>>((size_t)m->nRe * m->nRp * m->nm * nw2);
     } else {
       p.Pk32 = nullptr;
-      p.gw32 = nullptr;
     }
   } else {
     p.G1 = p.Bg = p.BH = nullptr;
-    p.Pk32 = p.gw32 = nullptr;
+    p.Pk32 = nullptr;
   }
 }
 
@@ -598,6 +602,7 @@ static epw_status prep_streams(epw_model *m) {
   CK(cudaEventCreateWithFlags(&m->ev_join, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&m->ev_phase, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&m->ev_gate, cudaEventDisableTiming));
+  CK(cudaEventCreateWithFlags(&m->ev_vertex, cudaEventDisableTiming));
   CK(cudaStreamCreateWithFlags(&m->aux2, cudaStreamNonBlocking));
   CK(cudaEventCreateWithFlags(&m->ev_fork2, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&m->ev_join2, cudaEventDisableTiming));
@@ -651,22 +656,29 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   } else if (!qs) {
     launch_fourier_d(nq, m->nRph, p.PqTph, m->Phiw, nm * nm, p.D, sq);
   }
-  // The eigensolves are one long wave of FP64-bound warps: they start on an empty GPU and spread
-  // over every SM, and the k-side vertex (a GEMM that fills the GPU) starts after them.  The other
-  // way round their blocks share the few SMs that happen to have room (13,824 of 9 x 9: 6.6 ms
-  // against 2.4; 1728: 3.3 against 0.8).
+  // The eigensolves are one long wave of FP64-bound warps that has to start on a GPU with room on every
+  // SM: launched while a GEMM fills it, their blocks share the few SMs that happen to have room
+  // (13,824 of 9 x 9: 6.6 ms against 2.4; 1728: 3.3 against 0.8).  So the k-side vertex starts after
+  // them where it runs on the tensor cores (FP64), and they start after it where it runs on the CUDA
+  // cores, which they slow down threefold (FP32: 809 us beside 9001 of 6 x 6, 284 alone).
   const bool gate = fork && fx && fx->dq;
+  const bool after_vertex = gate && need_B && prec != EPW_FP64;
   if (gate) CK(cudaEventRecord(m->ev_gate, sq));
-  launch_eigh_d(nq, nm, p.D, p.w2, p.ev, m->dstatus, sq);
-  launch_phonon_post(nq, nm, p.w2, p.ev, m->mass, omega_min, p.omegaT,
-                     prec == EPW_FP64 ? (cx<double> *)p.ET : nullptr, prec == EPW_FP64 ? nullptr : (cx<float> *)p.ET,
-                     omega_out, sq);
-  if (m->polar) {
-    if (prec == EPW_FP64)
-      launch_polar_factors<double>(m, nq, q, (const cx<double> *)p.ET, (cx<double> *)p.Cpol, sq);
-    else
-      launch_polar_factors<float>(m, nq, q, (const cx<float> *)p.ET, (cx<float> *)p.Cpol, sq);
-  }
+  auto q_tail = [&]() {
+    launch_eigh_d(nq, nm, p.D, p.w2, p.ev, m->dstatus, sq);
+    launch_phonon_post(nq, nm, p.w2, p.ev, m->mass, omega_min, p.omegaT,
+                       prec == EPW_FP64 ? (cx<double> *)p.ET : nullptr,
+                       prec == EPW_FP64 ? nullptr : (cx<float> *)p.ET, omega_out, sq);
+    if (m->polar) {
+      if (prec == EPW_FP64)
+        launch_polar_factors<double>(m, nq, q, (const cx<double> *)p.ET, (cx<double> *)p.Cpol, sq);
+      else
+        launch_polar_factors<float>(m, nq, q, (const cx<float> *)p.ET, (cx<float> *)p.Cpol, sq);
+    }
+    if (fx && fx->pair && fx->omK)
+      launch_tables64(nq, nm, p.omegaT, omega_min, fx->T, fx->omK, fx->nbT, fx->wmax, sq);
+  };
+  if (!after_vertex) q_tail();
   // k side (FP64): phases, H(k), eigensolve, then the k-side vertex; with a fork the
   // bands (H(k), eigensolve) run on a third stream beside the vertex GEMM, which
   // needs only the phases, and are joined before the U_k rotation
@@ -683,7 +695,7 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   if (fork2) CK(cudaEventRecord(m->ev_join2, sk));
   if (need_B && nk > 0) {
     const int ncol = m->nRp * nm * (int)nw2;
-    if (gate) CK(cudaStreamWaitEvent(st, m->ev_gate, 0));
+    if (gate && !after_vertex) CK(cudaStreamWaitEvent(st, m->ev_gate, 0));
     if (prec == EPW_FP64) {
       CKS(run_vertex64(m, nk, k, p, fx, st));
       if (fork2) CK(cudaStreamWaitEvent(st, m->ev_join2, 0));
@@ -691,9 +703,12 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
                              st);
     } else {
       launch_cast_c64_to_c32((size_t)nk * m->nRe, p.PkRM, p.Pk32, st);
-      launch_cast_c64_to_c32((size_t)m->nRe * ncol, m->gw, p.gw32, st);
-      launch_cgemm<float>(nk, ncol, m->nRe, p.Pk32, m->nRe, false, false, p.gw32, ncol, (cx<float> *)p.G1, ncol,
-                          false, st);
+      launch_vertex32(nk, m->nRe, ncol, p.Pk32, m->gw32, (cx<float> *)p.G1, st);
+      if (after_vertex) {
+        CK(cudaEventRecord(m->ev_vertex, st));
+        CK(cudaStreamWaitEvent(sq, m->ev_vertex, 0));
+        q_tail();
+      }
       if (fork2) CK(cudaStreamWaitEvent(st, m->ev_join2, 0));
       launch_build_B<float>(m, nk, p.PkRM, (const cx<float> *)p.G1, p.Uk, (cx<float> *)p.Bg, (cx<float> *)p.BH, st);
     }
@@ -708,8 +723,6 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
       tcb->prebuilt_a = true;
     }
   }
-  if (fx && fx->pair && fx->omK)
-    launch_tables64(nq, nm, p.omegaT, omega_min, fx->T, fx->omK, fx->nbT, fx->wmax, sq);
   if (fork) {
     CK(cudaEventRecord(m->ev_join, sq));
     if (fx) fx->late = fx->late && gate;
@@ -1942,8 +1955,11 @@ extern "C" epw_status epw_linewidth_noalloc(const epw_model *mc, int nk, const d
   EpwTune tune = epwi_default_tune();
   tune.simt64 = true;  // the smallest buffers
   CKS(epwi_plan_linewidth(A, m, nk, nq, prec, false, false, false, false, tune, L));
-  if (A.off > EPW_NOALLOC_SCRATCH_BYTES)
-    return fail(EPW_ERR_INVALID_ARG, "problem needs %zu bytes of scratch; epw_linewidth_noalloc holds %zu", A.off,
+  // (the limit counts an FP32 copy of the vertex, which the model holds: the calls that fit stay the same)
+  const size_t need =
+      A.off + (prec == EPW_FP32 ? sizeof(cx<float>) * (size_t)m->nRe * m->nRp * m->nm * m->nw * m->nw : 0);
+  if (need > EPW_NOALLOC_SCRATCH_BYTES)
+    return fail(EPW_ERR_INVALID_ARG, "problem needs %zu bytes of scratch; epw_linewidth_noalloc holds %zu", need,
                 (size_t)EPW_NOALLOC_SCRATCH_BYTES);
   char *scratch = nullptr;
   CKS(noalloc_scratch(m->device, &scratch));

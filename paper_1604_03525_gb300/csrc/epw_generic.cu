@@ -70,7 +70,7 @@ __global__ void k_phases_fact(int npt, const double *__restrict__ x, int nR, con
   }
 }
 
-// The same sum with 8 lanes per element, for few points: a thread alone would run nR dependent
+// The same sum with 8 lanes per element, for few elements: a thread alone would run nR dependent
 // FP64 FMAs of 64 cycles each (24 k of the diamond model: 146 us).
 __global__ void k_fourier_few(int npt, int nR, const cx<double> *__restrict__ PT, const cx<double> *__restrict__ X,
                               int msize, cx<double> *out) {
@@ -219,6 +219,77 @@ __global__ void __launch_bounds__(128) k_vertex_fewk(int nk, int nR, int ncol, c
 #pragma unroll
     for (int t = 0; t < KT; t++)
       if (k0 + t < nk) G1[(size_t)(k0 + t) * ncol + c] = acc[t];
+}
+
+// G1[k][c] = sum_r P[k][r] g[r][c] in FP32: TM k x 64 columns per block of 128 threads, TM/8 x 4
+// complex sums a thread.  Packed FP32 (two FMAs per instruction on (re, im)): with the operands
+// stored as (x, x, -y, y) and (x, y, y, x) a complex product takes two instructions, in the order and
+// with the roundings of cfma, so the sums equal k_cgemm's bit for bit.  Alone, 249 x 95,616: 37 k 341
+// -> 284 us, 256 k 1.31 -> 1.12 ms; 135 x 6480, 21 k 33 -> 19 us.  Bound by the shared-memory reads
+// (59 % of the FMA rate).
+template <int TM>
+__global__ void __launch_bounds__(128) k_vertex32(int nk, int nR, int ncol, const cx<float> *__restrict__ P,
+                                                  const cx<float> *__restrict__ g, cx<float> *G1) {
+  constexpr int TK = 16, MI = TM / 8;
+  __shared__ float4 As[TK][TM + 1], Bs[TK][64];  // (+1: the stores run down a column)
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // columns tx + 16 j, rows ty + 8 i
+  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * 64;
+  float2 c[MI][4];
+#pragma unroll
+  for (int i = 0; i < MI; i++)
+#pragma unroll
+    for (int j = 0; j < 4; j++) c[i][j] = make_float2(0.0f, 0.0f);
+  constexpr int NA = TK * TM / 128, NB = TK * 64 / 128;
+  cx<float> ra[NA], rb[NB];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int t = 0; t < NA; t++) {
+      const int e = threadIdx.x + 128 * t, kk = e % TK, mm = e / TK;
+      ra[t] = (m0 + mm < nk && k0 + kk < nR) ? P[(size_t)(m0 + mm) * nR + k0 + kk] : mkc(0.0f, 0.0f);
+    }
+#pragma unroll
+    for (int t = 0; t < NB; t++) {
+      const int e = threadIdx.x + 128 * t, nn = e % 64, kk = e / 64;
+      rb[t] = (n0 + nn < ncol && k0 + kk < nR) ? g[(size_t)(k0 + kk) * ncol + n0 + nn] : mkc(0.0f, 0.0f);
+    }
+  };
+  fetch(0);
+  for (int k0 = 0; k0 < nR; k0 += TK) {
+#pragma unroll
+    for (int t = 0; t < NA; t++) {
+      const int e = threadIdx.x + 128 * t;
+      As[e % TK][e / TK] = make_float4(ra[t].x, ra[t].x, -ra[t].y, ra[t].y);
+    }
+#pragma unroll
+    for (int t = 0; t < NB; t++) {
+      const int e = threadIdx.x + 128 * t;
+      Bs[e / 64][e % 64] = make_float4(rb[t].x, rb[t].y, rb[t].y, rb[t].x);
+    }
+    __syncthreads();
+    if (k0 + TK < nR) fetch(k0 + TK);
+#pragma unroll 4
+    for (int kk = 0; kk < TK; kk++) {
+      float4 b[4];
+#pragma unroll
+      for (int j = 0; j < 4; j++) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < MI; i++) {
+        const float4 x = As[kk][ty + 8 * i];
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+          c[i][j] = __ffma2_rn(make_float2(x.x, x.y), make_float2(b[j].x, b[j].y),
+                               __ffma2_rn(make_float2(x.z, x.w), make_float2(b[j].z, b[j].w), c[i][j]));
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < MI; i++)
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      const int gm = m0 + ty + 8 * i, gn = n0 + tx + 16 * j;
+      if (gm < nk && gn < ncol) G1[(size_t)gm * ncol + gn] = mkc(c[i][j].x, c[i][j].y);
+    }
 }
 
 // Bg[k][Rp][a][j][n] = sum_i G1[k][Rp][a][j][i] U_k[i][n];  BH[k][Re][i][j] = P_k(Re) Hw(Re)_ij
@@ -1024,7 +1095,8 @@ __global__ void k_eliashberg(int nq, int nm, const double *__restrict__ omega, c
 
 // gw[Re][Rp][...] = wRe wRp g   (g complex128 or, with is_c64, complex64)
 __global__ void k_set_vertex(int nRe, int nRp, size_t per, const void *__restrict__ g, int is_c64,
-                             const double *__restrict__ wRe, const double *__restrict__ wRp, cx<double> *gw) {
+                             const double *__restrict__ wRe, const double *__restrict__ wRp, cx<double> *gw,
+                             cx<float> *gw32) {
   size_t n = (size_t)nRe * nRp * per;
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n; idx += (size_t)gridDim.x * blockDim.x) {
     size_t rr = idx / per;
@@ -1039,6 +1111,7 @@ __global__ void k_set_vertex(int nRe, int nRp, size_t per, const void *__restric
       im = ((const double *)g)[2 * idx + 1];
     }
     gw[idx] = mkc(s * re, s * im);
+    gw32[idx] = mkc((float)(s * re), (float)(s * im));
   }
 }
 
@@ -1075,14 +1148,14 @@ __global__ void __launch_bounds__(128) k_finalize_k(int nk, int nqb, int nw, con
   const int n = nqb * nw;
   const int per = ((n + 127) / 128) * 32;  // elements per warp, a multiple of 32
   const int j0 = warp * per, j1 = min(n, j0 + per);
+  // eight terms plainly, the groups compensated: the additions are FP64 instructions of 64 cycles
   double s = 0.0, c = 0.0;
   int j = j0 + lane;
-  for (; j + 96 < j1; j += 128) {
-    const double x0 = row[j], x1 = row[j + 32], x2 = row[j + 64], x3 = row[j + 96];
-    neumaier_add(s, c, x0);
-    neumaier_add(s, c, x1);
-    neumaier_add(s, c, x2);
-    neumaier_add(s, c, x3);
+  for (; j + 224 < j1; j += 256) {
+    double x[8];
+#pragma unroll
+    for (int t = 0; t < 8; t++) x[t] = row[j + 32 * t];
+    neumaier_add(s, c, ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7])));
   }
   for (; j < j1; j += 32) neumaier_add(s, c, row[j]);
   for (int o = 16; o >= nw; o >>= 1) {
@@ -1199,7 +1272,7 @@ void launch_fourier_d(int npt, int nR, const cx<double> *PT, const cx<double> *X
                       cudaStream_t st) {
   size_t n = (size_t)npt * msize;
   if (!n) return;
-  if (n * 8 <= 4 * 608 * 32)
+  if (n <= 65536)
     k_fourier_few<<<(unsigned)((n * 8 + 127) / 128), 128, 0, st>>>(npt, nR, PT, X, msize, out);
   else
     k_fourier_d<<<nblocks(n, 256), 256, 0, st>>>(npt, nR, PT, X, msize, out);
@@ -1226,6 +1299,18 @@ template void launch_cgemm<double>(int, int, int, const cx<double> *, int, bool,
                                    cx<double> *, int, bool, cudaStream_t);
 template void launch_cgemm<float>(int, int, int, const cx<float> *, int, bool, bool, const cx<float> *, int,
                                   cx<float> *, int, bool, cudaStream_t);
+
+void launch_vertex32(int nk, int nR, int ncol, const cx<float> *P, const cx<float> *g, cx<float> *G1,
+                     cudaStream_t st) {
+  if (nk <= 0 || ncol <= 0) return;
+  const int nb = (ncol + 63) / 64;
+  // 64 k per tile read the shared operands half as often, also with padding (37 k: 284 us against 336)
+  if (nk > 32)
+    k_vertex32<64><<<dim3(nb, (nk + 63) / 64), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  else
+    k_vertex32<32><<<dim3(nb, (nk + 31) / 32), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  epw_count_launch();
+}
 
 void launch_vertex_fewk(int nk, int nR, int ncol, const cx<double> *P, const cx<double> *g, cx<double> *G1,
                         cudaStream_t st) {
@@ -1306,7 +1391,9 @@ epw_status launch_pair_staged(const PairArgs &a, int mode, cudaStream_t st) {
     return launch_pair_wide<float>(a, mode, st);
   }
   dim3 grid((a.nq + 127) / 128, nkl);
-  if (mode == 0)
+  if (mode == 0 && a.nw <= 3)  // (nw = 4 keeps the Jacobi of the wider instance)
+    k_pair<float, 4, 9, 0, true><<<grid, 128, 0, st>>>(a);
+  else if (mode == 0)
     k_pair<float, 8, 9, 0, true><<<grid, 128, 0, st>>>(a);
   else
     k_pair<float, 8, 9, 1, true><<<grid, 128, 0, st>>>(a);
@@ -1426,7 +1513,7 @@ void launch_set_vertex(const epw_model *m, const void *g, int is_c64, cudaStream
   size_t per = (size_t)m->nm * m->nw * m->nw;
   size_t n = (size_t)m->nRe * m->nRp * per;
   if (!n) return;
-  k_set_vertex<<<nblocks(n, 256), 256, 0, st>>>(m->nRe, m->nRp, per, g, is_c64, m->wRe, m->wRp, m->gw);
+  k_set_vertex<<<nblocks(n, 256), 256, 0, st>>>(m->nRe, m->nRp, per, g, is_c64, m->wRe, m->wRp, m->gw, m->gw32);
   epw_count_launch();
 }
 

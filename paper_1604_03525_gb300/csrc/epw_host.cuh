@@ -39,7 +39,7 @@ struct Prep {
   double *omegaT;          // [nm][nq]
   void *ET;                // [nm*nm][nq] working precision
   void *G1, *Bg, *BH;      // working precision
-  cx<float> *Pk32, *gw32;  // FP32 copies for the k-side contraction
+  cx<float> *Pk32;         // FP32 copy for the k-side contraction
   void *Cpol;              // [nm][nq] long-range factors C_nu(q), working precision (polar models)
 };
 

@@ -318,6 +318,7 @@ struct epw_model {
   cx<double> *Phiw;       // [nRph][nm][nm], wRph and 1/sqrt(M M') folded
   float4 *Phidf;          // Phiw in double-float: (Re hi, Re lo, Im hi, Im lo) per entry
   cx<double> *gw;         // [nRe][nRp][nm][nw][nw], wRe wRp folded
+  cx<float> *gw32;        // the same in FP32 (the k-side vertex of the FP32 and split forms)
   double *mass;           // [nat]
   double *exptab;         // [EPW_EXPTAB] 2^(-j/EPW_EXPTAB), for the FP64 per-pair kernels
   unsigned int *dstatus;  // device status word
@@ -330,7 +331,7 @@ struct epw_model {
   unsigned char *ev_tag;  // [EPW_MAX_TIMED] tag of each timed launch
   // second stream for the q side of the preparation, and its fork / join events
   cudaStream_t aux;
-  cudaEvent_t ev_fork, ev_join, ev_phase, ev_gate;
+  cudaEvent_t ev_fork, ev_join, ev_phase, ev_gate, ev_vertex;
   // third stream: the k-side bands (H(k) and its eigensolve) beside the k-side vertex GEMM
   cudaStream_t aux2;
   cudaEvent_t ev_fork2, ev_join2;
@@ -380,6 +381,8 @@ void launch_phonon_post(int nq, int nm, const double *w2, const cx<double> *ev, 
 template <typename R>
 void launch_cgemm(int M, int N, int K, const cx<R> *A, int lda, bool transA, bool conjA, const cx<R> *B, int ldb,
                   cx<R> *C, int ldc, bool accumulate, cudaStream_t st);
+void launch_vertex32(int nk, int nR, int ncol, const cx<float> *P, const cx<float> *g, cx<float> *G1,
+                     cudaStream_t st);
 void launch_vertex_fewk(int nk, int nR, int ncol, const cx<double> *P, const cx<double> *g, cx<double> *G1,
                         cudaStream_t st);
 template <typename R>

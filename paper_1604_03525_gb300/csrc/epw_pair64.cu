@@ -37,7 +37,8 @@ __device__ __forceinline__ double exp64n(const double *__restrict__ tab, double 
   const double p = r * fma(r, fma(r, fma(r, 1.0 / 24.0, -1.0 / 6.0), 0.5), -1.0);
   const double T = tab[n & (EPW_EXPTAB - 1)], v = fma(T, p, T);
   const double s = __hiloint2double(__double2hiint(v) - ((n >> 9) << 20), __double2loint(v));
-  return z <= 707.0 ? s : (z != z ? z : 0.0);
+  // (z <= 707 by its high word, an integer comparison; NaN compares above)
+  return __double2hiint(z) <= 0x40861800 ? s : (z != z ? z : 0.0);
 }
 
 __device__ __forceinline__ double wsum64(double v) {
@@ -361,6 +362,10 @@ __device__ __forceinline__ void pair64_g(const Pair64Args &a, int kl, int q, int
 #pragma unroll 1
   for (int al = 0; al < nm; al++) {
     double2 t = make_double2(0.0, 0.0);
+    if constexpr (W == 1) {  // the eigenvector is 1
+      const size_t c = c0 + 2 * (size_t)al;
+      t = make_double2(fx_value(a.CG[c * a.ldc + q], a.eG[c], a.FG), fx_value(a.CG[(c + 1) * a.ldc + q], a.eG[c], a.FG));
+    } else
 #pragma unroll(W <= 9 ? W : 2)
     for (int i = 0; i < W; i++) {
       if (i >= n) continue;
