@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(SP_WARPS * 32) k_pair_sparse(PairArgs a) {
       if (lane == 0) S.phi[0] = ph;
       for (int r = 0; r < n - 1; r++) {
         const float ux = __shfl_sync(0xffffffffu, u.x, r), uy = __shfl_sync(0xffffffffu, u.y, r);
-        ph = mkc(ph.x * ux - ph.y * uy, ph.x * uy + ph.y * ux);
+        ph = mkc(fmaf(ph.x, ux, -__fmul_rn(ph.y, uy)), fmaf(ph.x, uy, __fmul_rn(ph.y, ux)));
         if (lane == 0) S.phi[r + 1] = ph;
       }
     }
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(SP_WARPS * 32) k_pair_sparse(PairArgs a) {
           const float cc = cg * cg, ss = sg * sg, cs = cg * sg;
           const float dn = fmaf(cc, ak, fmaf(-2.0f * cs, ok, ss * bk));
           const float dn1 = fmaf(ss, ak, fmaf(2.0f * cs, ok, cc * bk));
-          const float e0 = fmaf(cs, ak - bk, (cc - ss) * ok);
+          const float e0 = fmaf(cs, ak - bk, __fsub_rn(cc, ss) * ok);
           if (lane == r) {
             dr = dn;
             er = e0;
