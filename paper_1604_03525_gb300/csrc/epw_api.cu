@@ -76,7 +76,7 @@ static epw_status upload(T **dst, const T *src, size_t n) {
 }
 
 static void free_model_arrays(epw_model *m) {
-  void *ptrs[] = {m->Re, m->Rp, m->Rph, m->wRe, m->wRp, m->Hw, m->Phiw, m->Phidf, m->gw, m->gw32, m->mass, m->exptab, m->dstatus,
+  void *ptrs[] = {m->Re, m->Rp, m->Rph, m->wRe, m->wRp, m->Hw, m->Phiw, m->Phidf, m->gw, m->mass, m->exptab, m->dstatus,
                   m->ws, m->pZ};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -195,17 +195,12 @@ extern "C" epw_status epw_load_wannier(const epw_wannier_desc *d, epw_model **ou
     free(m);
     return s;
   }
-  cudaError_t e = cudaMalloc((void **)&m->gw32, gw.size() * sizeof(cx<float>));
-  if (e == cudaSuccess) {
-    launch_cast_c64_to_c32(gw.size(), m->gw, m->gw32, 0);
-    e = cudaStreamSynchronize(0);
-  }
-  if (e == cudaSuccess) e = cudaMalloc((void **)&m->dstatus, 16);
+  cudaError_t e = cudaMalloc((void **)&m->dstatus, 16);
   if (e == cudaSuccess) e = cudaMemset(m->dstatus, 0, 16);
   if (e != cudaSuccess) {
     free_model_arrays(m);
     free(m);
-    return fail(e == cudaErrorMemoryAllocation ? EPW_ERR_OOM : EPW_ERR_CUDA, "model buffers: %s", cudaGetErrorString(e));
+    return fail(EPW_ERR_CUDA, "status word: %s", cudaGetErrorString(e));
   }
   *out = m;
   return EPW_OK;
@@ -367,6 +362,27 @@ static epw_status ensure_ws(epw_model *m, size_t bytes) {
   return EPW_OK;
 }
 
+// The fixed-point forms take more workspace than the CUDA cores' (digit planes, the contractions of at
+// least one k over all q).  Plans beyond this keep the CUDA cores' form, so that a q list of any
+// length that fits the device without them still does (18 bands, 18 modes: 93 KB a q and k).
+static const size_t FX_WS_BYTES = (size_t)64 << 30;
+
+// Plans a call's workspace (plan(A), twice: its size, then its pointers).  The fixed-point forms are
+// taken (fx_on) while the whole plan stays within FX_WS_BYTES.
+template <class PLAN>
+static epw_status plan_ws(epw_model *m, Arena &A, const Fx64 &fx, bool &fx_on, PLAN plan) {
+  A = Arena{nullptr, 0, 0};
+  CKS(plan(A));
+  if (A.off > FX_WS_BYTES && (fx.dq || fx.g1)) {
+    fx_on = false;
+    A = Arena{nullptr, 0, 0};
+    CKS(plan(A));
+  }
+  CKS(ensure_ws(m, A.off));
+  A = Arena{(char *)m->ws, m->ws_bytes, 0};
+  return plan(A);
+}
+
 static size_t rsize(int prec) { return prec == EPW_FP64 ? sizeof(cx<double>) : sizeof(cx<float>); }
 
 // Lay out (or, with a null base, measure) the preparation buffers.
@@ -403,12 +419,14 @@ static void plan_prep(Arena &A, const epw_model *m, int nk, int nq, int prec, bo
     p.BH = fx && fx->pair ? nullptr : A.take<char>(sR * (size_t)nk * m->nRe * nw2);
     if (prec != EPW_FP64) {
       p.Pk32 = A.take<cx<float>>((size_t)nk * m->nRe);
+      p.gw32 = A.take<cx<float>>((size_t)m->nRe * m->nRp * m->nm * nw2);
     } else {
       p.Pk32 = nullptr;
+      p.gw32 = nullptr;
     }
   } else {
     p.G1 = p.Bg = p.BH = nullptr;
-    p.Pk32 = nullptr;
+    p.Pk32 = p.gw32 = nullptr;
   }
 }
 
@@ -619,6 +637,7 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   epw_model *m = const_cast<epw_model *>(mc);
   const int nw = m->nw, nm = m->nm;
   const size_t nw2 = (size_t)nw * nw;
+  const bool exact = fx && fx->exact;
   cudaStream_t sq = st;
   fork = fork && nq > 0 && nk > 0;
   if (fork) {
@@ -635,19 +654,19 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   } else if (fx && fx->pair) {
     CK(cudaMemsetAsync(fx->bad, 0, sizeof(int), st));
   } else if (prec == EPW_FP64) {
-    launch_phases(nq, q, m->nRe, m->Re, m->rmax, nullptr, (cx<double> *)p.PqTe, nullptr, sq);
-    if (!m->same_ep) launch_phases(nq, q, m->nRp, m->Rp, m->rmax, nullptr, (cx<double> *)p.PqTp, nullptr, sq);
-    if (!m->same_eph) launch_phases(nq, q, m->nRph, m->Rph, m->rmax, nullptr, p.PqTph, nullptr, sq);
+    launch_phases(nq, q, m->nRe, m->Re, m->rmax, nullptr, (cx<double> *)p.PqTe, nullptr, sq, exact);
+    if (!m->same_ep) launch_phases(nq, q, m->nRp, m->Rp, m->rmax, nullptr, (cx<double> *)p.PqTp, nullptr, sq, exact);
+    if (!m->same_eph) launch_phases(nq, q, m->nRph, m->Rph, m->rmax, nullptr, p.PqTph, nullptr, sq, exact);
   } else if (pa) {
     // staged and wide forms read no phase arrays: the A operand (from FP64 phases when Re = Rph)
     const bool dq = fx && fx->dq;
     *pa->done = dq && m->same_eph && pa->hi;
     if (!*pa->done && (!dq || (m->same_eph && pa->hi)))
-      launch_phases(nq, q, m->nRph, m->Rph, m->rmax, nullptr, p.PqTph, nullptr, sq);
+      launch_phases(nq, q, m->nRph, m->Rph, m->rmax, nullptr, p.PqTph, nullptr, sq, exact);
   } else {
-    launch_phases(nq, q, m->nRe, m->Re, m->rmax, nullptr, m->same_eph ? p.PqTph : nullptr, (cx<float> *)p.PqTe, sq);
-    if (!m->same_ep) launch_phases(nq, q, m->nRp, m->Rp, m->rmax, nullptr, nullptr, (cx<float> *)p.PqTp, sq);
-    if (!m->same_eph) launch_phases(nq, q, m->nRph, m->Rph, m->rmax, nullptr, p.PqTph, nullptr, sq);
+    launch_phases(nq, q, m->nRe, m->Re, m->rmax, nullptr, m->same_eph ? p.PqTph : nullptr, (cx<float> *)p.PqTe, sq, exact);
+    if (!m->same_ep) launch_phases(nq, q, m->nRp, m->Rp, m->rmax, nullptr, nullptr, (cx<float> *)p.PqTp, sq, exact);
+    if (!m->same_eph) launch_phases(nq, q, m->nRph, m->Rph, m->rmax, nullptr, p.PqTph, nullptr, sq, exact);
   }
   if (tcb && fork && !qs) CK(cudaEventRecord(m->ev_phase, sq));
   // phonons (FP64 eigensolve)
@@ -660,12 +679,13 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   // SM: launched while a GEMM fills it, their blocks share the few SMs that happen to have room
   // (13,824 of 9 x 9: 6.6 ms against 2.4; 1728: 3.3 against 0.8).  So the k-side vertex starts after
   // them where it runs on the tensor cores (FP64), and they start after it where it runs on the CUDA
-  // cores, which they slow down threefold (FP32: 809 us beside 9001 of 6 x 6, 284 alone).
-  const bool gate = fork && fx && fx->dq;
+  // cores, which they slow down threefold (FP32: 809 us beside 9001 of 6 x 6, 284 alone); the kernels
+  // after that vertex wait until they are launched (13,824 of 9 x 9 among them: 16.8 ms).
+  const bool gate = fork && fx && (fx->dq || exact);
   const bool after_vertex = gate && need_B && prec != EPW_FP64;
   if (gate) CK(cudaEventRecord(m->ev_gate, sq));
   auto q_tail = [&]() {
-    launch_eigh_d(nq, nm, p.D, p.w2, p.ev, m->dstatus, sq);
+    launch_eigh_d(nq, nm, p.D, p.w2, p.ev, m->dstatus, sq, exact);
     launch_phonon_post(nq, nm, p.w2, p.ev, m->mass, omega_min, p.omegaT,
                        prec == EPW_FP64 ? (cx<double> *)p.ET : nullptr,
                        prec == EPW_FP64 ? nullptr : (cx<float> *)p.ET, omega_out, sq);
@@ -682,7 +702,7 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   // k side (FP64): phases, H(k), eigensolve, then the k-side vertex; with a fork the
   // bands (H(k), eigensolve) run on a third stream beside the vertex GEMM, which
   // needs only the phases, and are joined before the U_k rotation
-  launch_phases(nk, k, m->nRe, m->Re, m->rmax, p.PkRM, p.PkT, nullptr, st);
+  launch_phases(nk, k, m->nRe, m->Re, m->rmax, p.PkRM, p.PkT, nullptr, st, exact);
   const bool fork2 = fork && need_B;
   cudaStream_t sk = st;
   if (fork2) {
@@ -690,8 +710,8 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
     CK(cudaStreamWaitEvent(m->aux2, m->ev_fork2, 0));
     sk = m->aux2;
   }
-  launch_fourier_d(nk, m->nRe, p.PkT, m->Hw, (int)nw2, p.Hk, sk);
-  launch_eigh_d(nk, nw, p.Hk, p.epsk, p.Uk, m->dstatus, sk);
+  launch_fourier_d(nk, m->nRe, p.PkT, m->Hw, (int)nw2, p.Hk, sk, exact);
+  launch_eigh_d(nk, nw, p.Hk, p.epsk, p.Uk, m->dstatus, sk, exact);
   if (fork2) CK(cudaEventRecord(m->ev_join2, sk));
   if (need_B && nk > 0) {
     const int ncol = m->nRp * nm * (int)nw2;
@@ -703,11 +723,13 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
                              st);
     } else {
       launch_cast_c64_to_c32((size_t)nk * m->nRe, p.PkRM, p.Pk32, st);
-      launch_vertex32(nk, m->nRe, ncol, p.Pk32, m->gw32, (cx<float> *)p.G1, st);
+      launch_vertex32(nk, m->nRe, ncol, p.Pk32, m->gw, p.gw32, (cx<float> *)p.G1, st);
       if (after_vertex) {
         CK(cudaEventRecord(m->ev_vertex, st));
         CK(cudaStreamWaitEvent(sq, m->ev_vertex, 0));
+        CK(cudaEventRecord(m->ev_gate, sq));
         q_tail();
+        CK(cudaStreamWaitEvent(st, m->ev_gate, 0));
       }
       if (fork2) CK(cudaStreamWaitEvent(st, m->ev_join2, 0));
       launch_build_B<float>(m, nk, p.PkRM, (const cx<float> *)p.G1, p.Uk, (cx<float> *)p.Bg, (cx<float> *)p.BH, st);
@@ -873,6 +895,16 @@ epw_status epwi_plan_linewidth(Arena &A, const epw_model *m, int nk, int nq, int
   tune.pair64 = !tune.simt64 && prec == EPW_FP64 && fx_pair(m, nk, nq);
   tune.g1_64 = !tune.simt64 && prec == EPW_FP64 && fx_g1(m, nk);
   L.kchunk = k_per_pass(m, nk, nq, prec, tune);
+  if (!tune.simt64) {
+    Arena a{nullptr, 0, 0};
+    LwPlan t;
+    CKS(plan_linewidth_pass(a, m, L.kchunk, nq, prec, false, false, tune, t));
+    if (a.off > FX_WS_BYTES && (t.fx.dq || t.fx.g1)) {
+      tune.simt64 = true;
+      tune.pair64 = tune.g1_64 = false;
+      L.kchunk = k_per_pass(m, nk, nq, prec, tune);
+    }
+  }
   double *kd = sk ? A.take<double>(3 * (size_t)nk) : nullptr;  // the whole k list, staged from the host
   CKS(plan_linewidth_pass(A, m, L.kchunk, nq, prec, sq, swq, tune, L));
   L.p.kd = kd;
@@ -1139,10 +1171,15 @@ extern "C" epw_status epw_interp_g(const epw_model *mc, int nk, const double *k,
   bool need_B = true;
   cx<double> *Hq = nullptr, *Uq = nullptr;
   double *wkq = nullptr;
-  auto plan = [&](Arena &A, Prep &p, double *&ekd, double *&ekqd, double *&omd, double *&gd) -> epw_status {
+  Prep p;
+  double *ekd, *ekqd, *omd, *gd;
+  bool fx_on = true;
+  auto plan = [&](Arena &A) -> epw_status {
     const size_t per = (size_t)nq * nw * (40 * nw + 8);  // H(k+q) twice, its eigenvectors and eigenvalues
-    plan_fx(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, !tc && fx_dq(m, nq),
-            precision == EPW_FP64 && want_pairs && fx_pair(m, nk, nq), precision == EPW_FP64 && nk > 0 && g && fx_g1(m, nk), fx, per);
+    plan_fx(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, fx_on && precision == EPW_FP64 && fx_dq(m, nq),
+            fx_on && precision == EPW_FP64 && want_pairs && fx_pair(m, nk, nq),
+            fx_on && precision == EPW_FP64 && nk > 0 && g && fx_g1(m, nk), fx, per);
+    fx.exact = precision != EPW_FP64;
     if (fx.pair) {
       const size_t np = (size_t)nq * fx.kc;
       fx.omK = nullptr;  // (no tables: no occupations here)
@@ -1162,13 +1199,8 @@ extern "C" epw_status epw_interp_g(const epw_model *mc, int nk, const double *k,
     if (staged) return tc_staged_plan(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, op, STAGED_CT_BYTES, sg);
     return EPW_OK;
   };
-  Arena A{nullptr, 0, 0};
-  Prep p;
-  double *ekd, *ekqd, *omd, *gd;
-  CKS(plan(A, p, ekd, ekqd, omd, gd));
-  CKS(ensure_ws(m, A.off));
-  A = Arena{(char *)m->ws, m->ws_bytes, 0};
-  CKS(plan(A, p, ekd, ekqd, omd, gd));
+  Arena A;
+  CKS(plan_ws(m, A, fx, fx_on, plan));
   const double *kd = k, *qd = q;
   if (sk) {
     CK(cudaMemcpyAsync(p.kd, k, sizeof(double) * 3 * nk, cudaMemcpyHostToDevice, st));
@@ -1302,7 +1334,7 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
   const bool swq = wq && nq > 0 && !is_device_ptr(wq), scot = nk > 0 && !is_device_ptr(cot);
   const bool sdg = dg && !is_device_ptr(dg), sdT = dT && !is_device_ptr(dT), sdE = dEF && !is_device_ptr(dEF);
   const size_t sR = rsize(prec);
-  const bool pair64 = prec == EPW_FP64 && nk > 0 && nq > 0 && fx_pair(m, nk, nq);
+  bool fx_on = true, pair64 = false;
   // k chunk so that the per-chunk adjoint buffers stay near 1 GiB
   size_t per_k = (size_t)nq * per * sR + 2 * (size_t)m->nRp * per * sR;
   int nkc = (int)std::max<size_t>(1, std::min<size_t>((size_t)std::max(nk, 1), ((size_t)1 << 30) / std::max<size_t>(per_k, 1)));
@@ -1324,9 +1356,11 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
   b.sg = TcStaged{};
   auto plan = [&](Arena &A) -> epw_status {
     const int kpq = fx_kpad(nq);
-    plan_fx(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, !tcb && fx_dq(m, nq), pair64,
-            prec == EPW_FP64 && nk > 0 && fx_g1(m, nk), b.fx,
+    pair64 = fx_on && prec == EPW_FP64 && nk > 0 && nq > 0 && fx_pair(m, nk, nq);
+    plan_fx(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, fx_on && prec == EPW_FP64 && fx_dq(m, nq), pair64,
+            fx_on && prec == EPW_FP64 && nk > 0 && fx_g1(m, nk), b.fx,
             per * ((size_t)nq * 16 + 2 * FX_S * (size_t)kpq + 16 * (size_t)fx_splits(kpq) * m->nRp + 16 * (size_t)m->nRp));
+    b.fx.exact = prec != EPW_FP64;
     plan_prep(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, prec, sk, sq, swq, true, b.p, &b.fx);
     b.cotd = scot ? A.take<double>((size_t)nk * m->nw) : (double *)cot;
     if (pair64) {
@@ -1367,11 +1401,8 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
     b.dgd = sdg ? A.take<double>(2 * ng) : dg;
     return EPW_OK;
   };
-  Arena A{nullptr, 0, 0};
-  CKS(plan(A));
-  CKS(ensure_ws(m, A.off));
-  A = Arena{(char *)m->ws, m->ws_bytes, 0};
-  CKS(plan(A));
+  Arena A;
+  CKS(plan_ws(m, A, b.fx, fx_on, plan));
   Prep &p = b.p;
   const double *kd = k, *qd = q, *wqd = wq;
   if (sk) {
@@ -1425,7 +1456,7 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
                       k0 > 0));
     }
   } else if (nk > 0 && nq > 0 && tcb) {
-    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st));
+    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx));
     b.tc.Cpol = m->polar ? (const float2 *)p.Cpol : nullptr;
     b.tc.Uk64 = p.Uk;
     b.tc.Pq64 = m->same_eph ? p.PqTph : nullptr;
@@ -1434,10 +1465,8 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
                                          b.cotd, b.tc, b.tw, (cx<float> *)b.gwbar, b.sc, st);
     if (s != EPW_OK) return fail(s, "tensor-core adjoint failed");
   } else if (nk > 0 && nq > 0) {
-    const PhaseA pa = staged_a(m, b.sg);
     b.fx.late = staged;
-    CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx,
-                 staged ? &pa : nullptr));
+    CKS(run_prep(m, nk, kd, nq, qd, prec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx));
     b.sg.Pq64 = m->same_eph ? p.PqTph : nullptr;
     if (staged) {
       CKS(tc_staged_phases(m, nq, qd, b.sg, st));
@@ -1555,7 +1584,8 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
   // chunks of k per q block: enough blocks to fill the GPU a few times over
   const int nqb = (std::max(nq, 1) + 127) / 128;
   const int want = std::max(1, (4 * 152 + nqb - 1) / nqb);
-  int kper = std::max(1, (std::max(nk, 1) + want - 1) / want);
+  const int kper0 = std::max(1, (std::max(nk, 1) + want - 1) / want);
+  int kper = kper0;
   // (FP64 in fixed point: warps of 32 q x kper k, about eight waves of two per sub-partition)
   const int kper64 = (int)std::max<long>(1, (long)std::max(nk, 1) * ((std::max(nq, 1) + 31) / 32) / 9728);
   struct B {
@@ -1565,16 +1595,18 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
     double *partial, *pid, *lamd, *zd, *dosd, *terms, *wkd;
     int nchunk;
   } b;
+  bool fx_on = true;
   auto plan = [&](Arena &A) -> epw_status {
-    plan_fx(A, m, std::max(nk, 1), std::max(nq, 1), fx_dq(m, nq),
-            par->precision == EPW_FP64 && nk > 0 && nq > 0 && fx_pair(m, nk, nq),
-            par->precision == EPW_FP64 && nk > 0 && fx_g1(m, nk), b.fx);
+    plan_fx(A, m, std::max(nk, 1), std::max(nq, 1), fx_on && par->precision == EPW_FP64 && fx_dq(m, nq),
+            fx_on && par->precision == EPW_FP64 && nk > 0 && nq > 0 && fx_pair(m, nk, nq),
+            fx_on && par->precision == EPW_FP64 && nk > 0 && fx_g1(m, nk), b.fx);
+    b.fx.exact = par->precision != EPW_FP64;
     plan_prep(A, m, std::max(nk, 1), std::max(nq, 1), wprec, sk, sq, false, true, b.p, &b.fx);
     b.wkd = swk ? A.take<double>((size_t)nk) : nullptr;  // k weights staged from the host
     b.sg = TcStaged{};
+    kper = b.fx.pair ? kper64 : kper0;
     int nchunk = (std::max(nk, 1) + kper - 1) / kper;
     if (b.fx.pair) {
-      kper = kper64;
       nchunk = 0;
       for (int k0 = 0; k0 < nk; k0 += b.fx.kc) nchunk += (std::min(b.fx.kc, nk - k0) + kper - 1) / kper;
     }
@@ -1597,11 +1629,8 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
     b.terms = A.take<double>((size_t)std::max(nk, 1));
     return EPW_OK;
   };
-  Arena A{nullptr, 0, 0};
-  CKS(plan(A));
-  CKS(ensure_ws(m, A.off));
-  A = Arena{(char *)m->ws, m->ws_bytes, 0};
-  CKS(plan(A));
+  Arena A;
+  CKS(plan_ws(m, A, b.fx, fx_on, plan));
   Prep &p = b.p;
   const double *kd = k, *qd = q, *wkd = wk;
   if (sk) {
@@ -1623,11 +1652,9 @@ extern "C" epw_status epw_phonon_selfenergy(const epw_model *mc, int nk, const d
     if (b.zd) CK(cudaMemsetAsync(b.zd, 0, sizeof(double) * (size_t)nq, st));
   }
   if (nk > 0 && nq > 0) {
-    const PhaseA pa = staged_a(m, b.sg);
     b.fx.T = par->T_K;
     b.fx.late = b.fx.pair;
-    CKS(run_prep(m, nk, kd, nq, qd, wprec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx,
-                 tcp ? &pa : nullptr));
+    CKS(run_prep(m, nk, kd, nq, qd, wprec, par->omega_min_eV, true, p, nullptr, st, true, nullptr, &b.fx));
   } else if (nk > 0) {
     // bands at k only (N(E_F))
     launch_phases(nk, kd, m->nRe, m->Re, m->rmax, p.PkRM, p.PkT, nullptr, st);
@@ -1748,8 +1775,10 @@ extern "C" epw_status epw_selfenergy(const epw_model *mc, int nk, const double *
     double *omd, *sigd, *specd, *re0;
     double2 *part;
   } b;
+  bool fx_on = true;
   auto plan = [&](Arena &A) -> epw_status {
-    plan_fx(A, m, nk, std::max(nq, 1), fx_dq(m, nq), false, wprec == EPW_FP64 && nq > 0 && fx_g1(m, nk), b.fx);
+    plan_fx(A, m, nk, std::max(nq, 1), fx_on && fx_dq(m, nq), false,
+            fx_on && wprec == EPW_FP64 && nq > 0 && fx_g1(m, nk), b.fx);
     plan_prep(A, m, nk, std::max(nq, 1), wprec, sk, sq, swq, true, b.p, &b.fx);
     b.sg = TcStaged{};
     if (tcp) {
@@ -1765,11 +1794,8 @@ extern "C" epw_status epw_selfenergy(const epw_model *mc, int nk, const double *
     b.re0 = A.take<double>((size_t)kc * nw);
     return EPW_OK;
   };
-  Arena A{nullptr, 0, 0};
-  CKS(plan(A));
-  CKS(ensure_ws(m, A.off));
-  A = Arena{(char *)m->ws, m->ws_bytes, 0};
-  CKS(plan(A));
+  Arena A;
+  CKS(plan_ws(m, A, b.fx, fx_on, plan));
   Prep &p = b.p;
   const double *kd = k, *qd = q, *wqd = wq;
   if (sk) {
@@ -1955,11 +1981,8 @@ extern "C" epw_status epw_linewidth_noalloc(const epw_model *mc, int nk, const d
   EpwTune tune = epwi_default_tune();
   tune.simt64 = true;  // the smallest buffers
   CKS(epwi_plan_linewidth(A, m, nk, nq, prec, false, false, false, false, tune, L));
-  // (the limit counts an FP32 copy of the vertex, which the model holds: the calls that fit stay the same)
-  const size_t need =
-      A.off + (prec == EPW_FP32 ? sizeof(cx<float>) * (size_t)m->nRe * m->nRp * m->nm * m->nw * m->nw : 0);
-  if (need > EPW_NOALLOC_SCRATCH_BYTES)
-    return fail(EPW_ERR_INVALID_ARG, "problem needs %zu bytes of scratch; epw_linewidth_noalloc holds %zu", need,
+  if (A.off > EPW_NOALLOC_SCRATCH_BYTES)
+    return fail(EPW_ERR_INVALID_ARG, "problem needs %zu bytes of scratch; epw_linewidth_noalloc holds %zu", A.off,
                 (size_t)EPW_NOALLOC_SCRATCH_BYTES);
   char *scratch = nullptr;
   CKS(noalloc_scratch(m->device, &scratch));

@@ -198,7 +198,7 @@ double job_cost(const epw_linewidth_job &j) {
   const epw_model *m = j.model;
   const double flops = 8.0 * m->nRe * m->nw * m->nw * (m->nm + 1) * (double)j.nk * j.nq;
   const int p = j.params.precision;
-  const double rate = p == EPW_FP64 ? 0.5e12 : p == EPW_FP32 ? 10e12 : 200e12;
+  const double rate = p == EPW_FP64 || p == EPW_FP32 ? 10e12 : 200e12;  // FP64 measured 13-18e12, FP32 8e12
   return flops / rate * 1e3 + 0.05;
 }
 

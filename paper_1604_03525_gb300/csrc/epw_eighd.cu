@@ -19,38 +19,66 @@
 
 namespace {
 
-// Parameters of the rotation that zeroes a_pq: c, (sx, sy) = s a_pq/|a_pq|, and tm = t |a_pq|
-// (app -= tm, aqq += tm).  With theta = (aqq - app) / (2 |a_pq|) and h = 1/sqrt(1 + theta^2):
-// c^2 = (1 + |theta| h) / 2, s = sign(theta) h / (2c), t = s / c.
-__device__ __forceinline__ void jrot_d(double app, double aqq, double ax, double ay, double m2, double &c, double &sx,
-                                       double &sy, double &tm) {
-  const double r = rsqrt(m2);
-  const double th = (aqq - app) * (0.5 * r);
-  // clamped: theta^2 must not overflow (a rotation that small changes nothing)
-  const double at = fmin(fabs(th), 1e150);
-  const double h = rsqrt(fma(at, at, 1.0));
-  const double rc = rsqrt(fma(0.5 * at, h, 0.5));  // 1/c
-  c = fma(0.5 * at, h, 0.5) * rc;
-  double s = 0.5 * h * rc;
-  s = th < 0.0 ? -s : s;
-  tm = s * rc * (m2 * r);
-  const double sr = s * r;
-  sx = sr * ax;
-  sy = sr * ay;
+// X: jacobi_herm's arithmetic to the bit (three square roots and divisions, its order of products):
+// for the FP32 adjoint, whose gradient is summed and rounded in FP32, so that one phonon that is
+// cast to FP32 the other way moves a few percent of its entries by a last place.
+//
+// The rotation that zeroes a_pq: c, (sx, sy) = s a_pq/|a_pq|, and the new diagonal.  With theta =
+// (aqq - app) / (2 |a_pq|) and h = 1/sqrt(1 + theta^2): c^2 = (1 + |theta| h) / 2, s = sign(theta) h
+// / (2c), t = s / c.
+template <bool X>
+__device__ __forceinline__ void jrot_d(double &app, double &aqq, double ax, double ay, double m2, double &c, double &sx,
+                                       double &sy) {
+  if constexpr (X) {
+    const double mag = sqrt(m2), rinv = 1.0 / mag;
+    const double th = (aqq - app) * (0.5 * rinv);
+    double t = 1.0 / (fabs(th) + sqrt(fma(th, th, 1.0)));
+    t = th < 0.0 ? -t : t;
+    c = 1.0 / sqrt(fma(t, t, 1.0));
+    const double s = t * c;
+    app = fma(-t, mag, app);
+    aqq = fma(t, mag, aqq);
+    sx = s * (ax * rinv);
+    sy = s * (ay * rinv);
+  } else {
+    const double r = rsqrt(m2);
+    const double th = (aqq - app) * (0.5 * r);
+    // clamped: theta^2 must not overflow (a rotation that small changes nothing)
+    const double at = fmin(fabs(th), 1e150);
+    const double h = rsqrt(fma(at, at, 1.0));
+    const double rc = rsqrt(fma(0.5 * at, h, 0.5));  // 1/c
+    c = fma(0.5 * at, h, 0.5) * rc;
+    double s = 0.5 * h * rc;
+    s = th < 0.0 ? -s : s;
+    const double tm = s * rc * (m2 * r);
+    const double sr = s * r;
+    app -= tm;
+    aqq += tm;
+    sx = sr * ax;
+    sy = sr * ay;
+  }
 }
 
 // (u, v) <- (c u - conj(se) v, se u + c v), se = sx + i sy
+template <bool X>
 __device__ __forceinline__ void jrow_d(double c, double sx, double sy, double2 &u, double2 &v) {
   const double2 a = u, b = v;
-  u.x = fma(-sx, b.x, fma(-sy, b.y, c * a.x));
-  u.y = fma(-sx, b.y, fma(sy, b.x, c * a.y));
-  v.x = fma(sx, a.x, fma(-sy, a.y, c * b.x));
-  v.y = fma(sx, a.y, fma(sy, a.x, c * b.y));
+  if constexpr (X) {
+    u.x = fma(c, a.x, -fma(sx, b.x, __dmul_rn(sy, b.y)));
+    u.y = fma(c, a.y, -fma(sx, b.y, -__dmul_rn(sy, b.x)));
+    v.x = fma(c, b.x, fma(sx, a.x, -__dmul_rn(sy, a.y)));
+    v.y = fma(c, b.y, fma(sx, a.y, __dmul_rn(sy, a.x)));
+  } else {
+    u.x = fma(-sx, b.x, fma(-sy, b.y, c * a.x));
+    u.y = fma(-sx, b.y, fma(sy, b.x, c * a.y));
+    v.x = fma(sx, a.x, fma(-sy, a.y, c * b.x));
+    v.y = fma(sx, a.y, fma(sy, a.x, c * b.y));
+  }
 }
 
 // ------------------------------------------------------ one thread per matrix
 // A (upper triangle) and V in registers: every index is a compile-time constant.
-template <int N>
+template <int N, bool X>
 __global__ void __launch_bounds__(64) k_eigh_reg(int nmat, const double2 *__restrict__ Ain, double *w, double2 *V,
                                                  unsigned *dstatus) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -86,10 +114,8 @@ __global__ void __launch_bounds__(64) k_eigh_reg(int nmat, const double2 *__rest
       for (int q = p + 1; q < N; q++) {
         const double ax = A[p][q].x, ay = A[p][q].y, m2 = fma(ax, ax, ay * ay);
         if (m2 != 0.0) {
-          double c, sx, sy, tm;
-          jrot_d(d[p], d[q], ax, ay, m2, c, sx, sy, tm);
-          d[p] -= tm;
-          d[q] += tm;
+          double c, sx, sy;
+          jrot_d<X>(d[p], d[q], ax, ay, m2, c, sx, sy);
           A[p][q] = make_double2(0.0, 0.0);
 #pragma unroll
           for (int r = 0; r < N; r++) {
@@ -97,7 +123,7 @@ __global__ void __launch_bounds__(64) k_eigh_reg(int nmat, const double2 *__rest
             // A[r][p], A[r][q] from the stored upper triangle (lower entries are conjugates)
             double2 u = r < p ? A[r][p] : make_double2(A[p][r].x, -A[p][r].y);
             double2 v = r < q ? A[r][q] : make_double2(A[q][r].x, -A[q][r].y);
-            jrow_d(c, sx, sy, u, v);
+            jrow_d<X>(c, sx, sy, u, v);
             if (r < p)
               A[r][p] = u;
             else
@@ -108,7 +134,7 @@ __global__ void __launch_bounds__(64) k_eigh_reg(int nmat, const double2 *__rest
               A[q][r] = make_double2(v.x, -v.y);
           }
 #pragma unroll
-          for (int r = 0; r < N; r++) jrow_d(c, sx, sy, U[r][p], U[r][q]);
+          for (int r = 0; r < N; r++) jrow_d<X>(c, sx, sy, U[r][p], U[r][q]);
         }
       }
   }
@@ -126,7 +152,7 @@ __global__ void __launch_bounds__(64) k_eigh_reg(int nmat, const double2 *__rest
 }
 
 // The same with indexed (local-memory) arrays, for n beyond the registers.
-template <int N>
+template <int N, bool X>
 __global__ void __launch_bounds__(64) k_eigh_loc(int nmat, const double2 *__restrict__ Ain, double *w, double2 *V,
                                                  unsigned *dstatus) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -162,22 +188,20 @@ __global__ void __launch_bounds__(64) k_eigh_loc(int nmat, const double2 *__rest
       for (int q = p + 1; q < N; q++) {
         const double ax = A[p][q].x, ay = A[p][q].y, m2 = fma(ax, ax, ay * ay);
         if (m2 == 0.0) continue;
-        double c, sx, sy, tm;
-        jrot_d(d[p], d[q], ax, ay, m2, c, sx, sy, tm);
-        d[p] -= tm;
-        d[q] += tm;
+        double c, sx, sy;
+        jrot_d<X>(d[p], d[q], ax, ay, m2, c, sx, sy);
         A[p][q] = A[q][p] = make_double2(0.0, 0.0);
 #pragma unroll
         for (int r = 0; r < N; r++) {
           if (r != p && r != q) {
             double2 u = A[r][p], v = A[r][q];
-            jrow_d(c, sx, sy, u, v);
+            jrow_d<X>(c, sx, sy, u, v);
             A[r][p] = u;
             A[p][r] = make_double2(u.x, -u.y);
             A[r][q] = v;
             A[q][r] = make_double2(v.x, -v.y);
           }
-          jrow_d(c, sx, sy, U[r][p], U[r][q]);
+          jrow_d<X>(c, sx, sy, U[r][p], U[r][q]);
         }
       }
   }
@@ -198,7 +222,7 @@ __global__ void __launch_bounds__(64) k_eigh_loc(int nmat, const double2 *__rest
 // lane l of the group takes l, l + L, ...  Control flow is uniform over the warp (__syncwarp):
 // a group whose matrix has converged only keeps step with the others.
 constexpr int EC_WARPS = 4;  // one warp per SM sub-partition
-template <int L>
+template <int L, bool X>
 __global__ void __launch_bounds__(EC_WARPS * 32) k_eigh_coop(int nmat, int n, const double2 *__restrict__ Ain,
                                                              double *w, double2 *V, unsigned *dstatus) {
   extern __shared__ __align__(16) double2 ec_sm[];
@@ -236,25 +260,25 @@ __global__ void __launch_bounds__(EC_WARPS * 32) k_eigh_coop(int nmat, int n, co
     for (int p = 0; p < n - 1; p++)
       for (int q = p + 1; q < n; q++) {
         const double2 apq = A[p * n + q];
-        const double app = A[p * n + p].x, aqq = A[q * n + q].x;
+        double app = A[p * n + p].x, aqq = A[q * n + q].x;
         const double m2 = fma(apq.x, apq.x, apq.y * apq.y);
         const bool act = !done && m2 != 0.0;
         __syncwarp();
         if (act) {
-          double c, sx, sy, tm;
-          jrot_d(app, aqq, apq.x, apq.y, m2, c, sx, sy, tm);
+          double c, sx, sy;
+          jrot_d<X>(app, aqq, apq.x, apq.y, m2, c, sx, sy);
           for (int it = l; it < 2 * n; it += L) {
             const bool isA = it < n;
             const int r = isA ? it : it - n;
             if (isA && (r == p || r == q)) {
               // the 2 x 2 block
-              A[r * n + r].x = r == p ? app - tm : aqq + tm;
+              A[r * n + r].x = r == p ? app : aqq;
               A[r * n + (r == p ? q : p)] = make_double2(0.0, 0.0);
               continue;
             }
             double2 *row = (isA ? A : U) + r * n;
             double2 u = row[p], v = row[q];
-            jrow_d(c, sx, sy, u, v);
+            jrow_d<X>(c, sx, sy, u, v);
             row[p] = u;
             row[q] = v;
             if (isA) {
@@ -280,13 +304,13 @@ __global__ void __launch_bounds__(EC_WARPS * 32) k_eigh_coop(int nmat, int n, co
   }
 }
 
-template <int L>
+template <int L, bool X>
 void eigh_coop(int nmat, int n, const cx<double> *A, double *w, cx<double> *V, unsigned *dstatus, cudaStream_t st) {
   constexpr int per = EC_WARPS * (32 / L);  // matrices per block
   const size_t smem = (size_t)per * (2 * n * n + 1) * sizeof(double2);
   if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_eigh_coop<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_eigh_coop<L><<<(nmat + per - 1) / per, EC_WARPS * 32, smem, st>>>(nmat, n, (const double2 *)A, w, (double2 *)V,
+    cudaFuncSetAttribute(k_eigh_coop<L, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_eigh_coop<L, X><<<(nmat + per - 1) / per, EC_WARPS * 32, smem, st>>>(nmat, n, (const double2 *)A, w, (double2 *)V,
                                                                       dstatus);
 }
 
@@ -303,9 +327,8 @@ double eigh_cost(long nmat, int n, int L) {
   return waves * (40.0 + 12.0 * rows) * (L == 1 ? 1.0 : 1.25);
 }
 
-}  // namespace
-
-void launch_eigh_d(int nmat, int n, cx<double> *A, double *w, cx<double> *V, unsigned *dstatus, cudaStream_t st) {
+template <bool X>
+void eigh_d(int nmat, int n, cx<double> *A, double *w, cx<double> *V, unsigned *dstatus, cudaStream_t st) {
   if (!nmat) return;
   const double2 *Ad = (const double2 *)A;
   double2 *Vd = (double2 *)V;
@@ -319,31 +342,38 @@ void launch_eigh_d(int nmat, int n, cx<double> *A, double *w, cx<double> *V, uns
   const int s = nmat <= 608 * 32 ? 32 : 64;  // a block per warp while sub-partitions would idle
   const int grid = (nmat + s - 1) / s;
   if (L == 32)
-    eigh_coop<32>(nmat, n, A, w, V, dstatus, st);
+    eigh_coop<32, X>(nmat, n, A, w, V, dstatus, st);
   else if (L == 16)
-    eigh_coop<16>(nmat, n, A, w, V, dstatus, st);
+    eigh_coop<16, X>(nmat, n, A, w, V, dstatus, st);
   else if (L == 8)
-    eigh_coop<8>(nmat, n, A, w, V, dstatus, st);
+    eigh_coop<8, X>(nmat, n, A, w, V, dstatus, st);
   else if (L == 4)
-    eigh_coop<4>(nmat, n, A, w, V, dstatus, st);
+    eigh_coop<4, X>(nmat, n, A, w, V, dstatus, st);
   else {
     if (n > 6) {
       // indexed arrays live in L1, but not in all of it: with no shared memory left on an SM no
       // block that needs some can join it while this kernel runs
-      const void *f = n == 7 ? (const void *)k_eigh_loc<7> : n == 8 ? (const void *)k_eigh_loc<8> : (const void *)k_eigh_loc<9>;
+      const void *f = n == 7 ? (const void *)k_eigh_loc<7, X> : n == 8 ? (const void *)k_eigh_loc<8, X> : (const void *)k_eigh_loc<9, X>;
       cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
     }
     switch (n) {
-      case 1: k_eigh_reg<1><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
-      case 2: k_eigh_reg<2><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
-      case 3: k_eigh_reg<3><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
-      case 4: k_eigh_reg<4><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
-      case 5: k_eigh_reg<5><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
-      case 6: k_eigh_reg<6><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
-      case 7: k_eigh_loc<7><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
-      case 8: k_eigh_loc<8><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
-      default: k_eigh_loc<9><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
+      case 1: k_eigh_reg<1, X><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
+      case 2: k_eigh_reg<2, X><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
+      case 3: k_eigh_reg<3, X><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
+      case 4: k_eigh_reg<4, X><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
+      case 5: k_eigh_reg<5, X><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
+      case 6: k_eigh_reg<6, X><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
+      case 7: k_eigh_loc<7, X><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
+      case 8: k_eigh_loc<8, X><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
+      default: k_eigh_loc<9, X><<<grid, s, 0, st>>>(nmat, Ad, w, Vd, dstatus); break;
     }
   }
   epw_count_launch();
+}
+
+}  // namespace
+
+void launch_eigh_d(int nmat, int n, cx<double> *A, double *w, cx<double> *V, unsigned *dstatus, cudaStream_t st,
+                   bool exact) {
+  exact ? eigh_d<true>(nmat, n, A, w, V, dstatus, st) : eigh_d<false>(nmat, n, A, w, V, dstatus, st);
 }

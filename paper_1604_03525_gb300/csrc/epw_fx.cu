@@ -481,11 +481,6 @@ __global__ void __launch_bounds__(128) k_fx_hermitian(int nk, int nR, int n, con
   for (int r = lane + 32 * NV; r < kpad / 2; r += 32) put(r, r < nR ? value(r) : FxRows{0.0, 0.0, 0.0, 0.0});
 }
 
-__global__ void k_fx_scales(size_t n, const short *__restrict__ e, int F, double *scale) {
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i < n) scale[i] = e[i] == FX_BAD ? __longlong_as_double(0x7ff8000000000000LL) : pow2d(e[i] - F);
-}
-
 __global__ void k_fx_unpack(int npt, int n, const double *__restrict__ in, double2 *out) {
   const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (i >= (size_t)npt * n * n) return;
@@ -613,12 +608,6 @@ epw_status fx_gemm_f64(const FxOp &A, const FxOp &B, int F, double *out, size_t 
   g.ldo = ldo;
   g.dstatus = dstatus;
   return fx_run<true>(A, B, F, g, st);
-}
-
-void fx_scales(size_t n, const short *e, int F, double *scale, cudaStream_t st) {
-  if (!n) return;
-  k_fx_scales<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, e, F, scale);
-  epw_count_launch();
 }
 
 void fx_unpack_hermitian(int npt, int n, const double *in, cx<double> *out, cudaStream_t st) {

@@ -134,8 +134,5 @@ inline int fx_kb_split(int kpad) {  // 32-element K blocks per part
   return (kb + s - 1) / s;
 }
 inline int fx_splits(int kpad) { return (kpad / 32 + fx_kb_split(kpad) - 1) / fx_kb_split(kpad); }
-// scale[i] = 2^(e[i] - F), NaN for rows that are not finite
-void fx_scales(size_t n, const short *e, int F, double *scale, cudaStream_t st);
-
 // Unpacks the Hermitian matrices of fx_hermitian's rows: out[i][n][n] complex from in[i][n^2].
 void fx_unpack_hermitian(int npt, int n, const double *in, cx<double> *out, cudaStream_t st);

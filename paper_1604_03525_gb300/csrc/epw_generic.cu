@@ -226,10 +226,10 @@ __global__ void __launch_bounds__(128) k_vertex_fewk(int nk, int nR, int ncol, c
 // stored as (x, x, -y, y) and (x, y, y, x) a complex product takes two instructions, in the order and
 // with the roundings of cfma, so the sums equal k_cgemm's bit for bit.  Alone, 249 x 95,616: 37 k 341
 // -> 284 us, 256 k 1.31 -> 1.12 ms; 135 x 6480, 21 k 33 -> 19 us.  Bound by the shared-memory reads
-// (59 % of the FMA rate).
-template <int TM>
+// (59 % of the FMA rate).  G: g as the model holds it (cast on the way in) or its FP32 copy.
+template <int TM, typename G>
 __global__ void __launch_bounds__(128) k_vertex32(int nk, int nR, int ncol, const cx<float> *__restrict__ P,
-                                                  const cx<float> *__restrict__ g, cx<float> *G1) {
+                                                  const cx<G> *__restrict__ g, cx<float> *G1) {
   constexpr int TK = 16, MI = TM / 8;
   __shared__ float4 As[TK][TM + 1], Bs[TK][64];  // (+1: the stores run down a column)
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;  // columns tx + 16 j, rows ty + 8 i
@@ -240,7 +240,8 @@ __global__ void __launch_bounds__(128) k_vertex32(int nk, int nR, int ncol, cons
 #pragma unroll
     for (int j = 0; j < 4; j++) c[i][j] = make_float2(0.0f, 0.0f);
   constexpr int NA = TK * TM / 128, NB = TK * 64 / 128;
-  cx<float> ra[NA], rb[NB];
+  cx<float> ra[NA];
+  cx<G> rb[NB];
   auto fetch = [&](int k0) {
 #pragma unroll
     for (int t = 0; t < NA; t++) {
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(128) k_vertex32(int nk, int nR, int ncol, cons
 #pragma unroll
     for (int t = 0; t < NB; t++) {
       const int e = threadIdx.x + 128 * t, nn = e % 64, kk = e / 64;
-      rb[t] = (n0 + nn < ncol && k0 + kk < nR) ? g[(size_t)(k0 + kk) * ncol + n0 + nn] : mkc(0.0f, 0.0f);
+      rb[t] = (n0 + nn < ncol && k0 + kk < nR) ? g[(size_t)(k0 + kk) * ncol + n0 + nn] : mkc<G>(0, 0);
     }
   };
   fetch(0);
@@ -263,7 +264,8 @@ __global__ void __launch_bounds__(128) k_vertex32(int nk, int nR, int ncol, cons
 #pragma unroll
     for (int t = 0; t < NB; t++) {
       const int e = threadIdx.x + 128 * t;
-      Bs[e / 64][e % 64] = make_float4(rb[t].x, rb[t].y, rb[t].y, rb[t].x);
+      const cx<float> b = ccast<float>(rb[t]);
+      Bs[e / 64][e % 64] = make_float4(b.x, b.y, b.y, b.x);
     }
     __syncthreads();
     if (k0 + TK < nR) fetch(k0 + TK);
@@ -1095,8 +1097,7 @@ __global__ void k_eliashberg(int nq, int nm, const double *__restrict__ omega, c
 
 // gw[Re][Rp][...] = wRe wRp g   (g complex128 or, with is_c64, complex64)
 __global__ void k_set_vertex(int nRe, int nRp, size_t per, const void *__restrict__ g, int is_c64,
-                             const double *__restrict__ wRe, const double *__restrict__ wRp, cx<double> *gw,
-                             cx<float> *gw32) {
+                             const double *__restrict__ wRe, const double *__restrict__ wRp, cx<double> *gw) {
   size_t n = (size_t)nRe * nRp * per;
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n; idx += (size_t)gridDim.x * blockDim.x) {
     size_t rr = idx / per;
@@ -1111,7 +1112,6 @@ __global__ void k_set_vertex(int nRe, int nRp, size_t per, const void *__restric
       im = ((const double *)g)[2 * idx + 1];
     }
     gw[idx] = mkc(s * re, s * im);
-    gw32[idx] = mkc((float)(s * re), (float)(s * im));
   }
 }
 
@@ -1255,13 +1255,14 @@ __global__ void k_dg_scale(int nRe, int nRp, size_t per, const double *__restric
 
 // ------------------------------------------------------------------ launchers
 void launch_phases(int npt, const double *x, int nR, const int *R, int rmax, cx<double> *rm, cx<double> *T64,
-                   cx<float> *T32, cudaStream_t st) {
+                   cx<float> *T32, cudaStream_t st, bool exact) {
   size_t n = (size_t)npt * nR;
   if (!n) return;
   // FP64 instructions per thread (sincospi about 45) times waves of the 608 x 32 lanes: one thread
   // per point pays off once the points fill the GPU (1000 k x 135 R: 200 us against 10)
   const double w1 = std::max(1.0, npt / 19456.0), wn = std::max(1.0, (double)n / 19456.0);
-  if (rmax <= PH_RMAX && (3.0 * (2 * rmax + 1) * 45.0 + 8.0 * nR) * w1 < 52.0 * wn)
+  const bool fact = exact ? nR >= 2 * (2 * PH_RMAX + 1) : (3.0 * (2 * rmax + 1) * 45.0 + 8.0 * nR) * w1 < 52.0 * wn;
+  if (rmax <= PH_RMAX && fact)
     k_phases_fact<<<(npt + 127) / 128, 128, 0, st>>>(npt, x, nR, R, rmax < 0 ? 0 : rmax, rm, T64, T32);
   else
     k_phases<<<nblocks(n, 256), 256, 0, st>>>(npt, x, nR, R, rm, T64, T32);
@@ -1269,10 +1270,10 @@ void launch_phases(int npt, const double *x, int nR, const int *R, int rmax, cx<
 }
 
 void launch_fourier_d(int npt, int nR, const cx<double> *PT, const cx<double> *X, int msize, cx<double> *out,
-                      cudaStream_t st) {
+                      cudaStream_t st, bool exact) {
   size_t n = (size_t)npt * msize;
   if (!n) return;
-  if (n <= 65536)
+  if (n <= 65536 && !exact)
     k_fourier_few<<<(unsigned)((n * 8 + 127) / 128), 128, 0, st>>>(npt, nR, PT, X, msize, out);
   else
     k_fourier_d<<<nblocks(n, 256), 256, 0, st>>>(npt, nR, PT, X, msize, out);
@@ -1300,15 +1301,20 @@ template void launch_cgemm<double>(int, int, int, const cx<double> *, int, bool,
 template void launch_cgemm<float>(int, int, int, const cx<float> *, int, bool, bool, const cx<float> *, int,
                                   cx<float> *, int, bool, cudaStream_t);
 
-void launch_vertex32(int nk, int nR, int ncol, const cx<float> *P, const cx<float> *g, cx<float> *G1,
+// Up to 64 k read g once: straight from FP64.  More k read it once per 64: from an FP32 copy in g32.
+void launch_vertex32(int nk, int nR, int ncol, const cx<float> *P, const cx<double> *g, cx<float> *g32, cx<float> *G1,
                      cudaStream_t st) {
   if (nk <= 0 || ncol <= 0) return;
   const int nb = (ncol + 63) / 64;
   // 64 k per tile read the shared operands half as often, also with padding (37 k: 284 us against 336)
-  if (nk > 32)
-    k_vertex32<64><<<dim3(nb, (nk + 63) / 64), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
-  else
-    k_vertex32<32><<<dim3(nb, (nk + 31) / 32), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  if (nk > 64) {
+    launch_cast_c64_to_c32((size_t)nR * ncol, g, g32, st);
+    k_vertex32<64, float><<<dim3(nb, (nk + 63) / 64), 128, 0, st>>>(nk, nR, ncol, P, g32, G1);
+  } else if (nk > 32) {
+    k_vertex32<64, double><<<dim3(nb, 1), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  } else {
+    k_vertex32<32, double><<<dim3(nb, 1), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  }
   epw_count_launch();
 }
 
@@ -1513,7 +1519,7 @@ void launch_set_vertex(const epw_model *m, const void *g, int is_c64, cudaStream
   size_t per = (size_t)m->nm * m->nw * m->nw;
   size_t n = (size_t)m->nRe * m->nRp * per;
   if (!n) return;
-  k_set_vertex<<<nblocks(n, 256), 256, 0, st>>>(m->nRe, m->nRp, per, g, is_c64, m->wRe, m->wRp, m->gw, m->gw32);
+  k_set_vertex<<<nblocks(n, 256), 256, 0, st>>>(m->nRe, m->nRp, per, g, is_c64, m->wRe, m->wRp, m->gw);
   epw_count_launch();
 }
 

@@ -39,7 +39,7 @@ struct Prep {
   double *omegaT;          // [nm][nq]
   void *ET;                // [nm*nm][nq] working precision
   void *G1, *Bg, *BH;      // working precision
-  cx<float> *Pk32;         // FP32 copy for the k-side contraction
+  cx<float> *Pk32, *gw32;  // FP32 copies for the k-side contraction
   void *Cpol;              // [nm][nq] long-range factors C_nu(q), working precision (polar models)
 };
 
@@ -48,6 +48,7 @@ struct Prep {
 struct Fx64 {
   bool dq;               // D(q) that way
   bool pair;             // the pairs' contractions that way
+  bool exact;            // phonons and bands at k to the bit of the CUDA cores' sums and jacobi_herm (launch_eigh_d)
   FxOp Aph, Phi;         // q phases of the Rph set, force constants
   double *Dh;            // [nq][nm^2] (fx_hermitian's rows)
   FxOp Ae, Ap;           // q phases of the Re and Rp sets (Aph's planes where the sets agree)

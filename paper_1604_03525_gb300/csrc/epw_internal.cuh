@@ -318,7 +318,6 @@ struct epw_model {
   cx<double> *Phiw;       // [nRph][nm][nm], wRph and 1/sqrt(M M') folded
   float4 *Phidf;          // Phiw in double-float: (Re hi, Re lo, Im hi, Im lo) per entry
   cx<double> *gw;         // [nRe][nRp][nm][nw][nw], wRe wRp folded
-  cx<float> *gw32;        // the same in FP32 (the k-side vertex of the FP32 and split forms)
   double *mass;           // [nat]
   double *exptab;         // [EPW_EXPTAB] 2^(-j/EPW_EXPTAB), for the FP64 per-pair kernels
   unsigned int *dstatus;  // device status word
@@ -371,17 +370,21 @@ void epw_count_launch();
 // ------------------------------------------------------------- kernels
 // Generic SIMT path (epw_generic.cu)
 // rmax: the largest |R component| of the set (one-axis factors when small)
+// exact: the form (products of one-axis factors or each R by itself) by nR alone
 void launch_phases(int npt, const double *x, int nR, const int *R, int rmax, cx<double> *out_rowmajor,
-                   cx<double> *out_T, cx<float> *out_T32, cudaStream_t st);
+                   cx<double> *out_T, cx<float> *out_T32, cudaStream_t st, bool exact = false);
+// exact: the sums over R in one chain, as for many points
 void launch_fourier_d(int npt, int nR, const cx<double> *P, const cx<double> *X, int msize, cx<double> *out,
-                      cudaStream_t st);
-void launch_eigh_d(int nmat, int n, cx<double> *A, double *w, cx<double> *V, unsigned *dstatus, cudaStream_t st);
+                      cudaStream_t st, bool exact = false);
+// exact: jacobi_herm's rotations to the bit
+void launch_eigh_d(int nmat, int n, cx<double> *A, double *w, cx<double> *V, unsigned *dstatus, cudaStream_t st,
+                   bool exact = false);
 void launch_phonon_post(int nq, int nm, const double *w2, const cx<double> *ev, const double *mass, double omega_min,
                         double *omegaT, cx<double> *ET64, cx<float> *ET32, double *omega_out, cudaStream_t st);
 template <typename R>
 void launch_cgemm(int M, int N, int K, const cx<R> *A, int lda, bool transA, bool conjA, const cx<R> *B, int ldb,
                   cx<R> *C, int ldc, bool accumulate, cudaStream_t st);
-void launch_vertex32(int nk, int nR, int ncol, const cx<float> *P, const cx<float> *g, cx<float> *G1,
+void launch_vertex32(int nk, int nR, int ncol, const cx<float> *P, const cx<double> *g, cx<float> *g32, cx<float> *G1,
                      cudaStream_t st);
 void launch_vertex_fewk(int nk, int nR, int ncol, const cx<double> *P, const cx<double> *g, cx<double> *G1,
                         cudaStream_t st);

@@ -168,8 +168,12 @@ __global__ void __launch_bounds__(128) k_adj32(PairArgs a) {
           const float nb_ = occ_bose<float>(w, a.T);
           const double dn = (double)nb_ * ((double)nb_ + 1.0) * (double)w * ikT2;
           Wv = (float)(c * ((double)(nb_ + f) * dp + (double)(nb_ + 1.0f - f) * dm));
-          const double g2 = (double)cabs2(g[v]);
-          const double dd = (double)gauss_diff_r<float>(x, w, inv_sigma, gnorm);
+          // (cabs2 and gauss_diff_r with their fused products written out: dL/dT and dL/dE_F cancel, and
+          // round as k_pair's do)
+          const double g2 = (double)fmaf(g[v].x, g[v].x, __fmul_rn(g[v].y, g[v].y));
+          const float as = x * inv_sigma, bs = w * inv_sigma, y2 = 2.0f * as * bs;
+          const double dd = fabsf(y2) > 1.0f ? dp - dm
+                                             : -2.0f * gnorm * expf(-fmaf(as, as, __fmul_rn(bs, bs))) * sinhf(y2);
           tT = fma(g2, dn * ((double)dp + (double)dm) + dfT * dd, tT);
           tE = fma(g2, dfE * dd, tE);
         }

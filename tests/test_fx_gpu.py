@@ -102,3 +102,63 @@ def test_kside_vertex_forms_agree(epw, nw, nRe, nRp, nk):
     for i in {0, nk // 2, nk - 1}:
         one = m.linewidth(k[i:i + 1], q, **par)
         assert np.abs(all_k[i] - one[0]).max() < 1e-12 * np.abs(one).max()
+
+
+@pytest.mark.parametrize("lat,nw,nat,nRe,nRp,nk,nq", [("sc", 1, 1, 27, 81, 9000, 33), ("fcc", 4, 1, 120, 79, 700, 7),
+                                                      ("hex", 5, 3, 57, 93, 40, 33), ("diamond", 8, 2, 55, 87, 30, 9)])
+def test_phonons(epw, oracle_lib, lat, nw, nat, nRe, nRp, nk, nq):
+    """Warps of 32 q around a full and a nearly empty one, few and many k per warp.  Pi'' cancels between
+    terms of both signs: relative to its largest entry."""
+    wm, rng = _model(lat, nw, nat, nRe, nRp)
+    k, q = rng.random((nk, 3)), rng.random((nq, 3))
+    wk = rng.random(nk) / nk
+    ref = oracle_lib.phonon_self(wm, k, q, wk, 300.0, 0.1, 0.1)
+    m = epw.Model(wm)
+    got = m.phonon_selfenergy(k, q, wk, T=300.0, EF=0.1, sigma=0.1, precision=epw.FP64)
+    m.sync()
+    assert np.abs(got[0] - ref[0]).max() < 1e-9 * np.abs(ref[0]).max()
+    assert _rel(got[1], ref[1]) < 1e-9 and _rel(got[2], ref[2]) < 1e-9
+
+
+@pytest.mark.parametrize("nq", [2047, 2049, 4099])
+def test_gradient_of_a_long_q_list(epw, nq):
+    """The adjoint's sum over q in one part and in several (each part has its own fixed point): the
+    gradient over the list against the sum over pieces of at most 700 q."""
+    wm, rng = _model("fcc", 4, 1, 43, 19)
+    k, q = rng.random((3, 3)), rng.random((nq, 3))
+    wq, cot = rng.random(nq) / nq, rng.random((3, 4))
+    m = epw.Model(wm)
+    par = dict(T=300.0, EF=0.1, sigma=0.1, precision=epw.FP64)
+    got = m.linewidth_backward(k, q, cot, wq, **par)
+    ref = [sum(x) for x in zip(*(m.linewidth_backward(k, q[i:i + 700], cot, wq[i:i + 700], **par)
+                                 for i in range(0, nq, 700)))]
+    m.sync()
+    for a, b in zip(got, ref):
+        assert np.abs(a - b).max() < 1e-9 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("nk,nq", [(1, 2000), (3, 257), (20, 129)])
+def test_interpolation_of_a_list(epw, oracle_lib, nk, nq):
+    wm, rng = _model("fcc", 4, 1, 120, 79)
+    k, q = rng.random((nk, 3)), rng.random((nq, 3))
+    ek, ekq, om, g = epw.Model(wm).interp(k, q)
+    rk, rkq, rom, rg = oracle_lib.interp(wm, k, q)
+    assert _rel(ek, rk) < 1e-9 and _rel(ekq, rkq) < 1e-9 and _rel(om, rom) < 1e-9
+    # |g|^2 summed over the bands at k + q and the modes does not depend on the eigenvectors' phases
+    a, b = ((np.abs(x) ** 2).sum(axis=(2, 3)) for x in (g, rg))
+    assert _rel(a, b) < 1e-9
+
+
+@pytest.mark.parametrize("nw,nat,nRe,nRp", [(1, 1, 27, 19), (4, 1, 79, 43), (5, 3, 33, 57)])
+@pytest.mark.parametrize("nk", [32, 33, 64, 65, 130])
+def test_kside_vertex_fp32(epw, nw, nat, nRe, nRp, nk):
+    """The FP32 k-side vertex over its tiles (32 and 64 k, g in FP64 and as an FP32 copy): each k alone
+    and in the list, within the FP32 form's tolerance."""
+    wm, rng = _model("hex", nw, nat, nRe, nRp)
+    k, q = rng.random((nk, 3)), rng.random((150, 3))
+    m = epw.Model(wm)
+    par = dict(T=300.0, EF=0.0, sigma=0.3, precision=epw.FP32)
+    all_k = m.linewidth(k, q, **par)
+    for i in {0, 31, nk - 1}:
+        one = m.linewidth(k[i:i + 1], q, **par)
+        assert np.abs(all_k[i] - one[0]).max() < 2e-3 * np.abs(one).max()
