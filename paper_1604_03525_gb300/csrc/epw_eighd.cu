@@ -7,7 +7,8 @@
 // warps per SM at 76).  So the cost of a rotation is its FP64 instruction count, and a matrix
 // that fills only some lanes of a warp wastes the rest:
 //   - rotation parameters from three reciprocal square roots (about 7 instructions each)
-//     instead of three square roots and three divisions (about 57): jrot_d;
+//     instead of three square roots and three divisions (about 57): jrot_d (not with X: 13,824 of
+//     9 x 9 3.2 ms against 2.4);
 //   - few matrices: L lanes per matrix, each taking rows of A and of V (k_eigh_coop), so a
 //     rotation costs 12 ceil((2n-2)/L) instructions beside its parameters instead of 12 (2n-2);
 //   - many matrices: one thread per matrix, in registers for n <= 6 (k_eigh_reg).

@@ -10,7 +10,8 @@
 //     one of a mode's three Gaussians) are listed per warp and taken 32 at a time;
 //   - Xbar is row-major over q (zeroed before), each term adding its column's entries in memory:
 //     the terms that a warp handles between two barriers differ in (pair, n).
-// It is bound by the listed terms' FP64 sums and by Xbar's traffic.
+// It is bound by the listed terms' FP64 sums and by Xbar's traffic: hex nw = 5, 9 modes, 216 k x 13,824 q
+// 9.1 ms (82 with every term).
 #include "epw_internal.cuh"
 
 namespace {
