@@ -22,6 +22,8 @@
 // which keeps the shared-memory reads (96 KB per 896 cycles) below the 128 B/cycle limit.  448 of
 // the 512 columns are used, so the accumulators are not doubled; the epilogue (8 warps) reads
 // them into 64-bit registers and hands them back before it converts or stores anything.
+// Measured: diamond nw = 8, 24 k x 8000 q 3.0 ms, 76 % of the BF16 peak in digit products; fcc nw = 4,
+// 125 k x 13,824 q 2.5 ms, 61 %.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

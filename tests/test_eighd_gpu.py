@@ -54,3 +54,19 @@ def test_linewidth_does_not_depend_on_the_count(epw, nat, nq):
     w[nq - 1] = 1.0
     one = m.linewidth(k, q[nq - 1:], **par)
     assert np.abs(m.linewidth(k, q, w, **par) - one).max() < 1e-11 * np.abs(one).max()
+
+
+@pytest.mark.parametrize("nat", range(1, 7))
+@pytest.mark.parametrize("n", [1, 700, 25000])
+def test_both_kinds_of_rotations(epw, nat, n):
+    """The FP32 form takes its FP64 phonons and bands from jacobi_herm's rotations, the FP64 form from
+    the cheaper ones: omega^2 and e_k agree to 1e-12 of the largest (a few n ulp each)."""
+    rng = np.random.default_rng(170 + nat)
+    wm = W.make_model("fcc", 3 * nat, nat, [1.0 + 0.1 * i for i in range(nat)], 13, 13, rng)
+    m = epw.Model(wm)
+    x, one = rng.random((n, 3)), rng.random((1, 3))
+    for k, q in ((one, x), (x, one)):
+        a, b = (m.interp(k, q, precision=p, want_g=False) for p in (epw.FP32, epw.FP64))
+        assert np.abs(a[0] - b[0]).max() < 1e-12 * np.abs(b[0]).max()
+        wa, wb = (np.sign(w[2]) * w[2] ** 2 for w in (a, b))
+        assert np.abs(wa - wb).max() < 1e-12 * np.abs(wb).max()
