@@ -673,7 +673,7 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   if (!qs && fx && fx->dq) {
     CKS(run_fx_q(m, nq, q, *fx, p.D, sq, pa && *pa->done ? pa : nullptr));
   } else if (!qs) {
-    launch_fourier_d(nq, m->nRph, p.PqTph, m->Phiw, nm * nm, p.D, sq);
+    launch_fourier_d(nq, m->nRph, p.PqTph, m->Phiw, nm * nm, p.D, sq, exact);
   }
   // The eigensolves are one long wave of FP64-bound warps that has to start on a GPU with room on every
   // SM: launched while a GEMM fills it, their blocks share the few SMs that happen to have room

@@ -20,9 +20,10 @@
 
 namespace {
 
-// X: jacobi_herm's arithmetic to the bit (three square roots and divisions, its order of products):
-// for the FP32 adjoint, whose gradient is summed and rounded in FP32, so that one phonon that is
-// cast to FP32 the other way moves a few percent of its entries by a last place.
+// X: jacobi_herm's arithmetic to the bit (three square roots and divisions, its order of products, of a
+// product's imaginary part the second term fused), whatever the number of matrices: for the FP32 adjoint,
+// whose gradient is summed and rounded in FP32, so that one phonon that is cast to FP32 the other way
+// moves a few percent of its entries by a last place.
 //
 // The rotation that zeroes a_pq: c, (sx, sy) = s a_pq/|a_pq|, and the new diagonal.  With theta =
 // (aqq - app) / (2 |a_pq|) and h = 1/sqrt(1 + theta^2): c^2 = (1 + |theta| h) / 2, s = sign(theta) h
@@ -60,15 +61,21 @@ __device__ __forceinline__ void jrot_d(double &app, double &aqq, double ax, doub
   }
 }
 
+// off + |a|^2 (X: jacobi_herm's roundings; a sweep more or less is a last place of every entry)
+template <bool X>
+__device__ __forceinline__ double joff_d(double off, double2 a) {
+  return X ? off + fma(a.x, a.x, __dmul_rn(a.y, a.y)) : fma(a.x, a.x, fma(a.y, a.y, off));
+}
+
 // (u, v) <- (c u - conj(se) v, se u + c v), se = sx + i sy
 template <bool X>
 __device__ __forceinline__ void jrow_d(double c, double sx, double sy, double2 &u, double2 &v) {
   const double2 a = u, b = v;
   if constexpr (X) {
     u.x = fma(c, a.x, -fma(sx, b.x, __dmul_rn(sy, b.y)));
-    u.y = fma(c, a.y, -fma(sx, b.y, -__dmul_rn(sy, b.x)));
+    u.y = fma(c, a.y, -fma(-sy, b.x, __dmul_rn(sx, b.y)));
     v.x = fma(c, b.x, fma(sx, a.x, -__dmul_rn(sy, a.y)));
-    v.y = fma(c, b.y, fma(sx, a.y, __dmul_rn(sy, a.x)));
+    v.y = fma(c, b.y, fma(sy, a.x, __dmul_rn(sx, a.y)));
   } else {
     u.x = fma(-sx, b.x, fma(-sy, b.y, c * a.x));
     u.y = fma(-sx, b.y, fma(sy, b.x, c * a.y));
@@ -105,7 +112,7 @@ __global__ void __launch_bounds__(64) k_eigh_reg(int nmat, const double2 *__rest
     for (int i = 0; i < N; i++) {
       dg = fma(d[i], d[i], dg);
 #pragma unroll
-      for (int j = i + 1; j < N; j++) off = fma(A[i][j].x, A[i][j].x, fma(A[i][j].y, A[i][j].y, off));
+      for (int j = i + 1; j < N; j++) off = joff_d<X>(off, A[i][j]);
     }
     done = off <= jacobi_tol<double>::tol2 * (dg + 2.0 * off);
     if (done || sweep == jacobi_tol<double>::maxsweep) break;
@@ -179,7 +186,7 @@ __global__ void __launch_bounds__(64) k_eigh_loc(int nmat, const double2 *__rest
     for (int i = 0; i < N; i++) {
       dg = fma(d[i], d[i], dg);
 #pragma unroll 1
-      for (int j = i + 1; j < N; j++) off = fma(A[i][j].x, A[i][j].x, fma(A[i][j].y, A[i][j].y, off));
+      for (int j = i + 1; j < N; j++) off = joff_d<X>(off, A[i][j]);
     }
     done = off <= jacobi_tol<double>::tol2 * (dg + 2.0 * off);
     if (done || sweep == jacobi_tol<double>::maxsweep) break;
@@ -249,12 +256,24 @@ __global__ void __launch_bounds__(EC_WARPS * 32) k_eigh_coop(int nmat, int n, co
     for (int i = l; i < n; i += L) {
       const double x = A[i * n + i].x;
       dg = fma(x, x, dg);
-      for (int j = i + 1; j < n; j++) off = fma(A[i * n + j].x, A[i * n + j].x, fma(A[i * n + j].y, A[i * n + j].y, off));
+      for (int j = i + 1; j < n; j++) off = joff_d<X>(off, A[i * n + j]);
     }
 #pragma unroll
     for (int o = L / 2; o > 0; o >>= 1) {
       off += __shfl_xor_sync(0xffffffffu, off, o);
       dg += __shfl_xor_sync(0xffffffffu, dg, o);
+    }
+    if constexpr (X) {
+      // the lanes' sums come in another order than jacobi_herm's (n^2 / 2 roundings of 2^-53): where that could
+      // decide, its order
+      const double thr = jacobi_tol<double>::tol2 * (dg + 2.0 * off);
+      if (fabs(off - thr) <= 1e-12 * thr) {
+        off = dg = 0.0;
+        for (int i = 0; i < n; i++) {
+          dg = fma(A[i * n + i].x, A[i * n + i].x, dg);
+          for (int j = i + 1; j < n; j++) off = joff_d<X>(off, A[i * n + j]);
+        }
+      }
     }
     done = off <= jacobi_tol<double>::tol2 * (dg + 2.0 * off);
     if (__all_sync(0xffffffffu, done) || sweep == jacobi_tol<double>::maxsweep) break;

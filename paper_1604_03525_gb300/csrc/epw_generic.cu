@@ -88,6 +88,23 @@ __global__ void k_fourier_few(int npt, int nR, const cx<double> *__restrict__ PT
   if (in && l == 0) out[(size_t)i * msize + e] = acc;
 }
 
+// k_fourier_d's sum to the bit (one chain over r) for few elements: two lanes per element, one for the
+// real and one for the imaginary part, so that a lane's chain is 2 nR dependent FMAs instead of 4 nR.
+__global__ void __launch_bounds__(64) k_fourier_chain(int npt, int nR, const cx<double> *__restrict__ PT,
+                                                      const cx<double> *__restrict__ X, int msize, double *out) {
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, idx = t >> 1;
+  if (idx >= (size_t)npt * msize) return;
+  const bool im = t & 1;
+  const int i = (int)(idx % npt), e = (int)(idx / npt);
+  double acc = 0.0;
+#pragma unroll 8
+  for (int r = 0; r < nR; r++) {
+    const cx<double> p = PT[(size_t)r * npt + i], x = X[(size_t)r * msize + e];
+    acc = fma(p.x, im ? x.y : x.x, fma(im ? p.y : -p.y, im ? x.x : x.y, acc));
+  }
+  out[2 * ((size_t)i * msize + e) + (im ? 1 : 0)] = acc;
+}
+
 // out[i][e] = sum_r PT[r][i] X[r][e]   (PT transposed phases [nR][npt])
 __global__ void k_fourier_d(int npt, int nR, const cx<double> *__restrict__ PT, const cx<double> *__restrict__ X,
                             int msize, cx<double> *out) {
@@ -1275,6 +1292,8 @@ void launch_fourier_d(int npt, int nR, const cx<double> *PT, const cx<double> *X
   if (!n) return;
   if (n <= 65536 && !exact)
     k_fourier_few<<<(unsigned)((n * 8 + 127) / 128), 128, 0, st>>>(npt, nR, PT, X, msize, out);
+  else if (n <= 65536)
+    k_fourier_chain<<<(unsigned)((n * 2 + 63) / 64), 64, 0, st>>>(npt, nR, PT, X, msize, (double *)out);
   else
     k_fourier_d<<<nblocks(n, 256), 256, 0, st>>>(npt, nR, PT, X, msize, out);
   epw_count_launch();
