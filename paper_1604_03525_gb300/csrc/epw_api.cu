@@ -435,6 +435,12 @@ static void plan_prep(Arena &A, const epw_model *m, int nk, int nq, int prec, bo
 static double fp64_us(double per_thread, double threads) {
   return per_thread * 0.032 * std::max(1.0, threads / (32.0 * 608.0));
 }
+// FP32 and split forms: below this many q the phonons come from the CUDA cores' sums and jacobi_herm's
+// rotations to the bit as well (Fx64::exact): one mode factor that is cast to FP32 the other way moves a
+// linewidth by about 6e-8 / nq, so short lists have nothing to average it over and little to gain.
+static const int EXACT_NQ = 2048;
+static bool exact_q(int prec, int nq) { return prec != EPW_FP64 && nq < EXACT_NQ; }
+
 // D(q) as digit planes costs two passes over them and about 30 us of launches; the CUDA cores
 // take 4 nR nm^2 FP64 instructions per q (316,000 q of 249 R and 6 modes: 18.6 ms).
 static bool fx_dq(const epw_model *m, int nq) {
@@ -638,6 +644,10 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   const int nw = m->nw, nm = m->nm;
   const size_t nw2 = (size_t)nw * nw;
   const bool exact = fx && fx->exact;
+  // The k side of the FP32 and split forms, always: it is cast to FP32 and split, and a value that is cast
+  // the other way moves every q of its k alike (one in about 50 lists of 256 k of the diamond model; 4e-8
+  // of the linewidths of that k).
+  const bool exact_k = exact || prec != EPW_FP64;
   cudaStream_t sq = st;
   fork = fork && nq > 0 && nk > 0;
   if (fork) {
@@ -681,7 +691,7 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   // them where it runs on the tensor cores (FP64), and they start after it where it runs on the CUDA
   // cores, which they slow down threefold (FP32: 809 us beside 9001 of 6 x 6, 284 alone); the kernels
   // after that vertex wait until they are launched (13,824 of 9 x 9 among them: 16.8 ms).
-  const bool gate = fork && fx && (fx->dq || exact);
+  const bool gate = fork && fx && (fx->dq || (exact && nq >= EXACT_NQ));
   const bool after_vertex = gate && need_B && prec != EPW_FP64;
   if (gate) CK(cudaEventRecord(m->ev_gate, sq));
   auto q_tail = [&]() {
@@ -702,7 +712,7 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   // k side (FP64): phases, H(k), eigensolve, then the k-side vertex; with a fork the
   // bands (H(k), eigensolve) run on a third stream beside the vertex GEMM, which
   // needs only the phases, and are joined before the U_k rotation
-  launch_phases(nk, k, m->nRe, m->Re, m->rmax, p.PkRM, p.PkT, nullptr, st, exact);
+  launch_phases(nk, k, m->nRe, m->Re, m->rmax, p.PkRM, p.PkT, nullptr, st, exact_k);
   const bool fork2 = fork && need_B;
   cudaStream_t sk = st;
   if (fork2) {
@@ -710,8 +720,8 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
     CK(cudaStreamWaitEvent(m->aux2, m->ev_fork2, 0));
     sk = m->aux2;
   }
-  launch_fourier_d(nk, m->nRe, p.PkT, m->Hw, (int)nw2, p.Hk, sk, exact);
-  launch_eigh_d(nk, nw, p.Hk, p.epsk, p.Uk, m->dstatus, sk, exact);
+  launch_fourier_d(nk, m->nRe, p.PkT, m->Hw, (int)nw2, p.Hk, sk, exact_k);
+  launch_eigh_d(nk, nw, p.Hk, p.epsk, p.Uk, m->dstatus, sk, exact_k);
   if (fork2) CK(cudaEventRecord(m->ev_join2, sk));
   if (need_B && nk > 0) {
     const int ncol = m->nRp * nm * (int)nw2;
@@ -839,7 +849,9 @@ static epw_status plan_linewidth_pass(Arena &A, const epw_model *m, int nk, int 
   L.tc = TcBuffers{};
   L.w = TcwBuffers{};
   const bool narrow = tc && tc_supported(m);
-  plan_fx(A, m, nk, nq, !tune.simt64 && !narrow && fx_dq(m, nq), tune.pair64, tune.g1_64, L.fx);
+  const bool ex = exact_q(prec, nq);
+  plan_fx(A, m, nk, nq, !tune.simt64 && !narrow && !ex && fx_dq(m, nq), tune.pair64, tune.g1_64, L.fx);
+  L.fx.exact = ex;
   plan_prep(A, m, nk, nq, tc ? EPW_FP32 : prec, false, sq, swq, true, L.p, &L.fx);
   if (narrow) {
     CKS(tc_plan(A, m, nk, nq, op, L.tc));
@@ -1033,7 +1045,7 @@ static epw_status linewidth_pass(epw_model *m, int nk, const double *kd, int nq,
   if (tcp && !L.tc.ok && !L.sg.ok && !L.w.ok)
     return fail(EPW_ERR_UNSUPPORTED, "no tensor-core form for nw=%d, 3nat=%d", m->nw, m->nm);
   if (tcp && L.tc.ok) {
-    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, &L.tc));
+    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, &L.tc, &L.fx));
     L.tc.Cpol = m->polar ? (const float2 *)p.Cpol : nullptr;
     L.tc.Uk64 = p.Uk;
     L.tc.Pq64 = m->same_eph ? p.PqTph : nullptr;
@@ -1777,8 +1789,10 @@ extern "C" epw_status epw_selfenergy(const epw_model *mc, int nk, const double *
   } b;
   bool fx_on = true;
   auto plan = [&](Arena &A) -> epw_status {
-    plan_fx(A, m, nk, std::max(nq, 1), fx_on && fx_dq(m, nq), false,
+    const bool ex = exact_q(wprec, nq);
+    plan_fx(A, m, nk, std::max(nq, 1), fx_on && !ex && fx_dq(m, nq), false,
             fx_on && wprec == EPW_FP64 && nq > 0 && fx_g1(m, nk), b.fx);
+    b.fx.exact = ex;
     plan_prep(A, m, nk, std::max(nq, 1), wprec, sk, sq, swq, true, b.p, &b.fx);
     b.sg = TcStaged{};
     if (tcp) {
@@ -1989,7 +2003,7 @@ extern "C" epw_status epw_linewidth_noalloc(const epw_model *mc, int nk, const d
   A = Arena{scratch, (size_t)EPW_NOALLOC_SCRATCH_BYTES, 0};
   CKS(epwi_plan_linewidth(A, m, nk, nq, prec, false, false, false, false, tune, L));
   Prep &p = L.p;
-  CKS(run_prep(m, nk, k, nq, q, prec, par->omega_min_eV, true, p, nullptr, st, /*fork=*/false));
+  CKS(run_prep(m, nk, k, nq, q, prec, par->omega_min_eV, true, p, nullptr, st, /*fork=*/false, nullptr, &L.fx));
   PairArgs a;
   std::memset(&a, 0, sizeof(a));
   a.nk = nk;

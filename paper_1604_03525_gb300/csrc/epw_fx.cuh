@@ -59,21 +59,20 @@ __device__ __forceinline__ void fx_phase_digits(double c, double s, uint32_t (&p
   fx_digits2(__double2ll_rn(c * 36028797018963968.0), __double2ll_rn(s * 36028797018963968.0), p);  // 2^55
 }
 
-constexpr int FX_PRMAX = 8;   // largest |R_j| of the factor table
 constexpr int FX_PPB = 16;    // points per block
 struct FxFactors {
-  double2 f[FX_PPB][3][2 * FX_PRMAX + 1];
+  double2 f[FX_PPB][3][2 * PH_RMAX + 1];
 };
 // Phases e^{2 pi i x.R} of a block's FX_PPB points: the one-axis factors e^{2 pi i (x_j n mod 1)},
 // n = 1..rmax (n < 0: the conjugate), one per thread, then a warp per point, lanes over R (contiguous
-// K on the way out) up to `half` (0 beyond nR).  rmax > FX_PRMAX: the phase of each R by itself.
+// K on the way out) up to `half` (0 beyond nR).  rmax > PH_RMAX: the phase of each R by itself.
 // row(point, finite) once per point, put(point, r, cos, sin) for every r.  Blocks of 128 threads.
 template <class ROW, class PUT>
 __device__ __forceinline__ void fx_point_phases(int npt, const double *__restrict__ x, int nR,
                                                 const int *__restrict__ R, int rmax, int half, FxFactors &F, ROW row,
                                                 PUT put) {
   const int p0 = blockIdx.x * FX_PPB, np = min(FX_PPB, npt - p0);
-  const bool fact = rmax <= FX_PRMAX;
+  const bool fact = rmax <= PH_RMAX;
   if (fact) {
     const int per = 3 * (rmax + 1);
     for (int t = threadIdx.x; t < np * per; t += 128) {
@@ -82,8 +81,8 @@ __device__ __forceinline__ void fx_point_phases(int npt, const double *__restric
       a -= rint(a);
       double s, c;
       sincospi(2.0 * a, &s, &c);
-      F.f[p][j][FX_PRMAX + n] = make_double2(c, s);
-      F.f[p][j][FX_PRMAX - n] = make_double2(c, -s);
+      F.f[p][j][PH_RMAX + n] = make_double2(c, s);
+      F.f[p][j][PH_RMAX - n] = make_double2(c, -s);
     }
   }
   __syncthreads();
@@ -97,11 +96,11 @@ __device__ __forceinline__ void fx_point_phases(int npt, const double *__restric
       double c = 0.0, s = 0.0;
       if (r < nR && fin) {
         if (fact) {
-          const double2 f0 = F.f[p][0][R[3 * r] + FX_PRMAX], f1 = F.f[p][1][R[3 * r + 1] + FX_PRMAX],
-                        f2 = F.f[p][2][R[3 * r + 2] + FX_PRMAX];
-          const double2 f = make_double2(fma(f0.x, f1.x, -f0.y * f1.y), fma(f0.x, f1.y, f0.y * f1.x));
-          c = fma(f.x, f2.x, -f.y * f2.y);
-          s = fma(f.x, f2.y, f.y * f2.x);
+          const double2 f0 = F.f[p][0][R[3 * r] + PH_RMAX], f1 = F.f[p][1][R[3 * r + 1] + PH_RMAX],
+                        f2 = F.f[p][2][R[3 * r + 2] + PH_RMAX];
+          const cx<double> f = phase_product(mkc(f0.x, f0.y), mkc(f1.x, f1.y), mkc(f2.x, f2.y));
+          c = f.x;
+          s = f.y;
         } else {
           double a = q0 * R[3 * r] + q1 * R[3 * r + 1] + q2 * R[3 * r + 2];
           a -= rint(a);

@@ -43,7 +43,6 @@ __global__ void k_phases(int npt, const double *__restrict__ x, int nR, const in
 // the factors for R_j in [-rmax, rmax] (rmax <= PH_RMAX, the largest |R_j| of the set)
 // formed once per point (FP64 argument reduction, sincospi), then two complex
 // products per R.  One thread per point.
-constexpr int PH_RMAX = 8;
 __global__ void k_phases_fact(int npt, const double *__restrict__ x, int nR, const int *__restrict__ R, int rmax,
                               cx<double> *rowmajor, cx<double> *T64, cx<float> *T32) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -61,10 +60,33 @@ __global__ void k_phases_fact(int npt, const double *__restrict__ x, int nR, con
   }
   for (int r = 0; r < nR; r++) {
     const cx<double> f0 = F[0][R[3 * r] + PH_RMAX], f1 = F[1][R[3 * r + 1] + PH_RMAX], f2 = F[2][R[3 * r + 2] + PH_RMAX];
-    const cx<double> f01 = mkc(f0.x * f1.x - f0.y * f1.y, f0.x * f1.y + f0.y * f1.x);
-    const cx<double> p = mkc(f01.x * f2.x - f01.y * f2.y, f01.x * f2.y + f01.y * f2.x);
+    const cx<double> p = phase_product(f0, f1, f2);
     if (rowmajor) rowmajor[(size_t)i * nR + r] = p;
     const size_t idx = (size_t)r * npt + i;
+    if (T64) T64[idx] = p;
+    if (T32) T32[idx] = mkc((float)p.x, (float)p.y);
+  }
+}
+
+// k_phases_fact's phases to the bit, one thread per (point, R): three factors and two products each, for
+// few points, where a thread per point is one long chain (1000 k x 135 R: 200 us).  For the k side of the
+// FP32 and split forms, whose casts must not depend on the number of k.
+__global__ void k_phases_prod(int npt, const double *__restrict__ x, int nR, const int *__restrict__ R,
+                              cx<double> *rowmajor, cx<double> *T64, cx<float> *T32) {
+  const size_t n = (size_t)npt * nR;
+  for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n; idx += (size_t)gridDim.x * blockDim.x) {
+    const int i = (int)(idx % npt), r = (int)(idx / npt);
+    cx<double> f[3];
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+      double a = x[3 * (size_t)i + j] * R[3 * r + j];
+      a -= rint(a);
+      double s, c;
+      sincospi(2.0 * a, &s, &c);
+      f[j] = mkc(c, s);
+    }
+    const cx<double> p = phase_product(f[0], f[1], f[2]);
+    if (rowmajor) rowmajor[(size_t)i * nR + r] = p;
     if (T64) T64[idx] = p;
     if (T32) T32[idx] = mkc((float)p.x, (float)p.y);
   }
@@ -1278,8 +1300,12 @@ void launch_phases(int npt, const double *x, int nR, const int *R, int rmax, cx<
   // FP64 instructions per thread (sincospi about 45) times waves of the 608 x 32 lanes: one thread
   // per point pays off once the points fill the GPU (1000 k x 135 R: 200 us against 10)
   const double w1 = std::max(1.0, npt / 19456.0), wn = std::max(1.0, (double)n / 19456.0);
-  const bool fact = exact ? nR >= 2 * (2 * PH_RMAX + 1) : (3.0 * (2 * rmax + 1) * 45.0 + 8.0 * nR) * w1 < 52.0 * wn;
-  if (rmax <= PH_RMAX && fact)
+  const double cost1 = (3.0 * (2 * rmax + 1) * 45.0 + 8.0 * nR) * w1;
+  if (exact && !ph_factors(nR, rmax))
+    k_phases<<<nblocks(n, 256), 256, 0, st>>>(npt, x, nR, R, rm, T64, T32);
+  else if (exact && 150.0 * wn < cost1)
+    k_phases_prod<<<nblocks(n, 128), 128, 0, st>>>(npt, x, nR, R, rm, T64, T32);
+  else if (exact || (rmax <= PH_RMAX && cost1 < 52.0 * wn))
     k_phases_fact<<<(npt + 127) / 128, 128, 0, st>>>(npt, x, nR, R, rmax < 0 ? 0 : rmax, rm, T64, T32);
   else
     k_phases<<<nblocks(n, 256), 256, 0, st>>>(npt, x, nR, R, rm, T64, T32);

@@ -57,6 +57,16 @@ __host__ __device__ __forceinline__ R cabs2(cx<R> a) { return a.x * a.x + a.y * 
 template <typename R, typename S>
 __host__ __device__ __forceinline__ cx<R> ccast(cx<S> a) { return mkc((R)a.x, (R)a.y); }
 
+// f0 f1 f2 of the one-axis factors of a phase, the fused products written out, so that every kernel that
+// forms it rounds alike.
+__device__ __forceinline__ cx<double> phase_product(cx<double> f0, cx<double> f1, cx<double> f2) {
+  const cx<double> p = mkc(fma(f0.x, f1.x, -__dmul_rn(f0.y, f1.y)), fma(f0.y, f1.x, __dmul_rn(f0.x, f1.y)));
+  return mkc(fma(p.x, f2.x, -__dmul_rn(p.y, f2.y)), fma(p.y, f2.x, __dmul_rn(p.x, f2.y)));
+}
+constexpr int PH_RMAX = 8;  // largest |R_j| of the factor tables
+// The formula of phases that are cast to FP32 or split: factors, or each R by itself for a small set.
+inline bool ph_factors(int nR, int rmax) { return rmax <= PH_RMAX && nR >= 2 * (2 * PH_RMAX + 1); }
+
 // ------------------------------------------------------------ occupations
 // Bose-Einstein n(w) = 1/(e^{w/kT} - 1); T <= 0 gives 0.
 __device__ __forceinline__ double bose_d(double w, double T) {
@@ -370,7 +380,7 @@ void epw_count_launch();
 // ------------------------------------------------------------- kernels
 // Generic SIMT path (epw_generic.cu)
 // rmax: the largest |R component| of the set (one-axis factors when small)
-// exact: the form (products of one-axis factors or each R by itself) by nR alone
+// exact: the formula (products of one-axis factors or each R by itself) by the R set alone (ph_factors)
 void launch_phases(int npt, const double *x, int nR, const int *R, int rmax, cx<double> *out_rowmajor,
                    cx<double> *out_T, cx<float> *out_T32, cudaStream_t st, bool exact = false);
 // exact: the sums over R in one chain, as for many points

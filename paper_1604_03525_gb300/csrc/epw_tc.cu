@@ -1579,6 +1579,7 @@ void tc_phases_a(int op, int nq, const double *q, int nR, const int *R, int rmax
   if (nq <= 0) return;
   const size_t plane = (size_t)o.rows * o.kpad;
   const int grid = (nq + FX_PPB - 1) / FX_PPB;
+  if (!ph_factors(nR, rmax)) rmax = PH_RMAX + 1;  // each R by itself, as in the operand from FP64 phases
   if (op == TC_OP_BF16)
     k_phases_a<__nv_bfloat16><<<grid, 128, 0, st>>>(nq, q, nR, R, rmax, o.kpad, plane, o.d, o.e, kpad,
                                                     (__nv_bfloat16 *)hi, (__nv_bfloat16 *)lo);
