@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -467,9 +468,10 @@ static const size_t FX_GW_BYTES = (size_t)2 << 30;
 // Contraction chunk of the FP64 form.
 static const size_t FX_CT_BYTES = (size_t)2 << 30;
 
-// more: further bytes per k of a chunk (the adjoint's and the interpolation's buffers).
+// more: further bytes per k of a chunk (the adjoint's and the interpolation's buffers); kmax: most k of a
+// chunk (the adjoint sums over its k in one fixed point).
 static void plan_fx(Arena &A, const epw_model *m, int nk, int nq, bool dq, bool pair, bool g1, Fx64 &f,
-                    size_t more = 0) {
+                    size_t more = 0, int kmax = INT_MAX) {
   f = Fx64{};
   f.dq = dq || pair;
   f.pair = pair;
@@ -492,7 +494,8 @@ static void plan_fx(Arena &A, const epw_model *m, int nk, int nq, bool dq, bool 
   f.ldc = (size_t)(nq + 127) / 128 * 128;
   const size_t cols = nw2 * (1 + 2 * (size_t)m->nm);
   const size_t kplanes = 2 * FX_S * nw2 * ((size_t)fx_kpad(m->nRe) + 2 * (size_t)m->nm * fx_kpad(m->nRp));
-  f.kc = (int)std::min<size_t>((size_t)nk, std::max<size_t>(1, FX_CT_BYTES / (cols * f.ldc * 8 + kplanes + more)));
+  f.kc = (int)std::min<size_t>((size_t)std::min(nk, kmax),
+                               std::max<size_t>(1, FX_CT_BYTES / (cols * f.ldc * 8 + kplanes + more)));
   f.BH = fx_plan(A, f.kc * nw2, fx_kpad(m->nRe), true);
   f.BG = fx_plan(A, f.kc * nw2 * 2 * m->nm, fx_kpad(m->nRp), true);
   f.CH = A.take<long long>(f.kc * nw2 * f.ldc);
@@ -1371,7 +1374,8 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
     pair64 = fx_on && prec == EPW_FP64 && nk > 0 && nq > 0 && fx_pair(m, nk, nq);
     plan_fx(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, fx_on && prec == EPW_FP64 && fx_dq(m, nq), pair64,
             fx_on && prec == EPW_FP64 && nk > 0 && fx_g1(m, nk), b.fx,
-            per * ((size_t)nq * 16 + 2 * FX_S * (size_t)kpq + 16 * (size_t)fx_splits(kpq) * m->nRp + 16 * (size_t)m->nRp));
+            per * ((size_t)nq * 16 + 2 * FX_S * (size_t)kpq + 16 * (size_t)fx_splits(kpq) * m->nRp + 16 * (size_t)m->nRp),
+            FX_KMAX / 2);
     b.fx.exact = prec != EPW_FP64;
     plan_prep(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, prec, sk, sq, swq, true, b.p, &b.fx);
     b.cotd = scot ? A.take<double>((size_t)nk * m->nw) : (double *)cot;
@@ -1464,7 +1468,7 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
       gk.kpad = pk.kpad = fx_kpad(kc);
       fx_rows(m->nRp * per, kc, kc, b.G1b, gk, st);
       fx_phases_conj(kc, kd + 3 * (size_t)k0, m->nRe, m->Re, pk, st);
-      CKS(fx_gemm_f64(gk, pk, fx_bits(std::min(kc, FX_KMAX / 2)), (double *)b.gT, 2 * (size_t)m->nRe, m->dstatus, st,
+      CKS(fx_gemm_f64(gk, pk, fx_bits(kc), (double *)b.gT, 2 * (size_t)m->nRe, m->dstatus, st,
                       k0 > 0));
     }
   } else if (nk > 0 && nq > 0 && tcb) {

@@ -28,6 +28,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "epw_fx.cuh"
 #include "epw_tc.cuh"
@@ -530,6 +531,8 @@ epw_status fx_run(const FxOp &A, const FxOp &B, int F, FxArgs &g, cudaStream_t s
   g.kblocks = A.kpad / FX_BK;
   g.kb_split = g.ostride ? fx_kb_split(A.kpad) : g.kblocks;
   g.splits = (g.kblocks + g.kb_split - 1) / g.kb_split;
+  // a part of n complex terms sums to at most sqrt(2) n 2^F in units of the row scales: within 63 bits
+  if (1.5 * (FX_BK / 2) * std::min(g.kblocks, g.kb_split) > std::ldexp(1.0, 63 - F)) return EPW_ERR_UNSUPPORTED;
   g.shift_hi = F - 38;  // hi counts 2^-38, lo 2^-62
   g.shift_lo = 62 - F;
   g.eA = A.e;
