@@ -3,7 +3,6 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
-#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -469,9 +468,10 @@ static const size_t FX_GW_BYTES = (size_t)2 << 30;
 static const size_t FX_CT_BYTES = (size_t)2 << 30;
 
 // more: further bytes per k of a chunk (the adjoint's and the interpolation's buffers); kmax: most k of a
-// chunk (the adjoint sums over its k in one fixed point).
+// chunk (the adjoint sums over its k in one fixed point; the kernels have k on the grid's second axis).
+static const int FX_KC_MAX = 65535;
 static void plan_fx(Arena &A, const epw_model *m, int nk, int nq, bool dq, bool pair, bool g1, Fx64 &f,
-                    size_t more = 0, int kmax = INT_MAX) {
+                    size_t more = 0, int kmax = FX_KC_MAX) {
   f = Fx64{};
   f.dq = dq || pair;
   f.pair = pair;

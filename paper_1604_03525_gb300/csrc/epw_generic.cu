@@ -1368,6 +1368,11 @@ void launch_vertex_fewk(int nk, int nR, int ncol, const cx<double> *P, const cx<
                         cudaStream_t st) {
   if (nk <= 0 || ncol <= 0) return;
   const int nb = (ncol + 127) / 128;
+  if (nk > 65535) {  // k is on the grid's second axis
+    launch_vertex_fewk(65535, nR, ncol, P, g, G1, st);
+    launch_vertex_fewk(nk - 65535, nR, ncol, P + (size_t)65535 * nR, g, G1 + (size_t)65535 * ncol, st);
+    return;
+  }
   if (nk >= 4 && (long)nb * ((nk + 3) / 4) >= 608)
     k_vertex_fewk<4><<<dim3(nb, (nk + 3) / 4), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
   else if (nk >= 3 && nb >= 304)
