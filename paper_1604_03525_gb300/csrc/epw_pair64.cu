@@ -875,14 +875,14 @@ __global__ void __launch_bounds__(256) k_g64(Pair64Args a) {
   }
 }
 
-// One thread per (aj, Rp) (Rp contiguous in B), looping over k.
+// One thread per (k, aj, Rp), Rp contiguous in B.
 __global__ void k_adj_rotate64(int nk, int k0, int nRp, int nm, int nw, int splits, size_t stride,
                                const double *__restrict__ B, const cx<double> *__restrict__ Uk, cx<double> *G1) {
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   const int naj = nm * nw;
   if (t >= (size_t)naj * nRp) return;
   const int r = (int)(t % nRp), aj = (int)(t / nRp);
-  for (int k = 0; k < nk; k++) {
+  for (int k = blockIdx.y; k < nk; k += gridDim.y) {
     double2 b[EPW_MAX_NW];
     for (int n = 0; n < nw; n++) {
       const double *s = B + ((size_t)k * naj * nw + (size_t)aj * nw + n) * 2 * nRp + 2 * r;
@@ -1008,7 +1008,8 @@ epw_status launch_g64(const Pair64Args &a, cudaStream_t st) {
 void launch_adj_rotate64(int nk, int k0, int nRp, int nm, int nw, int splits, size_t stride, const double *B,
                          const cx<double> *Uk, cx<double> *G1, cudaStream_t st) {
   const size_t n = (size_t)nm * nw * nRp;
-  k_adj_rotate64<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(nk, k0, nRp, nm, nw, splits, stride, B, Uk, G1);
+  if (nk <= 0) return;
+  k_adj_rotate64<<<dim3((unsigned)((n + 127) / 128), nk < 65535 ? nk : 65535), 128, 0, st>>>(nk, k0, nRp, nm, nw, splits, stride, B, Uk, G1);
   epw_count_launch();
 }
 
