@@ -352,23 +352,35 @@ extern "C" int epw_abi_version(void) { return EPW_ABI_VERSION; }
 // -------------------------------------------------------------- workspace
 static epw_status ensure_ws(epw_model *m, size_t bytes) {
   if (bytes <= m->ws_bytes) return EPW_OK;
+  size_t avail = 0, total = 0;
+  CK(cudaMemGetInfo(&avail, &total));
+  // what would not fit even in place of the old workspace leaves that one where it is
+  if (bytes > avail + m->ws_bytes)
+    return fail(EPW_ERR_OOM, "workspace of %zu bytes: %zu are free", bytes, avail + m->ws_bytes);
   CK(cudaDeviceSynchronize());
   if (m->ws) cudaFree(m->ws);
   m->ws = nullptr;
   m->ws_bytes = 0;
-  size_t b = bytes + bytes / 8 + (1 << 20);
-  CK(cudaMalloc(&m->ws, b));
-  m->ws_bytes = b;
-  return EPW_OK;
+  for (size_t b : {bytes + bytes / 8 + (1 << 20), bytes}) {  // with room to grow, if there is any
+    const cudaError_t e = cudaMalloc(&m->ws, b);
+    if (e == cudaSuccess) {
+      m->ws_bytes = b;
+      return EPW_OK;
+    }
+    m->ws = nullptr;
+    cudaGetLastError();
+    if (e != cudaErrorMemoryAllocation) return fail(EPW_ERR_CUDA, "workspace: %s", cudaGetErrorString(e));
+  }
+  return fail(EPW_ERR_OOM, "workspace of %zu bytes: out of memory", bytes);
 }
 
 // The fixed-point forms take more workspace than the CUDA cores' (digit planes, the contractions of at
-// least one k over all q).  Plans beyond this keep the CUDA cores' form, so that a q list of any
-// length that fits the device without them still does (18 bands, 18 modes: 93 KB a q and k).
+// least one k over all q; 18 bands, 18 modes: 93 KB a q and k).  Plans beyond this, or beyond what the device
+// has left, keep the CUDA cores' form, so that a q list of any length that fits without them still does.
 static const size_t FX_WS_BYTES = (size_t)64 << 30;
 
 // Plans a call's workspace (plan(A), twice: its size, then its pointers).  The fixed-point forms are
-// taken (fx_on) while the whole plan stays within FX_WS_BYTES.
+// taken (fx_on) while the whole plan stays within FX_WS_BYTES and can be allocated.
 template <class PLAN>
 static epw_status plan_ws(epw_model *m, Arena &A, const Fx64 &fx, bool &fx_on, PLAN plan) {
   A = Arena{nullptr, 0, 0};
@@ -378,7 +390,15 @@ static epw_status plan_ws(epw_model *m, Arena &A, const Fx64 &fx, bool &fx_on, P
     A = Arena{nullptr, 0, 0};
     CKS(plan(A));
   }
-  CKS(ensure_ws(m, A.off));
+  epw_status s = ensure_ws(m, A.off);
+  if (s == EPW_ERR_OOM && fx_on && (fx.dq || fx.g1)) {
+    fx_on = false;
+    A = Arena{nullptr, 0, 0};
+    CKS(plan(A));
+    s = ensure_ws(m, A.off);
+    if (s == EPW_OK) g_err[0] = 0;
+  }
+  CKS(s);
   A = Arena{(char *)m->ws, m->ws_bytes, 0};
   return plan(A);
 }
@@ -932,13 +952,26 @@ static epw_status plan_linewidth(Arena &A, const epw_model *m, int nk, int nq, i
   return epwi_plan_linewidth(A, m, nk, nq, prec, sk, sq, swq, sout, epwi_default_tune(), L);
 }
 
+// The plan of a linewidth call and its workspace; with tune.simt64 where the fixed-point forms' would not fit
+// the device.
+static epw_status plan_linewidth_ws(epw_model *m, int nk, int nq, int prec, bool sk, bool sq, bool swq, bool sout,
+                                    EpwTune &tune, LwPlan &L) {
+  for (tune = epwi_default_tune();; tune.simt64 = true) {
+    Arena A{nullptr, 0, 0};
+    CKS(epwi_plan_linewidth(A, m, nk, nq, prec, sk, sq, swq, sout, tune, L));
+    const epw_status s = ensure_ws(m, A.off);
+    if (s == EPW_ERR_OOM && (L.fx.dq || L.fx.g1)) continue;
+    if (s == EPW_OK) g_err[0] = 0;
+    return s;
+  }
+}
+
 extern "C" epw_status epw_reserve(epw_model *m, int nk, int nq, int precision) {
   CKS(check_common(m, nk, (const double *)1, nq, (const double *)1));
   if (precision < EPW_FP64 || precision > EPW_TF32X3) return fail(EPW_ERR_INVALID_ARG, "unknown precision");
-  Arena A{nullptr, 0, 0};
+  EpwTune tune;
   LwPlan L;
-  CKS(plan_linewidth(A, m, nk, nq, precision, true, true, true, true, L));
-  return ensure_ws(m, A.off);
+  return plan_linewidth_ws(m, nk, nq, precision, true, true, true, true, tune, L);
 }
 
 // Planning by shape alone: the same plan as epw_reserve on a host-side model that holds the
@@ -997,12 +1030,11 @@ extern "C" epw_status epw_linewidth(const epw_model *mc, int nk, const double *k
     CK(cudaMemsetAsync(imsigma, 0, sizeof(double) * (size_t)nk * m->nw, st));
     return EPW_OK;
   }
-  Arena A{nullptr, 0, 0};
+  EpwTune tune;
   LwPlan L;
-  CKS(plan_linewidth(A, m, nk, nq, prec, sk, sq, swq, sout, L));
-  CKS(ensure_ws(m, A.off));
-  A = Arena{(char *)m->ws, m->ws_bytes, 0};
-  CKS(plan_linewidth(A, m, nk, nq, prec, sk, sq, swq, sout, L));
+  CKS(plan_linewidth_ws(m, nk, nq, prec, sk, sq, swq, sout, tune, L));
+  Arena A{(char *)m->ws, m->ws_bytes, 0};
+  CKS(epwi_plan_linewidth(A, m, nk, nq, prec, sk, sq, swq, sout, tune, L));
   Prep &p = L.p;
   const double *kd = k, *qd = q, *wqd = wq;
   if (sk) {

@@ -157,15 +157,23 @@ epw_status tune_job(const epw_linewidth_job &j, int path, cudaStream_t st, EpwTu
   // shapes take seconds per trial over a 48^3 q grid)
   const int nk_t = std::min(j.nk, path == PATH_FUSED ? 608 : 16);
   size_t need = 0;
-  for (const EpwTune &t : cand) {
-    Arena A{nullptr, 0, 0};
-    LwPlan L;
-    BCKS(epwi_plan_linewidth(A, j.model, nk_t, j.nq, j.params.precision, false, false, false, false, t, L));
-    need = std::max(need, A.off);
-  }
   const size_t out_bytes = sizeof(double) * (size_t)nk_t * j.model->nw;
   char *ws = nullptr;
-  BCK(cudaMalloc((void **)&ws, need + out_bytes + 512));
+  bool simt64 = false;  // (the trials only: the choice is of tiles)
+  for (;; simt64 = true) {
+    need = 0;
+    for (EpwTune t : cand) {
+      Arena A{nullptr, 0, 0};
+      LwPlan L;
+      t.simt64 = simt64;
+      BCKS(epwi_plan_linewidth(A, j.model, nk_t, j.nq, j.params.precision, false, false, false, false, t, L));
+      need = std::max(need, A.off);
+    }
+    const cudaError_t e = cudaMalloc((void **)&ws, need + out_bytes + 512);
+    if (e == cudaSuccess) break;
+    if (e != cudaErrorMemoryAllocation || simt64) BCK(e);
+    cudaGetLastError();
+  }
   double *outp = (double *)(ws + ((need + 255) & ~size_t(255)));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaEventCreate(&e0);
@@ -175,7 +183,9 @@ epw_status tune_job(const epw_linewidth_job &j, int path, cudaStream_t st, EpwTu
   epw_status s = EPW_OK;
   for (size_t i = 0; i < cand.size() && s == EPW_OK; i++) {
     float ms = 0.0f;
-    s = trial(j, nk_t, cand[i], ws, need, outp, st, e0, e1, &ms);
+    EpwTune t = cand[i];
+    t.simt64 = simt64;
+    s = trial(j, nk_t, t, ws, need, outp, st, e0, e1, &ms);
     if (s == EPW_OK && (ib < 0 || ms < best)) {
       best = ms;
       ib = (int)i;
@@ -343,21 +353,33 @@ epw_status create_impl(int njobs, const epw_linewidth_job *jobs, epw_batch *b) {
   // another on one stream (every candidate graph maps regions onto branches), so they
   // share the region, which is as large as its largest job
   b->region = assign(b, MAX_BRANCHES);
-  std::vector<size_t> rsize(MAX_BRANCHES, 0), roff(MAX_BRANCHES, 0);
-  for (int j = 0; j < nj; j++) {
-    const epw_linewidth_job &J = b->jobs[j];
-    if (J.nk == 0 || J.nq == 0) continue;
-    Arena A{nullptr, 0, 0};
-    BCKS(epwi_plan_linewidth(A, J.model, J.nk, J.nq, J.params.precision, false, false, false, false, b->tunes[j],
-                             b->plans[j]));
-    rsize[b->region[j]] = std::max(rsize[b->region[j]], (A.off + 255) & ~size_t(255));
-  }
+  std::vector<size_t> rsize, roff;
   size_t total = 0;
-  for (int r = 0; r < MAX_BRANCHES; r++) {
-    roff[r] = total;
-    total += rsize[r];
+  // (with the CUDA cores' FP64 forms in a second attempt, where the fixed-point ones' workspace does not fit)
+  for (int attempt = 0;; attempt++) {
+    rsize.assign(MAX_BRANCHES, 0);
+    roff.assign(MAX_BRANCHES, 0);
+    for (int j = 0; j < nj; j++) {
+      const epw_linewidth_job &J = b->jobs[j];
+      if (J.nk == 0 || J.nq == 0) continue;
+      Arena A{nullptr, 0, 0};
+      BCKS(epwi_plan_linewidth(A, J.model, J.nk, J.nq, J.params.precision, false, false, false, false, b->tunes[j],
+                               b->plans[j]));
+      rsize[b->region[j]] = std::max(rsize[b->region[j]], (A.off + 255) & ~size_t(255));
+    }
+    total = 0;
+    for (int r = 0; r < MAX_BRANCHES; r++) {
+      roff[r] = total;
+      total += rsize[r];
+    }
+    if (!total) break;
+    const cudaError_t e = cudaMalloc((void **)&b->ws, total);
+    if (e == cudaSuccess) break;
+    b->ws = nullptr;
+    if (e != cudaErrorMemoryAllocation || attempt) BCK(e);
+    cudaGetLastError();
+    for (EpwTune &t : b->tunes) t.simt64 = true;
   }
-  if (total) BCK(cudaMalloc((void **)&b->ws, total));
   b->ws_bytes = total;
   for (int j = 0; j < nj; j++) {
     const epw_linewidth_job &J = b->jobs[j];
