@@ -410,6 +410,7 @@ static void plan_prep(Arena &A, const epw_model *m, int nk, int nq, int prec, bo
                       bool stage_wq, bool need_B, Prep &p, const Fx64 *fx = nullptr) {
   const size_t sR = rsize(prec);
   const size_t nw2 = (size_t)m->nw * m->nw, nm2 = (size_t)m->nm * m->nm;
+  p.bad = nullptr;
   p.kd = stage_k ? A.take<double>(3 * (size_t)nk) : nullptr;
   p.qd = stage_q ? A.take<double>(3 * (size_t)nq) : nullptr;
   p.wqd = stage_wq ? A.take<double>((size_t)nq) : nullptr;
@@ -765,7 +766,9 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
         CK(cudaStreamWaitEvent(st, m->ev_gate, 0));
       }
       if (fork2) CK(cudaStreamWaitEvent(st, m->ev_join2, 0));
-      launch_build_B<float>(m, nk, p.PkRM, (const cx<float> *)p.G1, p.Uk, (cx<float> *)p.Bg, (cx<float> *)p.BH, st);
+      if (p.bad) CK(cudaMemsetAsync(p.bad, 0, sizeof(int), st));
+      launch_build_B<float>(m, nk, p.PkRM, (const cx<float> *)p.G1, p.Uk, (cx<float> *)p.Bg, (cx<float> *)p.BH, st,
+                            p.bad);
     }
   }
   if (tcb && nk > 0 && nq > 0) {
@@ -1410,6 +1413,7 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
             FX_KMAX / 2);
     b.fx.exact = prec != EPW_FP64;
     plan_prep(A, m, nk > 0 ? nk : 1, nq > 0 ? nq : 1, prec, sk, sq, swq, true, b.p, &b.fx);
+    if (staged) b.p.bad = A.take<int>(1);
     b.cotd = scot ? A.take<double>((size_t)nk * m->nw) : (double *)cot;
     if (pair64) {
       const size_t kc = b.fx.kc, kpk = fx_kpad((int)kc);
@@ -1560,6 +1564,7 @@ extern "C" epw_status epw_linewidth_backward(const epw_model *mc, int nk, const 
         a.Cq = b.sg.Ct;
         a.ldc = b.sg.pair_ld();
         a.cpk = b.sg.cpk;
+        a.bad = p.bad;
       }
       if (staged) CK(cudaMemsetAsync(b.xbar, 0, sR * (size_t)nq * kc * per, st));
       epw_status s = staged ? launch_adj_staged(a, st)

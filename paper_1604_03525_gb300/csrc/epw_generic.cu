@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(128) k_vertex32(int nk, int nR, int ncol, cons
 // Bg[k][Rp][a][j][n] = sum_i G1[k][Rp][a][j][i] U_k[i][n];  BH[k][Re][i][j] = P_k(Re) Hw(Re)_ij
 template <typename R>
 __global__ void k_build_Bg(int nk, int nRp, int nm, int nw, const cx<R> *__restrict__ G1,
-                           const cx<double> *__restrict__ Uk, cx<R> *Bg) {
+                           const cx<double> *__restrict__ Uk, cx<R> *Bg, int *bad) {
   size_t n = (size_t)nk * nRp * nm * nw * nw;
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < n; idx += (size_t)gridDim.x * blockDim.x) {
     int nn = (int)(idx % nw);
@@ -347,6 +347,7 @@ __global__ void k_build_Bg(int nk, int nRp, int nm, int nw, const cx<R> *__restr
     cx<R> acc = mkc<R>(0, 0);
     for (int i = 0; i < nw; i++) cfma(acc, g[i], ccast<R>(U[i * nw + nn]));
     Bg[idx] = acc;
+    if (bad && !(fabs(acc.x) < R(1e15) && fabs(acc.y) < R(1e15))) atomicOr(bad, 1);
   }
 }
 
@@ -1384,10 +1385,10 @@ void launch_vertex_fewk(int nk, int nR, int ncol, const cx<double> *P, const cx<
 
 template <typename R>
 void launch_build_B(const epw_model *m, int nk, const cx<double> *Pk, const cx<R> *G1, const cx<double> *Uk,
-                    cx<R> *Bg, cx<R> *BH, cudaStream_t st) {
+                    cx<R> *Bg, cx<R> *BH, cudaStream_t st, int *bad) {
   size_t nbg = (size_t)nk * m->nRp * m->nm * m->nw * m->nw;
   if (nbg && Bg) {
-    k_build_Bg<R><<<nblocks(nbg, 256), 256, 0, st>>>(nk, m->nRp, m->nm, m->nw, G1, Uk, Bg);
+    k_build_Bg<R><<<nblocks(nbg, 256), 256, 0, st>>>(nk, m->nRp, m->nm, m->nw, G1, Uk, Bg, bad);
     epw_count_launch();
   }
   size_t nbh = (size_t)nk * m->nRe * m->nw * m->nw;
@@ -1397,9 +1398,9 @@ void launch_build_B(const epw_model *m, int nk, const cx<double> *Pk, const cx<R
   }
 }
 template void launch_build_B<double>(const epw_model *, int, const cx<double> *, const cx<double> *,
-                                     const cx<double> *, cx<double> *, cx<double> *, cudaStream_t);
+                                     const cx<double> *, cx<double> *, cx<double> *, cudaStream_t, int *);
 template void launch_build_B<float>(const epw_model *, int, const cx<double> *, const cx<float> *,
-                                    const cx<double> *, cx<float> *, cx<float> *, cudaStream_t);
+                                    const cx<double> *, cx<float> *, cx<float> *, cudaStream_t, int *);
 
 void launch_cast_c64_to_c32(size_t n, const cx<double> *in, cx<float> *out, cudaStream_t st) {
   if (!n) return;

@@ -41,6 +41,7 @@ struct Prep {
   void *G1, *Bg, *BH;      // working precision
   cx<float> *Pk32, *gw32;  // FP32 copies for the k-side contraction
   void *Cpol;              // [nm][nq] long-range factors C_nu(q), working precision (polar models)
+  int *bad;                // FP32 forms, or null: Bg holds entries that are not finite (or beyond 1e15)
 };
 
 // Fixed-point (tensor-core) contractions of the FP64 work: D(q) in every form, H(k+q) and

@@ -400,7 +400,7 @@ void launch_vertex_fewk(int nk, int nR, int ncol, const cx<double> *P, const cx<
                         cudaStream_t st);
 template <typename R>
 void launch_build_B(const epw_model *m, int nk, const cx<double> *Pk, const cx<R> *G1, const cx<double> *Uk,
-                    cx<R> *Bg, cx<R> *BH, cudaStream_t st);
+                    cx<R> *Bg, cx<R> *BH, cudaStream_t st, int *bad = nullptr);
 void launch_cast_c64_to_c32(size_t n, const cx<double> *in, cx<float> *out, cudaStream_t st);
 
 struct PairArgs {
@@ -428,6 +428,7 @@ struct PairArgs {
   const float *Cq;
   size_t ldc;
   int cpk;
+  const int *bad;  // staged adjoint: nonzero, the vertex holds entries that are not finite
   int nk_total;  // phonon side: all k-points of the call (the 1/nk weight when wq (= w_k) is null)
   // long-range vertex: g_nu += i C_nu(q) (U_k+q^dagger U_k), C [nm][nq] (R precision), U_k FP64 [nk][nw][nw]
   const void *Cpol;

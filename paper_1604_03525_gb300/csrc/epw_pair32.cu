@@ -22,6 +22,7 @@ template <int W>
 struct A32Warp {
   cx<float> u[W][32];  // each lane's current eigenvector
   float em[32];
+  bool all[32];          // every term, also those whose Gaussians are zero
   unsigned short list[32 * W];
 };
 
@@ -61,6 +62,9 @@ __global__ void __launch_bounds__(128) k_adj32(PairArgs a) {
   if (nc && valid) atomicOr(a.dstatus, EPW_DEV_NOT_CONVERGED);
 
   const double *ek = a.eps_k + (size_t)k * n, *cot = a.cot + (size_t)k * n;
+  // a vertex, weight or cotangent that is not finite shows in every term, zero Gaussians too
+  bool all = *a.bad != 0 || (a.wq && !isfinite(a.wq[q]));
+  for (int j = 0; j < n; j++) all |= !isfinite(cot[j]);
   const float inv_sigma = (float)(1.0 / a.sigma);
   const float gnorm = (float)(1.0 / (a.sigma * 1.7724538509055160273));
   const double kT = EPW_KB * a.T, ikT2 = 1.0 / (kT * a.T), ikT = 1.0 / kT, inq = 1.0 / nq;
@@ -69,8 +73,10 @@ __global__ void __launch_bounds__(128) k_adj32(PairArgs a) {
     const float w = (float)a.omegaT[(size_t)v * nq + q];
     if (w >= (float)a.omega_min && w > 0.0f) wmax = fmaxf(wmax, w);
   }
-  // (a band or a vertex that is not a number reaches everything)
-  const float thr = !valid ? -1.0f : wmax >= 0.0f ? (wmax + A32_CUT * (float)a.sigma) * 1.00001f : -1.0f;
+  // (a band that is not a number reaches everything)
+  const float thr = !valid ? -1.0f
+                    : all ? __int_as_float(0x7f800000)
+                    : wmax >= 0.0f ? (wmax + A32_CUT * (float)a.sigma) * 1.00001f : -1.0f;
   unsigned need = 0;
 #pragma unroll UW
   for (int m = 0; m < W; m++) {
@@ -106,6 +112,7 @@ __global__ void __launch_bounds__(128) k_adj32(PairArgs a) {
       for (int i = 0; i < W; i++)
         if (i < n) sw.u[i][lane] = u[i];
       sw.em[lane] = em;
+      sw.all[lane] = all;
     }
     const int cnt = __popc(todo);
     int off = cnt;
@@ -157,6 +164,7 @@ __global__ void __launch_bounds__(128) k_adj32(PairArgs a) {
       const double ff = fermi_ff_d((double)em - a.EF, a.T);
       const double dfE = ff * ikT, dfT = ff * ((double)em - a.EF) * ikT2;
       const double c = cot[nb] * EPW_PI * (a.wq ? a.wq[qs] : inq);
+      const bool als = sw.all[sl];
       double tT = 0.0, tE = 0.0;
 #pragma unroll UM
       for (int v = 0; v < MM; v++) {
@@ -165,18 +173,18 @@ __global__ void __launch_bounds__(128) k_adj32(PairArgs a) {
         const bool keep = w >= (float)a.omega_min && w > 0.0f;
         const float dp = gauss_r<float>(x + w, inv_sigma, gnorm), dm = gauss_r<float>(x - w, inv_sigma, gnorm);
         float Wv = 0.0f;
-        if (keep && !(dp == 0.0f && dm == 0.0f)) {
-          const float nb_ = occ_bose<float>(w, a.T);
+        if (als || (keep && !(dp == 0.0f && dm == 0.0f))) {
+          const float nb_ = keep ? occ_bose<float>(w, a.T) : 0.0f;
           const double dn = (double)nb_ * ((double)nb_ + 1.0) * (double)w * ikT2;
-          Wv = (float)(c * ((double)(nb_ + f) * dp + (double)(nb_ + 1.0f - f) * dm));
+          Wv = (float)((keep ? c : 0.0) * ((double)(nb_ + f) * dp + (double)(nb_ + 1.0f - f) * dm));
           // (cabs2 and gauss_diff_r with their fused products written out: dL/dT and dL/dE_F cancel, and
           // round as k_pair's do)
           const double g2 = (double)fmaf(g[v].x, g[v].x, __fmul_rn(g[v].y, g[v].y));
           const float as = x * inv_sigma, bs = w * inv_sigma, y2 = 2.0f * as * bs;
           const double dd = fabsf(y2) > 1.0f ? dp - dm
                                              : -2.0f * gnorm * expf(-fmaf(as, as, __fmul_rn(bs, bs))) * sinhf(y2);
-          tT = fma(g2, dn * ((double)dp + (double)dm) + dfT * dd, tT);
-          tE = fma(g2, dfE * dd, tE);
+          tT = fma(g2, keep ? dn * ((double)dp + (double)dm) + dfT * dd : 0.0, tT);
+          tE = fma(g2, keep ? dfE * dd : 0.0, tE);
         }
         g[v] = (2.0f * Wv) * g[v];
       }

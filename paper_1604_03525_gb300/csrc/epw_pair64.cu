@@ -521,6 +521,14 @@ __device__ __forceinline__ void p64_terms(const Pair64Args &a, const Eig64<W, EX
   }
 }
 
+// Reach of a pair's terms: the largest kept frequency and a Gaussian's width; everything (all) where a
+// vertex or a weight that is not finite has to show in terms whose Gaussians are zero too.
+__device__ __forceinline__ double p64_threshold(const Pair64Args &a, bool valid, double wmax, bool all) {
+  if (!valid) return -1.0;
+  if (all) return __longlong_as_double(0x7ff0000000000000LL);
+  return __double2hiint(wmax) >= 0 ? wmax + P64_CUT * a.sigma : -1.0;
+}
+
 template <int W, bool EX, int MM>
 __global__ void __launch_bounds__(128, 2) k_lw64(Pair64Args a) {
   __shared__ double sh[4][W];
@@ -539,8 +547,7 @@ __global__ void __launch_bounds__(128, 2) k_lw64(Pair64Args a) {
   const bool conv = pair64_eig<W, EX>(a, kl, q, S);
   if (!conv && valid) atomicOr(a.dstatus, EPW_DEV_NOT_CONVERGED);
   const double wm = a.wmax[q];
-  double thr = valid && __double2hiint(wm) >= 0 ? wm + P64_CUT * a.sigma : -1.0;
-  if (thr >= 0.0 && *a.bad) thr = __longlong_as_double(0x7ff0000000000000LL);
+  const double thr = p64_threshold(a, valid, wm, *a.bad || (a.wq && !isfinite(a.wq[q])));
   double acc[W];
 #pragma unroll(W <= P64_REGW ? W : 1)
   for (int j = 0; j < W; j++) acc[j] = 0.0;
@@ -613,8 +620,9 @@ __global__ void __launch_bounds__(128, 2) k_adj64(Pair64Args a) {
   const bool conv = pair64_eig<W, EX>(a, kl, q, S);
   if (!conv && valid) atomicOr(a.dstatus, EPW_DEV_NOT_CONVERGED);
   const double wm = a.wmax[q];
-  double thr = valid && __double2hiint(wm) >= 0 ? wm + P64_CUT * a.sigma : -1.0;
-  if (thr >= 0.0 && *a.bad) thr = __longlong_as_double(0x7ff0000000000000LL);
+  bool all = *a.bad || (a.wq && !isfinite(a.wq[q]));
+  for (int j = 0; j < n; j++) all |= !isfinite(cot[j]);
+  const double thr = p64_threshold(a, valid, wm, all);
   P64Warp<W, MS> &sw = sws[warp];
   const int qw = qi - lane;
   double sT = 0.0, sE = 0.0;
@@ -632,8 +640,10 @@ __global__ void __launch_bounds__(128, 2) k_adj64(Pair64Args a) {
     for (int v = 0; v < MM; v++) {
       if (v >= nm) continue;
       const double w = a.omK[(size_t)v * a.nq + qs];
-      if (__double2hiint(w) < 0) {
-        g[v] = make_double2(0.0, 0.0);
+      if (__double2hiint(w) < 0) {  // left out (0 times a vertex that is not finite is not 0)
+        g[v] = make_double2(0.0 * g[v].x, 0.0 * g[v].y);
+        tT = fma(g[v].x, g[v].y, tT);
+        tE = fma(g[v].x, g[v].y, tE);
         continue;
       }
       const double nbv = a.nbT[(size_t)v * a.nq + qs];
@@ -707,8 +717,6 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
   const int n = EX ? W : a.nw, nm = EX ? MM : a.nm;
   P64Warp<W, MS, false> &sw = sws[warp];
   const double wm = a.wmax[q];
-  double thr = valid && __double2hiint(wm) >= 0 ? wm + P64_CUT * a.sigma : -1.0;
-  if (thr >= 0.0 && *a.bad) thr = __longlong_as_double(0x7ff0000000000000LL);
   double sp[MM], sl_[MM], sz = 0.0;
 #pragma unroll
   for (int v = 0; v < MM; v++) sp[v] = sl_[v] = 0.0;
@@ -728,10 +736,12 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
     const bool conv = pair64_eig<W, EX>(a, kl, q, S);
     if (!conv && valid) atomicOr(a.dstatus, EPW_DEV_NOT_CONVERGED);
     const double wk = a.wk ? a.wk[k] : 1.0 / a.nk_total;
+    const bool all = *a.bad || !isfinite(wk);
+    const double thr = p64_threshold(a, valid, wm, all);
     // nesting: (sum_n delta(e_nk - E_F)) (sum_m delta(e_mk+q - E_F))
     double zn = 0.0, zm = 0.0;
     for (int j = 0; j < n; j++) zn += dn_s[j];
-    if (zn != 0.0) {
+    if (zn != 0.0 || all) {
 #pragma unroll(W <= P64_REGW ? W : 1)
       for (int m = 0; m < W; m++) {
         if (m >= n) continue;
@@ -766,7 +776,7 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
             gs[v] = a.gnorm * exp64n(a.exptab, y * y);
             any += gs[v];
           }
-          if (any == 0.0 && !*a.bad) {
+          if (any == 0.0 && !all) {
 #pragma unroll
             for (int v = 0; v < 2 * MM; v++) r[v] = 0.0;
             return;
