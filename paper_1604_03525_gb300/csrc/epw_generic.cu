@@ -1008,11 +1008,10 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 && MW <= 4 ? 3 : 1) k_pair
   }
 }
 
-// Sum over the per-warp partials (fixed order, compensated) into Sigma_nk(omega_i) (the extra point
+// Sum over the per-warp partials (fixed order, every term compensated) into Sigma_nk(omega_i) (the extra point
 // omega = 0 into re0): a block takes 64 grid points of one (k, n), its four warp pairs a quarter of
-// the q-warps each.  Eight partials are added plainly, the groups compensated: the additions are FP64
-// instructions of 64 cycles, and one thread per point over all of them took 234 us for 21 k x 4 bands
-// x 202 points x 250 partials.
+// the q-warps each.  The additions are FP64 instructions of 64 cycles: one thread per point over all of
+// the partials took 234 us for 21 k x 4 bands x 202 points x 250 partials.
 __global__ void __launch_bounds__(256) k_se_finalize(int k0, int nw, int nqw, int nom,
                                                      const double2 *__restrict__ part, double2 *sig, double *re0) {
   __shared__ double sh[4][4][64];
@@ -1023,17 +1022,11 @@ __global__ void __launch_bounds__(256) k_se_finalize(int k0, int nw, int nqw, in
   const int per = (nqw + 3) / 4, j1 = min(nqw, (y + 1) * per);
   double sr = 0.0, cr = 0.0, si = 0.0, ci = 0.0;
   if (i <= nom)
-    for (int j = y * per; j < j1; j += 8) {
-      double2 g = make_double2(0.0, 0.0);
-#pragma unroll
-      for (int t = 0; t < 8; t++)
-        if (j + t < j1) {
-          const double2 v = base[(size_t)(j + t) * stride + i];
-          g.x += v.x;
-          g.y += v.y;
-        }
-      neumaier_add(sr, cr, g.x);
-      neumaier_add(si, ci, g.y);
+#pragma unroll 4
+    for (int j = y * per; j < j1; j++) {
+      const double2 v = base[(size_t)j * stride + i];
+      neumaier_add(sr, cr, v.x);
+      neumaier_add(si, ci, v.y);
     }
   sh[y][0][x] = sr;
   sh[y][1][x] = cr;
@@ -1188,14 +1181,14 @@ __global__ void __launch_bounds__(128) k_finalize_k(int nk, int nqb, int nw, con
   const int n = nqb * nw;
   const int per = ((n + 127) / 128) * 32;  // elements per warp, a multiple of 32
   const int j0 = warp * per, j1 = min(n, j0 + per);
-  // eight terms plainly, the groups compensated: the additions are FP64 instructions of 64 cycles
   double s = 0.0, c = 0.0;
   int j = j0 + lane;
-  for (; j + 224 < j1; j += 256) {
-    double x[8];
-#pragma unroll
-    for (int t = 0; t < 8; t++) x[t] = row[j + 32 * t];
-    neumaier_add(s, c, ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7])));
+  for (; j + 96 < j1; j += 128) {
+    const double x0 = row[j], x1 = row[j + 32], x2 = row[j + 64], x3 = row[j + 96];
+    neumaier_add(s, c, x0);
+    neumaier_add(s, c, x1);
+    neumaier_add(s, c, x2);
+    neumaier_add(s, c, x3);
   }
   for (; j < j1; j += 32) neumaier_add(s, c, row[j]);
   for (int o = 16; o >= nw; o >>= 1) {
