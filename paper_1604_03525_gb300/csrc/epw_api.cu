@@ -456,12 +456,6 @@ static void plan_prep(Arena &A, const epw_model *m, int nk, int nq, int prec, bo
 static double fp64_us(double per_thread, double threads) {
   return per_thread * 0.032 * std::max(1.0, threads / (32.0 * 608.0));
 }
-// FP32 and split forms: below this many q the phonons come from the CUDA cores' sums and jacobi_herm's
-// rotations to the bit as well (Fx64::exact): one mode factor that is cast to FP32 the other way moves a
-// linewidth by about 6e-8 / nq, so short lists have nothing to average it over and little to gain.
-static const int EXACT_NQ = 2048;
-static bool exact_q(int prec, int nq) { return prec != EPW_FP64 && nq < EXACT_NQ; }
-
 // D(q) as digit planes costs two passes over them and about 30 us of launches; the CUDA cores
 // take 4 nR nm^2 FP64 instructions per q (316,000 q of 249 R and 6 modes: 18.6 ms).
 static bool fx_dq(const epw_model *m, int nq) {
@@ -715,7 +709,7 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   // them where it runs on the tensor cores (FP64), and they start after it where it runs on the CUDA
   // cores, which they slow down threefold (FP32: 809 us beside 9001 of 6 x 6, 284 alone); the kernels
   // after that vertex wait until they are launched (13,824 of 9 x 9 among them: 16.8 ms).
-  const bool gate = fork && fx && (fx->dq || (exact && nq >= EXACT_NQ));
+  const bool gate = fork && fx && (fx->dq || exact);
   const bool after_vertex = gate && need_B && prec != EPW_FP64;
   if (gate) CK(cudaEventRecord(m->ev_gate, sq));
   auto q_tail = [&]() {
@@ -875,9 +869,7 @@ static epw_status plan_linewidth_pass(Arena &A, const epw_model *m, int nk, int 
   L.tc = TcBuffers{};
   L.w = TcwBuffers{};
   const bool narrow = tc && tc_supported(m);
-  const bool ex = exact_q(prec, nq);
-  plan_fx(A, m, nk, nq, !tune.simt64 && !narrow && !ex && fx_dq(m, nq), tune.pair64, tune.g1_64, L.fx);
-  L.fx.exact = ex;
+  plan_fx(A, m, nk, nq, !tune.simt64 && !narrow && fx_dq(m, nq), tune.pair64, tune.g1_64, L.fx);
   plan_prep(A, m, nk, nq, tc ? EPW_FP32 : prec, false, sq, swq, true, L.p, &L.fx);
   if (narrow) {
     CKS(tc_plan(A, m, nk, nq, op, L.tc));
@@ -1083,7 +1075,7 @@ static epw_status linewidth_pass(epw_model *m, int nk, const double *kd, int nq,
   if (tcp && !L.tc.ok && !L.sg.ok && !L.w.ok)
     return fail(EPW_ERR_UNSUPPORTED, "no tensor-core form for nw=%d, 3nat=%d", m->nw, m->nm);
   if (tcp && L.tc.ok) {
-    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, &L.tc, &L.fx));
+    CKS(run_prep(m, nk, kd, nq, qd, EPW_FP32, par->omega_min_eV, true, p, nullptr, st, true, &L.tc));
     L.tc.Cpol = m->polar ? (const float2 *)p.Cpol : nullptr;
     L.tc.Uk64 = p.Uk;
     L.tc.Pq64 = m->same_eph ? p.PqTph : nullptr;
@@ -1830,10 +1822,8 @@ extern "C" epw_status epw_selfenergy(const epw_model *mc, int nk, const double *
   } b;
   bool fx_on = true;
   auto plan = [&](Arena &A) -> epw_status {
-    const bool ex = exact_q(wprec, nq);
-    plan_fx(A, m, nk, std::max(nq, 1), fx_on && !ex && fx_dq(m, nq), false,
+    plan_fx(A, m, nk, std::max(nq, 1), fx_on && fx_dq(m, nq), false,
             fx_on && wprec == EPW_FP64 && nq > 0 && fx_g1(m, nk), b.fx);
-    b.fx.exact = ex;
     plan_prep(A, m, nk, std::max(nq, 1), wprec, sk, sq, swq, true, b.p, &b.fx);
     b.sg = TcStaged{};
     if (tcp) {
@@ -2044,7 +2034,7 @@ extern "C" epw_status epw_linewidth_noalloc(const epw_model *mc, int nk, const d
   A = Arena{scratch, (size_t)EPW_NOALLOC_SCRATCH_BYTES, 0};
   CKS(epwi_plan_linewidth(A, m, nk, nq, prec, false, false, false, false, tune, L));
   Prep &p = L.p;
-  CKS(run_prep(m, nk, k, nq, q, prec, par->omega_min_eV, true, p, nullptr, st, /*fork=*/false, nullptr, &L.fx));
+  CKS(run_prep(m, nk, k, nq, q, prec, par->omega_min_eV, true, p, nullptr, st, /*fork=*/false));
   PairArgs a;
   std::memset(&a, 0, sizeof(a));
   a.nk = nk;

@@ -111,18 +111,38 @@ __global__ void k_fourier_few(int npt, int nR, const cx<double> *__restrict__ PT
 }
 
 // k_fourier_d's sum to the bit (one chain over r) for few elements: two lanes per element, one for the
-// real and one for the imaginary part, so that a lane's chain is 2 nR dependent FMAs instead of 4 nR.
+// real and one for the imaginary part, so that a lane's chain is 2 nR dependent FMAs (65 cycles each)
+// instead of 4 nR.  The next R's operands are on their way in registers while these are summed.
 __global__ void __launch_bounds__(64) k_fourier_chain(int npt, int nR, const cx<double> *__restrict__ PT,
                                                       const cx<double> *__restrict__ X, int msize, double *out) {
+  constexpr int NB = 8;
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x, idx = t >> 1;
   if (idx >= (size_t)npt * msize) return;
   const bool im = t & 1;
   const int i = (int)(idx % npt), e = (int)(idx / npt);
   double acc = 0.0;
-#pragma unroll 8
-  for (int r = 0; r < nR; r++) {
-    const cx<double> p = PT[(size_t)r * npt + i], x = X[(size_t)r * msize + e];
-    acc = fma(p.x, im ? x.y : x.x, fma(im ? p.y : -p.y, im ? x.x : x.y, acc));
+  cx<double> p[NB], x[NB];
+  auto fetch = [&](int r0) {
+#pragma unroll
+    for (int u = 0; u < NB; u++)
+      if (r0 + u < nR) {
+        p[u] = PT[(size_t)(r0 + u) * npt + i];
+        x[u] = X[(size_t)(r0 + u) * msize + e];
+      }
+  };
+  fetch(0);
+  for (int r0 = 0; r0 < nR; r0 += NB) {
+    cx<double> cp[NB], cx_[NB];
+#pragma unroll
+    for (int u = 0; u < NB; u++) {
+      cp[u] = p[u];
+      cx_[u] = x[u];
+    }
+    if (r0 + NB < nR) fetch(r0 + NB);
+#pragma unroll
+    for (int u = 0; u < NB; u++)
+      if (r0 + u < nR)
+        acc = fma(cp[u].x, im ? cx_[u].y : cx_[u].x, fma(im ? cp[u].y : -cp[u].y, im ? cx_[u].x : cx_[u].y, acc));
   }
   out[2 * ((size_t)i * msize + e) + (im ? 1 : 0)] = acc;
 }
