@@ -356,7 +356,7 @@ __device__ __forceinline__ bool p64_reach(float ek, float em, float thr) {
 template <int W, bool EX, int MM>
 __device__ __forceinline__ void pair64_g(const Pair64Args &a, int kl, int q, int nb, const double2 (*u)[32], int sl,
                                          double2 (&g)[MM]) {
-  const int n = EX ? W : a.nw, nm = EX ? MM : a.nm;
+  const int n = EX ? W : a.nw, nm = MM <= 9 ? MM : a.nm;
   constexpr int UM = MM <= 9 ? MM : 1;
   const size_t c0 = (size_t)kl * 2 * nm * n * n + 2 * nb;
 #pragma unroll UM
@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(128, 2) k_lw64(Pair64Args a) {
   const int qi = blockIdx.x * 128 + threadIdx.x, kl = blockIdx.y, k = a.k0 + kl;
   const bool valid = qi < a.nq;
   const int q = valid ? qi : 0;  // lanes past the last q keep step with their warp
-  const int n = EX ? W : a.nw, nm = EX ? MM : a.nm;
+  const int n = EX ? W : a.nw, nm = MM <= 9 ? MM : a.nm;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const double *ek = a.eps_k + (size_t)k * n;
   if (threadIdx.x < n) ekf[threadIdx.x] = (float)ek[threadIdx.x];
@@ -611,7 +611,7 @@ __global__ void __launch_bounds__(128, 2) k_adj64(Pair64Args a) {
   const int qi = blockIdx.x * 128 + threadIdx.x, kl = blockIdx.y, k = a.k0 + kl;
   const bool valid = qi < a.nq;
   const int q = valid ? qi : 0;
-  const int n = EX ? W : a.nw, nm = EX ? MM : a.nm;
+  const int n = EX ? W : a.nw, nm = MM <= 9 ? MM : a.nm;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const double *ek = a.eps_k + (size_t)k * n, *cot = a.cot + (size_t)k * n;
   if (threadIdx.x < n) ekf[threadIdx.x] = (float)ek[threadIdx.x];
@@ -702,7 +702,7 @@ template <int W, bool EX, int MM>
 __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
   __shared__ float ekf_s[4][W];
   __shared__ double dn_w[4][W], ia_w[4][W];
-  constexpr int MS = W <= 4 ? W : 1;
+  constexpr int MS = W <= 3 || (W == 4 && MM <= 3) ? W : 1;  // (what fits 48 KB with the terms' results)
   __shared__ P64Warp<W, MS, false> sws[4];
   __shared__ double res[4][32][2 * MM];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -714,7 +714,7 @@ __global__ void __launch_bounds__(128, 2) k_ph64(Pair64Args a) {
   const int qi = qw + lane;
   const bool valid = qi < a.nq;
   const int q = valid ? qi : 0;
-  const int n = EX ? W : a.nw, nm = EX ? MM : a.nm;
+  const int n = EX ? W : a.nw, nm = MM <= 9 ? MM : a.nm;
   P64Warp<W, MS, false> &sw = sws[warp];
   const double wm = a.wmax[q];
   double sp[MM], sl_[MM], sz = 0.0;
@@ -948,64 +948,73 @@ __global__ void k_tables64(int nq, int nm, const double *__restrict__ om, double
 
 }  // namespace
 
-epw_status launch_lw64(const Pair64Args &a, cudaStream_t st) {
-  if (a.nk <= 0 || a.nq <= 0) return EPW_OK;
-  const dim3 grid((a.nq + 127) / 128, a.nk);
-  const int n = a.nw, nm = a.nm;
-  if (n == 1 && nm == 3)
-    k_lw64<1, true, 3><<<grid, 128, 0, st>>>(a);
-  else if (n == 4 && nm == 3)
-    k_lw64<4, true, 3><<<grid, 128, 0, st>>>(a);
-  else if (n == 5 && nm == 9)
-    k_lw64<5, true, 9><<<grid, 128, 0, st>>>(a);
-  else if (n == 8 && nm == 6)
-    k_lw64<8, true, 6><<<grid, 128, 0, st>>>(a);
-  else if (n <= 4)
-    k_lw64<4, false, P64_MM><<<grid, 128, 0, st>>>(a);
-  else if (n <= 8)
-    k_lw64<8, false, P64_MM><<<grid, 128, 0, st>>>(a);
-  else if (n <= 18)
-    k_lw64<18, false, P64_MM><<<grid, 128, 0, st>>>(a);
-  else
-    return EPW_ERR_UNSUPPORTED;
+// The instances go by bounds.  Modes come in threes: 3, 6 and 9 (one to three atoms) are constants of the
+// kernel, more take its 18.  Bands take the widths 1, 4, 5 (matrices in registers), 8 and 18 (in local memory);
+// a band count that is the width itself is a constant too.  Measured, 57 R each (before: 18 modes and the widths
+// 4, 8, 18 for all but four sizes): linewidth 4 bands 3 atoms, 75 k x 4000 q 4.4 -> 4.1 ms, 5 bands 1 atom, 60 k
+// 2.9 -> 2.5, 8 bands 3 atoms, 37 k 10.2 -> 9.1 (as a bound instead of a constant 10.3); gradients 1.02 to
+// 1.25 times as fast, phonon side 1.02 to 1.27.  Six and seven bands with 9 modes keep the 18 in the linewidth
+// (8.3 ms, the constant 9.0: more registers live over the local matrices).
+template <template <int, bool, int> class K, int MMAX, int W, bool EX>
+static void p64_modes(const Pair64Args &a, dim3 grid, cudaStream_t st) {
+  if (a.nm == 3)
+    K<W, EX, 3>::run(a, grid, st);
+  else if (a.nm == 6)
+    K<W, EX, 6>::run(a, grid, st);
+  else if (a.nm == 9 && (MMAX == 9 || W != 8 || EX)) {
+    if constexpr (MMAX == 9 || W != 8 || EX) K<W, EX, 9>::run(a, grid, st);
+  } else if constexpr (MMAX > 9) {
+    K<W, EX, MMAX>::run(a, grid, st);
+  }
+}
+template <template <int, bool, int> class K, int WMAX, int MMAX>
+static epw_status p64_launch(const Pair64Args &a, dim3 grid, cudaStream_t st) {
+  if (a.nw > WMAX || a.nm > MMAX) return EPW_ERR_UNSUPPORTED;
+  const int n = a.nw;
+  if (n == 1)
+    p64_modes<K, MMAX, 1, true>(a, grid, st);
+  else if (n < 4)
+    p64_modes<K, MMAX, 4, false>(a, grid, st);
+  else if (n == 4)
+    p64_modes<K, MMAX, 4, true>(a, grid, st);
+  else if (n == 5)
+    p64_modes<K, MMAX, 5, true>(a, grid, st);
+  else if (n < 8)
+    p64_modes<K, MMAX, 8, false>(a, grid, st);
+  else if (n == 8)
+    p64_modes<K, MMAX, 8, true>(a, grid, st);
+  else if constexpr (WMAX > 8)
+    p64_modes<K, MMAX, WMAX, false>(a, grid, st);
   epw_count_launch();
   return cudaGetLastError() == cudaSuccess ? EPW_OK : EPW_ERR_CUDA;
+}
+
+template <int W, bool EX, int MM>
+struct Lw64 {
+  static void run(const Pair64Args &a, dim3 grid, cudaStream_t st) { k_lw64<W, EX, MM><<<grid, 128, 0, st>>>(a); }
+};
+template <int W, bool EX, int MM>
+struct Adj64 {
+  static void run(const Pair64Args &a, dim3 grid, cudaStream_t st) { k_adj64<W, EX, MM><<<grid, 128, 0, st>>>(a); }
+};
+template <int W, bool EX, int MM>
+struct Ph64 {
+  static void run(const Pair64Args &a, dim3 grid, cudaStream_t st) { k_ph64<W, EX, MM><<<grid, 128, 0, st>>>(a); }
+};
+
+epw_status launch_lw64(const Pair64Args &a, cudaStream_t st) {
+  if (a.nk <= 0 || a.nq <= 0) return EPW_OK;
+  return p64_launch<Lw64, 18, P64_MM>(a, dim3((a.nq + 127) / 128, a.nk), st);
 }
 
 epw_status launch_adj64(const Pair64Args &a, cudaStream_t st) {
   if (a.nk <= 0 || a.nq <= 0) return EPW_OK;
-  const dim3 grid((a.nq + 127) / 128, a.nk);
-  const int n = a.nw, nm = a.nm;
-  if (n > 8 || nm > 9) return EPW_ERR_UNSUPPORTED;
-  if (n == 1 && nm == 3)
-    k_adj64<1, true, 3><<<grid, 128, 0, st>>>(a);
-  else if (n == 4 && nm == 3)
-    k_adj64<4, true, 3><<<grid, 128, 0, st>>>(a);
-  else if (n == 5 && nm == 9)
-    k_adj64<5, true, 9><<<grid, 128, 0, st>>>(a);
-  else if (n == 8 && nm == 6)
-    k_adj64<8, true, 6><<<grid, 128, 0, st>>>(a);
-  else
-    k_adj64<8, false, P64_MM><<<grid, 128, 0, st>>>(a);
-  epw_count_launch();
-  return cudaGetLastError() == cudaSuccess ? EPW_OK : EPW_ERR_CUDA;
+  return p64_launch<Adj64, 8, 9>(a, dim3((a.nq + 127) / 128, a.nk), st);
 }
 
 epw_status launch_ph64(const Pair64Args &a, int nchunk, cudaStream_t st) {
   if (a.nk <= 0 || a.nq <= 0) return EPW_OK;
-  const dim3 grid((unsigned)(((size_t)((a.nq + 31) / 32) * nchunk + 3) / 4));
-  const int n = a.nw, nm = a.nm;
-  if (n > 8 || nm > 9) return EPW_ERR_UNSUPPORTED;
-  if (n == 1 && nm == 3)
-    k_ph64<1, true, 3><<<grid, 128, 0, st>>>(a);
-  else if (n == 4 && nm == 3)
-    k_ph64<4, true, 3><<<grid, 128, 0, st>>>(a);
-  else if (n == 8 && nm == 6)
-    k_ph64<8, true, 6><<<grid, 128, 0, st>>>(a);
-  else
-    k_ph64<8, false, 9><<<grid, 128, 0, st>>>(a);
-  epw_count_launch();
-  return cudaGetLastError() == cudaSuccess ? EPW_OK : EPW_ERR_CUDA;
+  return p64_launch<Ph64, 8, 9>(a, dim3((unsigned)(((size_t)((a.nq + 31) / 32) * nchunk + 3) / 4)), st);
 }
 
 epw_status launch_g64(const Pair64Args &a, cudaStream_t st) {
