@@ -1387,10 +1387,16 @@ void launch_vertex_fewk(int nk, int nR, int ncol, const cx<double> *P, const cx<
     launch_vertex_fewk(nk - 65535, nR, ncol, P + (size_t)65535 * nR, g, G1 + (size_t)65535 * ncol, st);
     return;
   }
-  if (nk >= 4 && (long)nb * ((nk + 3) / 4) >= 608)
-    k_vertex_fewk<4><<<dim3(nb, (nk + 3) / 4), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
-  else if (nk >= 3 && nb >= 304)
-    k_vertex_fewk<3><<<dim3(nb, (nk + 2) / 3), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  // up to four k a thread, the list split evenly (5 k: 3 and 2); one k where there would be too few blocks
+  const int passes = (nk + 3) / 4, kt = (nk + passes - 1) / passes;
+  const bool fill = (long)nb * passes >= (kt == 4 ? 608 : 304);
+  const dim3 grid(nb, fill ? passes : nk);
+  if (fill && kt == 4)
+    k_vertex_fewk<4><<<grid, 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  else if (fill && kt == 3)
+    k_vertex_fewk<3><<<grid, 128, 0, st>>>(nk, nR, ncol, P, g, G1);
+  else if (fill && kt == 2)
+    k_vertex_fewk<2><<<grid, 128, 0, st>>>(nk, nR, ncol, P, g, G1);
   else
     k_vertex_fewk<1><<<dim3(nb, nk), 128, 0, st>>>(nk, nR, ncol, P, g, G1);
   epw_count_launch();

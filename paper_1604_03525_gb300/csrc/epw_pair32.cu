@@ -28,14 +28,15 @@ struct A32Warp {
 
 template <int W, bool EX, int MM>
 __global__ void __launch_bounds__(128) k_adj32(PairArgs a) {
-  constexpr int UW = EX ? W : 1;
-  constexpr int UM = EX ? MM : 1;
+  constexpr bool REG = W <= 5;  // matrices in registers, every loop over bands unrolled
+  constexpr int UW = REG ? W : 1;
+  constexpr int UM = MM;
   __shared__ double sh[2][4];
   __shared__ A32Warp<W> sws[4];
   const int qi = blockIdx.x * 128 + threadIdx.x, kl = blockIdx.y, k = a.k0 + kl;
   const bool valid = qi < a.nq;
   const int q = valid ? qi : 0;  // lanes past the last q keep step with their warp
-  const int n = EX ? W : a.nw, nm = EX ? MM : a.nm, n2 = n * n, nq = a.nq;
+  const int n = EX ? W : a.nw, nm = MM, n2 = n * n, nq = a.nq;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, qw = qi - lane;
   const float *Ck = a.Cq + (size_t)kl * a.cpk * a.ldc;
   const cx<float> *ET = (const cx<float> *)a.ET;
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(128) k_adj32(PairArgs a) {
       need &= need - 1;
       float em = 0.0f;
       cx<float> u[W];
-      if constexpr (EX) {
+      if constexpr (REG) {
 #pragma unroll
         for (int c = 0; c < W; c++)
           if (c == m) {
@@ -227,14 +228,29 @@ __global__ void __launch_bounds__(128) k_adj32(PairArgs a) {
 
 }  // namespace
 
+// By bounds: the modes of one, two or three atoms as a constant; widths 4 and 5 in registers, 8 in local memory.
+template <int W, bool EX>
+static void adj32_modes(const PairArgs &a, cudaStream_t st) {
+  const dim3 grid((a.nq + 127) / 128, a.nkc);
+  if (a.nm == 3)
+    k_adj32<W, EX, 3><<<grid, 128, 0, st>>>(a);
+  else if (a.nm == 6)
+    k_adj32<W, EX, 6><<<grid, 128, 0, st>>>(a);
+  else
+    k_adj32<W, EX, 9><<<grid, 128, 0, st>>>(a);
+}
+
 epw_status launch_adj_staged(const PairArgs &a, cudaStream_t st) {
   if (a.nkc <= 0 || a.nq <= 0) return EPW_OK;
   if (!a.Cq || a.nw > 8 || a.nm > 9) return EPW_ERR_UNSUPPORTED;
-  const dim3 grid((a.nq + 127) / 128, a.nkc);
-  if (a.nw == 5 && a.nm == 9)
-    k_adj32<5, true, 9><<<grid, 128, 0, st>>>(a);
+  if (a.nw < 4)
+    adj32_modes<4, false>(a, st);
+  else if (a.nw == 4)
+    adj32_modes<4, true>(a, st);
+  else if (a.nw == 5)
+    adj32_modes<5, true>(a, st);
   else
-    k_adj32<8, false, 9><<<grid, 128, 0, st>>>(a);
+    adj32_modes<8, false>(a, st);
   epw_count_launch();
   return cudaGetLastError() == cudaSuccess ? EPW_OK : EPW_ERR_CUDA;
 }
