@@ -76,8 +76,10 @@ typedef enum {
 } epw_status;
 
 /* Arithmetic of the interpolation contractions and the per-pair eigensolves.
- *   EPW_FP64   : everything in FP64; larger contractions as exact digit products on the
- *                tensor cores (64-bit fixed point, at least FP64's accuracy).
+ *   EPW_FP64   : everything in FP64; larger contractions as digit products on the tensor
+ *                cores: operands to 56 bits below the largest element of their row, sums in
+ *                64-bit fixed point.  The error of a sum is at the level of an FP64 sum's
+ *                (2^-52 of the row's largest element per term).
  *   EPW_FP32   : contractions, eigensolves and rotations in FP32 (CUDA cores);
  *                phases, phonons, k-side eigensolves and the reduction in FP64.
  *   EPW_BF16X3 : contractions on the tensor cores (tcgen05) with operands split

@@ -7,9 +7,10 @@
 // are summed by tcgen05 kind::f16 MMAs, one FP32 accumulator per level l = i + j - 1:
 //   - a product is an integer of at most 2^14; an accumulator is emptied after at most 256
 //     terms per pair, so level l holds at most l 2^22 and levels 1 to 4 are exact for any input;
-//     levels 5 to 7 would have to exceed 2^24 to round (digits that all agree in sign and size),
-//     which leaves an error below 2^-45 of the row's maximum, inside the a-priori bound of an
-//     FP64 sum; for digits without such structure they are exact too (about 2^18);
+//     levels 5 to 7 would have to exceed 2^24 to round: digits that all agree in sign and size.  Then the
+//     last 16 of level 5's 80 accumulations round by a unit of 2^-46 of the row scales each at most, 2^-42
+//     beside a sum of such digits of about 2^7, inside the a-priori bound of an FP64 sum; for digits
+//     without such structure they are exact too (about 2^18);
 //   - the levels are combined in 64-bit integers at 2^-F of the row scales (F about 53), so the
 //     sum over K is exact and its order does not matter.
 // What is dropped (levels from 8 on) is about 2^-52 of the product of the row maxima; the FP64
