@@ -663,8 +663,8 @@ static epw_status run_prep(const epw_model *mc, int nk, const double *k, int nq,
   const size_t nw2 = (size_t)nw * nw;
   const bool exact = fx && fx->exact;
   // The k side of the FP32 and split forms, always: it is cast to FP32 and split, and a value that is cast
-  // the other way moves every q of its k alike (one in about 50 lists of 256 k of the diamond model; 4e-8
-  // of the linewidths of that k).
+  // the other way moves every q of its k alike (up to 4e-8 of that k's linewidths, 1.5e-9 of a list of 256
+  // k); a q's casts are one term of many (316,000 q: below 5e-12).
   const bool exact_k = exact || prec != EPW_FP64;
   cudaStream_t sq = st;
   fork = fork && nq > 0 && nk > 0;
