@@ -10,8 +10,8 @@
 //   - only the eigenvectors and the (m, n) terms are formed whose Gaussians do not underflow in
 //     FP64 (|e_nk - e_mk+q| <= max_nu w_qnu + 27.35 sigma; beyond, exp(-y^2) is exactly 0), so
 //     every sum equals the dense one; a warp takes its pairs' terms together, 32 at a time.
-// Measured: fcc nw = 4, 125 k x 13,824 q 7 ms, diamond nw = 8, 24 k x 8000 q 4.6 ms (contraction, Jacobi
-// and every term in one kernel on the CUDA cores: 126 and 181); k_ph64 fcc 8000 k x 216 q 8.6 ms (203).
+// Measured: fcc nw = 4, 125 k x 13,824 q 7 ms, diamond nw = 8, 24 k x 8000 q 4.8 ms (contraction, Jacobi
+// and every term in one kernel on the CUDA cores: 126 and 181); k_ph64 fcc 8000 k x 216 q 9.0 ms (203).
 #include "epw_pair64.cuh"
 
 namespace {
